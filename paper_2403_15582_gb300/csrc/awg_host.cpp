@@ -769,7 +769,7 @@ class HostPool {
 };
 
 // Scratch for launches of up to `tiles` tiles with tone split `split` (> 1): two buffers of
-// part_tiles x part_split partial tiles (capacities) and part_tiles tile counters each.  The
+// part_tiles x part_split partial tiles (capacities) and MAX_PARTS counters per tile each.  The
 // counters count every CTA of every launch, and a CTA is the last of its tile when its count is
 // split - 1 mod split; so they are zeroed when allocated and whenever the split changes.
 constexpr int32_t SPLIT_LAUNCH_TILES = 512;   // tiles per render launch when the split sums in scratch
@@ -786,7 +786,8 @@ int ensure_split_scratch(awg_t* h, int32_t tiles, int32_t split) {
     h->d_tctr = nullptr;
     h->part_tiles = h->part_split = 0;
     e = cudaMalloc((void**)&h->d_part, (size_t)2 * nt * ns * awgk::TILE * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_tctr, (size_t)2 * nt * sizeof(unsigned long long));
+    if (e == cudaSuccess)
+      e = cudaMalloc((void**)&h->d_tctr, (size_t)2 * nt * awgk::MAX_PARTS * sizeof(unsigned long long));
     if (e != cudaSuccess) {
       cudaGetLastError();
       return fail(AWG_ENOMEM, "cudaMalloc split scratch");
@@ -794,7 +795,7 @@ int ensure_split_scratch(awg_t* h, int32_t tiles, int32_t split) {
     h->part_tiles = nt;
     h->part_split = ns;
   }
-  if ((e = cudaMemset(h->d_tctr, 0, (size_t)2 * h->part_tiles * sizeof(unsigned long long))) != cudaSuccess)
+  if ((e = cudaMemset(h->d_tctr, 0, (size_t)2 * h->part_tiles * awgk::MAX_PARTS * sizeof(unsigned long long))) != cudaSuccess)
     return cuda_fail(e, "split counters");
   h->ctr_split = split;
   return AWG_OK;
@@ -804,7 +805,9 @@ int ensure_split_scratch(awg_t* h, int32_t tiles, int32_t split) {
 float* split_part(awg_t* h, int b) {
   return h->d_part + (size_t)b * (size_t)h->part_tiles * (size_t)h->part_split * awgk::TILE;
 }
-unsigned long long* split_ctr(awg_t* h, int b) { return h->d_tctr + (size_t)b * (size_t)h->part_tiles; }
+unsigned long long* split_ctr(awg_t* h, int b) {
+  return h->d_tctr + (size_t)b * (size_t)h->part_tiles * awgk::MAX_PARTS;
+}
 
 int upload_tones(awg_t* h) {
   int st = ensure(&h->d_tones, &h->cap_tones, std::max<size_t>(1, h->tones.size()), h, "tones");
@@ -1005,6 +1008,46 @@ int stage_end(awg_t* h) {
   return AWG_OK;
 }
 
+// Chirp slots active in the window [c, c + n) (tile-aligned span), excluding exact-table chirps, in
+// tone order: the render copies the records of a stage's tones in one piece.
+bool slot_active(const ChirpRec& cr, int64_t span0, int64_t span1) {
+  return cr.tone >= 0 && !(cr.flags & awgk::TONE_EXACT) && cr.n_s <= span1 && cr.n_s + cr.L >= span0;
+}
+std::vector<int32_t> active_slots(const awg_t* h, int64_t c, int64_t n, int64_t* tile0, int32_t* n_tiles) {
+  const int64_t t0 = c / awgk::TILE, t1 = (c + n - 1) / awgk::TILE;
+  const int64_t span0 = t0 * awgk::TILE, span1 = (t1 + 1) * awgk::TILE - 1;
+  std::vector<int32_t> active;
+  if (h->chirps.size() < h->tones.size() / 8) {   // few chirps: their slots, sorted
+    for (size_t sl = 0; sl < h->chirps.size(); ++sl)
+      if (slot_active(h->chirps[sl], span0, span1)) active.push_back((int32_t)sl);
+    auto by_tone = [&](int32_t x, int32_t y) { return h->chirps[(size_t)x].tone < h->chirps[(size_t)y].tone; };
+    if (!std::is_sorted(active.begin(), active.end(), by_tone)) std::sort(active.begin(), active.end(), by_tone);
+  } else {
+    for (const ToneRec& t : h->tones)
+      if (t.slot >= 0 && !(t.flags & awgk::TONE_EXACT) && t.n_s <= span1 && t.n_e >= span0) active.push_back(t.slot);
+  }
+  *tile0 = t0;
+  *n_tiles = (int32_t)(t1 - t0 + 1);
+  return active;
+}
+
+// Parts a tile's samples are cut into (RenderArgs::parts) for work of `tiles` tiles.  A CTA is one
+// rank of one part; c of them land on the busiest SM.  Halves and quarters repeat the run set-ups (per
+// SM 0.56 and 0.36 of a whole tile's time instead of 0.5 and 0.25), so they pay only where whole
+// tiles leave SMs idle or unevenly loaded; the added constants are the SM's poorer rate with few
+// warps.  All from the chirp loop with set-ups, timed by CTAs per SM: 2.7, 3.6, 3.75 ... 4.03e12
+// sines/s at 1, 2, 3 ... 7 whole tiles per SM, 2.1, 3.0, 3.3 ... 3.6 for halves, 1.5, 2.2, 2.5 ... 2.8 for
+// quarters.  The rotator's runs cannot be entered in the middle: whole tiles.
+int32_t render_parts(int64_t tiles, int32_t split, int32_t sine_mode) {
+  if (sine_mode == AWG_SINE_ROTATOR) return 1;
+  const int64_t sms = awgk::device_sm_count();
+  auto cost = [&](int32_t parts, double each, double more) {
+    return each * ((double)((tiles * split * parts + sms - 1) / sms) + more);
+  };
+  const double c1 = cost(1, 1.0, 0.5), c2 = cost(2, 0.56, 0.6), c4 = cost(4, 0.36, 0.9);
+  return c1 <= c2 && c1 <= c4 ? 1 : (c2 <= c4 ? 2 : 4);
+}
+
 int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream, int32_t q_stride,
                   const float* base, int32_t skip_static, const int32_t* tone_list = nullptr, int32_t n_list = 0,
                   int32_t list_split = 0, const int32_t* list_bounds = nullptr);
@@ -1051,16 +1094,9 @@ int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
   const int64_t tile_last = (c + n - 1) / awgk::TILE;
   const int64_t n_tiles64 = tile_last - tile0 + 1;
   if (n_tiles64 > (int64_t)(INT32_MAX / awgk::MAX_SPLIT)) return fail(AWG_EINVAL, "render window too long");
-  const int32_t n_tiles = (int32_t)n_tiles64;
-  const int64_t span0 = tile0 * awgk::TILE, span1 = (tile_last + 1) * awgk::TILE - 1;
-
-  std::vector<int32_t> active;
-  for (size_t sl = 0; sl < h->chirps.size(); ++sl) {
-    const ChirpRec& cr = h->chirps[sl];
-    if (cr.tone < 0 || (cr.flags & awgk::TONE_EXACT)) continue;
-    const int64_t ne = cr.n_s + cr.L;
-    if (cr.n_s <= span1 && ne >= span0) active.push_back((int32_t)sl);
-  }
+  int64_t tile0_;
+  int32_t n_tiles;
+  const std::vector<int32_t> active = active_slots(h, c, n, &tile0_, &n_tiles);
   int st = ensure(&h->d_recs, &h->cap_recs, std::max<size_t>(1, active.size() * (size_t)n_tiles), h, "tile records");
   if (st) return st;
   // With a split, the window goes out in launches of at most SPLIT_LAUNCH_TILES tiles, chained by
@@ -1091,12 +1127,14 @@ int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
     awgk::PrepArgs pa;
     std::memset(&pa, 0, sizeof(pa));
     pa.chirps = h->d_chirps;
+    pa.tones = h->d_tones;
     pa.recs = h->d_recs;
     pa.act_of_slot = h->d_act;
     pa.tile0 = tile0;
     pa.n_tiles = n_tiles;
     pa.n_active = (int32_t)std::min<size_t>(awgk::MAX_ACTIVE_PER_LAUNCH, active.size() - b);
     pa.act_base = (int32_t)b;
+    pa.rec_stride = (int32_t)active.size();
     std::memcpy(pa.W, h->W, sizeof(pa.W));
     std::memcpy(pa.inv_odd, h->inv_odd, sizeof(pa.inv_odd));
     for (int i = 0; i < pa.n_active; ++i) pa.slots[i] = active[b + (size_t)i];
@@ -1134,8 +1172,9 @@ int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
     const int64_t w1 = std::min(c + n, (tile0 + t0 + nt) * (int64_t)awgk::TILE);
     rs.tile0 = tile0 + t0;
     rs.n_tiles = nt;
-    rs.rec_stride = n_tiles;
+    rs.rec_stride = (int32_t)active.size();
     rs.rec_tile0 = t0;
+    rs.parts = render_parts(nt, split_used, h->sine_mode);
     rs.win_start = w0;
     rs.win_end = w1;
     rs.out_q = out_q ? out_q + (size_t)(w0 - c) * (size_t)(q_stride ? q_stride : 1) : nullptr;
@@ -1388,15 +1427,9 @@ int awgk::prepare_render(awg_t* h, int64_t n, int16_t* out_q, float* out_f, cuda
                          awgk::TileRec* recs, size_t recs_cap, int32_t* act, size_t* recs_need) {
   if (!h || n <= 0 || (!out_q && !out_f) || !ra) return fail(AWG_EINVAL, "prepare_render: bad arguments");
   const int64_t c = h->cursor;
-  const int64_t tile0 = c / awgk::TILE, tile_last = (c + n - 1) / awgk::TILE;
-  const int32_t n_tiles = (int32_t)(tile_last - tile0 + 1);
-  const int64_t span0 = tile0 * awgk::TILE, span1 = (tile_last + 1) * awgk::TILE - 1;
-  std::vector<int32_t> active;
-  for (size_t sl = 0; sl < h->chirps.size(); ++sl) {
-    const ChirpRec& cr = h->chirps[sl];
-    if (cr.tone < 0 || (cr.flags & awgk::TONE_EXACT)) continue;
-    if (cr.n_s <= span1 && cr.n_s + cr.L >= span0) active.push_back((int32_t)sl);
-  }
+  int64_t tile0;
+  int32_t n_tiles;
+  const std::vector<int32_t> active = active_slots(h, c, n, &tile0, &n_tiles);
   const size_t need = active.size() * (size_t)n_tiles;
   if (recs_need) *recs_need = need;
   if (recs || act) {
@@ -1415,12 +1448,14 @@ int awgk::prepare_render(awg_t* h, int64_t n, int16_t* out_q, float* out_f, cuda
     awgk::PrepArgs pa;
     std::memset(&pa, 0, sizeof(pa));
     pa.chirps = h->d_chirps;
+    pa.tones = h->d_tones;
     pa.recs = recs;
     pa.act_of_slot = act;
     pa.tile0 = tile0;
     pa.n_tiles = n_tiles;
     pa.n_active = (int32_t)std::min<size_t>(awgk::MAX_ACTIVE_PER_LAUNCH, active.size() - b);
     pa.act_base = (int32_t)b;
+    pa.rec_stride = (int32_t)active.size();
     std::memcpy(pa.W, h->W, sizeof(pa.W));
     std::memcpy(pa.inv_odd, h->inv_odd, sizeof(pa.inv_odd));
     for (int i = 0; i < pa.n_active; ++i) pa.slots[i] = active[b + (size_t)i];
@@ -1438,6 +1473,8 @@ int awgk::prepare_render(awg_t* h, int64_t n, int16_t* out_q, float* out_f, cuda
   ra->sine_mode = h->sine_mode;
   ra->tile0 = tile0;
   ra->n_tiles = n_tiles;
+  ra->rec_stride = (int32_t)active.size();
+  ra->parts = 1;
   ra->win_start = c;
   ra->win_end = c + n;
   ra->out_q = out_q;
@@ -1450,21 +1487,6 @@ int awgk::prepare_render(awg_t* h, int64_t n, int16_t* out_q, float* out_f, cuda
 }
 
 namespace {
-
-// Chirp slots active in the window [c, c + n) (tile-aligned span), excluding exact-table chirps.
-std::vector<int32_t> active_slots(const awg_t* h, int64_t c, int64_t n, int64_t* tile0, int32_t* n_tiles) {
-  const int64_t t0 = c / awgk::TILE, t1 = (c + n - 1) / awgk::TILE;
-  const int64_t span0 = t0 * awgk::TILE, span1 = (t1 + 1) * awgk::TILE - 1;
-  std::vector<int32_t> active;
-  for (size_t sl = 0; sl < h->chirps.size(); ++sl) {
-    const ChirpRec& cr = h->chirps[sl];
-    if (cr.tone < 0 || (cr.flags & awgk::TONE_EXACT)) continue;
-    if (cr.n_s <= span1 && cr.n_s + cr.L >= span0) active.push_back((int32_t)sl);
-  }
-  *tile0 = t0;
-  *n_tiles = (int32_t)(t1 - t0 + 1);
-  return active;
-}
 
 // n_chunks consecutive chunk renders, pipelined.  The chunks are taken in groups whose chirp tile
 // records fit a fixed budget; for each group one set-up launch computes the records of every
@@ -1556,12 +1578,15 @@ int render_chunks_impl(awg_t* h, int64_t chunk, int32_t n_chunks, int16_t* out, 
       awgk::PrepArgs pa;
       std::memset(&pa, 0, sizeof(pa));
       pa.chirps = h->d_chirps;
+      pa.tones = h->d_tones;
       pa.recs = h->d_seq_recs;
       pa.act_of_slot = h->d_seq_act;
       pa.tile0 = tile0;
       pa.n_tiles = n_tiles;
       pa.n_active = (int32_t)std::min<size_t>(awgk::MAX_ACTIVE_PER_LAUNCH, active.size() - b);
       pa.act_base = (int32_t)b;
+      pa.rec_stride = (int32_t)active.size();
+    pa.rec_stride = (int32_t)active.size();
       std::memcpy(pa.W, h->W, sizeof(pa.W));
       std::memcpy(pa.inv_odd, h->inv_odd, sizeof(pa.inv_odd));
       for (int i = 0; i < pa.n_active; ++i) pa.slots[i] = active[b + (size_t)i];
@@ -1571,6 +1596,10 @@ int render_chunks_impl(awg_t* h, int64_t chunk, int32_t n_chunks, int16_t* out, 
       if ((e = cudaEventRecord(pe[1], s)) != cudaSuccess) return cuda_fail(e, "event");
       if ((e = cudaEventRecord(pe[2], s)) != cudaSuccess) return cuda_fail(e, "event");
     }
+    // a launch overlaps the next one (which waits for it before it reuses the scratch): two launches
+    // fill the device together.  One form for the group: a change of kernel in mid-sequence costs
+    // more than a better fit of the last launch gives (500 against 488 us for 1500 tones in 8 chunks)
+    const int32_t parts = render_parts(std::min<int64_t>(2 * ((chunk + awgk::TILE - 1) / awgk::TILE), n_tiles), h->split, h->sine_mode);
     for (int32_t c = g0; c < g1; ++c) {
       const int64_t wc = c0 + (int64_t)c * chunk, len = span(c, c + 1);
       const int64_t t_first = wc / awgk::TILE, t_last = (wc + len - 1) / awgk::TILE;
@@ -1581,7 +1610,7 @@ int render_chunks_impl(awg_t* h, int64_t chunk, int32_t n_chunks, int16_t* out, 
       ra.chirps = h->d_chirps;
       ra.recs = h->d_seq_recs;
       ra.act_of_slot = h->d_seq_act;
-      ra.rec_stride = n_tiles;
+      ra.rec_stride = (int32_t)active.size();
       ra.rec_tile0 = (int32_t)(t_first - tile0);
       ra.K = h->K;
       ra.split = h->split;
@@ -1594,6 +1623,7 @@ int render_chunks_impl(awg_t* h, int64_t chunk, int32_t n_chunks, int16_t* out, 
       ra.scale = h->full_scale > 0 ? (float)(32767.0 / h->full_scale) : 0.f;
       ra.status = h->d_status;
       std::memcpy(ra.inv_odd, h->inv_odd, sizeof(ra.inv_odd));
+      ra.parts = parts;
       ra.pdl = c == g0 ? 1 : 2;
       ra.exit_ctr = h->d_seq_exit;
       if (h->split > 1) {   // alternating scratch (see tile_epilogue_split)
@@ -1601,7 +1631,7 @@ int render_chunks_impl(awg_t* h, int64_t chunk, int32_t n_chunks, int16_t* out, 
         ra.tile_ctr = split_ctr(h, c & 1);
       }
       if ((e = counted(h, awgk::launch_render(ra, s))) != cudaSuccess) return cuda_fail(e, "render launch");
-      h->seq_exit_target += (unsigned long long)ra.n_tiles * (unsigned long long)h->split;
+      h->seq_exit_target += (unsigned long long)ra.n_tiles * (unsigned long long)(ra.parts * h->split);
     }
     if ((e = counted(h, awgk::launch_join(h->d_seq_exit, h->seq_exit_target, h->d_status, awgk::JOIN_LIMIT_NS, s))) !=
         cudaSuccess)
@@ -2175,12 +2205,14 @@ int awg_render_phases(awg_t* h, int32_t tone, int64_t n0, int32_t count, uint32_
     awgk::PrepArgs pa;
     std::memset(&pa, 0, sizeof(pa));
     pa.chirps = h->d_chirps;
+    pa.tones = h->d_tones;
     pa.recs = h->d_recs;
     pa.act_of_slot = h->d_act;
     pa.tile0 = tile0;
     pa.n_tiles = n_tiles;
     pa.n_active = 1;
     pa.act_base = 0;
+    pa.rec_stride = 1;
     std::memcpy(pa.W, h->W, sizeof(pa.W));
     std::memcpy(pa.inv_odd, h->inv_odd, sizeof(pa.inv_odd));
     pa.slots[0] = t.slot;
@@ -2302,13 +2334,12 @@ int awg_render_noalloc(awg_t* h, int64_t n, int16_t* out, void* stream) {
   const int64_t n_tiles = tile_last - tile0 + 1;
   if (n_tiles > (int64_t)(INT32_MAX / awgk::MAX_SPLIT)) return fail(AWG_EINVAL, "render window too long");
   const int64_t span0 = tile0 * awgk::TILE, span1 = (tile_last + 1) * awgk::TILE - 1;
-  auto is_active = [&](const ChirpRec& cr) {
-    return cr.tone >= 0 && !(cr.flags & awgk::TONE_EXACT) && cr.n_s <= span1 && cr.n_s + cr.L >= span0;
-  };
+  // active chirps in tone order (no heap: the tones are scanned)
+  auto active_slot = [&](const ToneRec& t) { return t.slot >= 0 && slot_active(h->chirps[(size_t)t.slot], span0, span1); };
   int64_t n_active = 0;
-  for (size_t sl = 0; sl < h->chirps.size(); ++sl) {
-    if (!is_active(h->chirps[sl])) continue;
-    if ((int64_t)sl >= awgk::NOALLOC_MAX_SLOTS)
+  for (const ToneRec& t : h->tones) {
+    if (!active_slot(t)) continue;
+    if (t.slot >= awgk::NOALLOC_MAX_SLOTS)
       return fail(AWG_ENOMEM, "chirp slot index beyond the fixed scratch's slot map (AWG_NOALLOC_MAX_SLOTS)");
     ++n_active;
   }
@@ -2321,16 +2352,18 @@ int awg_render_noalloc(awg_t* h, int64_t n, int16_t* out, void* stream) {
   awgk::PrepArgs pa;
   std::memset(&pa, 0, sizeof(pa));
   pa.chirps = h->d_chirps;
+  pa.tones = h->d_tones;
   pa.recs = recs;
   pa.act_of_slot = act;
   pa.tile0 = tile0;
   pa.n_tiles = (int32_t)n_tiles;
+  pa.rec_stride = (int32_t)n_active;
   std::memcpy(pa.W, h->W, sizeof(pa.W));
   std::memcpy(pa.inv_odd, h->inv_odd, sizeof(pa.inv_odd));
   int32_t batch_base = 0;
-  for (size_t sl = 0; sl < h->chirps.size(); ++sl) {
-    if (!is_active(h->chirps[sl])) continue;
-    pa.slots[pa.n_active++] = (int32_t)sl;
+  for (const ToneRec& t : h->tones) {
+    if (!active_slot(t)) continue;
+    pa.slots[pa.n_active++] = t.slot;
     if (pa.n_active == awgk::MAX_ACTIVE_PER_LAUNCH) {
       pa.act_base = batch_base;
       if ((e = counted(h, awgk::launch_prep(pa, s))) != cudaSuccess) return cuda_fail(e, "prep launch");
@@ -2354,6 +2387,8 @@ int awg_render_noalloc(awg_t* h, int64_t n, int16_t* out, void* stream) {
   ra.sine_mode = h->sine_mode;
   ra.tile0 = tile0;
   ra.n_tiles = (int32_t)n_tiles;
+  ra.rec_stride = (int32_t)n_active;
+  ra.cluster = 1;
   ra.win_start = c;
   ra.win_end = c + n;
   ra.out_q = out;

@@ -20,6 +20,7 @@ constexpr int RT = RUNS;           // threads per render CTA
 constexpr int STAGE = 32;          // tones staged in shared memory at a time (double-buffered)
 constexpr int SINE_SFU = 0;        // static segments: SFU sine of every sample's phase
 constexpr int SINE_ROTATOR = 1;    // static segments: exact sin/cos at the run start, then rotations
+constexpr int MAX_PARTS = 4;       // CTAs that may share a tile's samples (render_parts)
 constexpr int MAX_SPLIT = 16;      // cluster size limit (non-portable 16 on sm_100-class parts)
 constexpr int MAX_ACTIVE_PER_LAUNCH = 7168;   // chirp slots per prep launch (kernel parameters: < 32 KB)
 
@@ -109,27 +110,35 @@ struct alignas(16) ChirpRec {
 static_assert(sizeof(ChirpRec) == 208, "ChirpRec layout");
 
 // Per (active chirp, tile) record: the chirp phase polynomial re-expressed at the tile start as
-// forward differences with stride RUN in the run index j (0 <= j < RUNS), for the phase and its
-// first three unit-stride differences.  Words (2^-64 turn), rounded.  B[0] is the phase word.
+// forward differences with stride RUN in the run index j (0 <= j < RUNS), for the phase (B_0..B_6)
+// and its first three unit-stride differences (E_0..E_5, G_0..G_4, H_0..H_3).  Words (2^-64 turn),
+// rounded; B_0 is the phase word.  The words stand in the order in which the run set-ups need them:
+// a linear chirp takes the first 6, one in LOW3 form the first 10; in a tile that such a chirp
+// covers without an amplitude ramp the others are neither formed nor written (rec_words).
 struct alignas(16) TileRec {
-  uint64_t B[7];
-  uint64_t E[6];
-  uint64_t G[5];
-  uint64_t H[4];
+  uint64_t w[22];
 };
 static_assert(sizeof(TileRec) == 176, "TileRec layout");
+// place of B_q, E_q, G_q, H_q: byte q of a constant
+AWG_HD constexpr int rec_b(int q) { return (int)((0xD0A0706020100ull >> (8 * q)) & 255); }   // 0 1 2 6 7 10 13
+AWG_HD constexpr int rec_e(int q) { return (int)((0xE0C0B080403ull >> (8 * q)) & 255); }   // 3 4 8 11 12 14
+AWG_HD constexpr int rec_g(int q) { return (int)((0x11100F0905ull >> (8 * q)) & 255); }   // 5 9 15 16 17
+AWG_HD constexpr int rec_h(int q) { return (int)((0x15141312ull >> (8 * q)) & 255); }   // 18 19 20 21
+constexpr int REC_WORDS_LINEAR = 6, REC_WORDS_LOW3 = 10, REC_WORDS = 22;
 
 // Arguments of one prep launch, the active chirp slots inline (kernel parameters are copied with
 // the launch: a launch of up to 1024 slots passes the small form, larger ones the full 7168).
 template <int CAP>
 struct PrepArgsT {
   const ChirpRec* chirps;
-  TileRec* recs;          // [n_active][n_tiles]
+  const ToneRec* tones;
+  TileRec* recs;          // [n_tiles][rec_stride], the window's active chirps in tone order
   int32_t* act_of_slot;   // slot -> active index (written here)
   int64_t tile0;          // absolute index of the first tile
   int32_t n_tiles;
   int32_t n_active;
   int32_t act_base;       // active index of slots[0]
+  int32_t rec_stride;     // records per tile (active chirps of the window)
   uint32_t W[7][7];       // W[q][i] = Delta^q_j C(j RUN, i) at j = 0 (all below 2^32)
   uint64_t inv_odd[3][3]; // inverses mod 2^192 of 3, 15, 45
   int32_t slots[CAP];
@@ -156,8 +165,8 @@ struct RenderArgs {
   uint64_t inv_odd[3][3];
   int32_t sine_mode;      // SINE_SFU or SINE_ROTATOR (static segments)
   int32_t q_stride;       // int16 output: sample i goes to out_q[i * q_stride] (0: 1; channel multiplexing)
-  // record rows: the records of active chirp a for window tile t are at recs[a * rec_stride +
-  // rec_tile0 + t] (rec_stride 0: n_tiles, the render's own set-up)
+  // records: active chirp a of the set-up's window (numbered in tone order) for this render's tile t
+  // is recs[(rec_tile0 + t) * rec_stride + a]
   int32_t rec_stride;
   int32_t rec_tile0;
   // pipelined chunk sequences (otherwise 0 / null): pdl 1 waits for the preceding kernel (the
@@ -176,9 +185,11 @@ struct RenderArgs {
   const int32_t* tone_list;
   int32_t n_list;
   int32_t bounds[MAX_SPLIT + 1];
-  // split sums without clusters (render_split_kernel; null: cluster reduction): partial tiles
-  // part[(tile split + rank) TILE + sample] and one counter per tile (a multiple of split between
-  // launches: every CTA adds 1)
+  int32_t cluster;        // 1: render_kernel, the split sums through a cluster's shared memory
+  int32_t parts;          // CTAs that share a tile's samples: 1, 2 or 4 (render_split_kernel)
+  // split sums without clusters: partial sums part[((tile parts + p) split + rank) (TILE / parts) +
+  // sample] and one counter per part of a tile (a multiple of split between launches: every CTA
+  // adds 1)
   float* part;
   unsigned long long* tile_ctr;
 };

@@ -9,8 +9,8 @@
 // chirps: Phi(n_s) + C (e^(alpha m) - 1) in FP64.
 //
 // Work decomposition (see awg_internal.h): a CTA renders one tile of TILE = 4096 absolute-aligned
-// samples; thread j owns the run of RUN = 32 samples starting at T0 + 32 j and keeps its 32 partial
-// sums in registers; the tones are split over `split` CTAs, whose partial tiles are added in rank
+// samples (or a half or a quarter of it, see Geo); thread j owns the run of RUN = 32 samples starting
+// at T0 + 32 j (or a half or a quarter of a run) and keeps its partial sums in registers; the tones are split over `split` CTAs, whose partial tiles are added in rank
 // order (through L2 scratch by the last CTA of the tile to finish, or through distributed shared
 // memory in a thread-block cluster), then scaled, rounded and stored by the same kernel.
 //
@@ -223,39 +223,39 @@ constexpr uint64_t HALF32_OFF = 1ull << 31;
 __device__ __forceinline__ RunPoly poly_state(const TileRec& rc, const RunBin& b, bool linear) {
   RunPoly r;
   if (linear) {   // B_q (q >= 3), E_q (q >= 2), G_q (q >= 1) and H are exactly zero
-    Top32 p = top_init(rc.B[0]);
-    top_mac(p, rc.B[1], b.c1);
-    top_mac(p, rc.B[2], b.c2);
-    Top32 f = top_init(rc.E[0]);
-    top_mac(f, rc.E[1], b.c1);
+    Top32 p = top_init(rc.w[rec_b(0)]);
+    top_mac(p, rc.w[rec_b(1)], b.c1);
+    top_mac(p, rc.w[rec_b(2)], b.c2);
+    Top32 f = top_init(rc.w[rec_e(0)]);
+    top_mac(f, rc.w[rec_e(1)], b.c1);
     r.p = top_get(p);
     r.f = top_get(f);
-    r.g = (uint32_t)(rc.G[0] >> 32);
+    r.g = (uint32_t)(rc.w[rec_g(0)] >> 32);
     r.h = 0;
     return r;
   }
-  Top32 p = top_init(rc.B[0]);
-  top_mac(p, rc.B[1], b.c1);
-  top_mac(p, rc.B[2], b.c2);
-  top_mac(p, rc.B[3], b.c3);
-  top_mac(p, rc.B[4], b.c4);
-  top_mac(p, rc.B[5], b.c5);
-  top_mac64(p, rc.B[6], b.c6);
-  Top32 f = top_init(rc.E[0]);
-  top_mac(f, rc.E[1], b.c1);
-  top_mac(f, rc.E[2], b.c2);
-  top_mac(f, rc.E[3], b.c3);
-  top_mac(f, rc.E[4], b.c4);
-  top_mac(f, rc.E[5], b.c5);
-  Top32 g = top_init(rc.G[0]);
-  top_mac(g, rc.G[1], b.c1);
-  top_mac(g, rc.G[2], b.c2);
-  top_mac(g, rc.G[3], b.c3);
-  top_mac(g, rc.G[4], b.c4);
-  Top32 h = top_init(rc.H[0]);
-  top_mac(h, rc.H[1], b.c1);
-  top_mac(h, rc.H[2], b.c2);
-  top_mac(h, rc.H[3], b.c3);
+  Top32 p = top_init(rc.w[rec_b(0)]);
+  top_mac(p, rc.w[rec_b(1)], b.c1);
+  top_mac(p, rc.w[rec_b(2)], b.c2);
+  top_mac(p, rc.w[rec_b(3)], b.c3);
+  top_mac(p, rc.w[rec_b(4)], b.c4);
+  top_mac(p, rc.w[rec_b(5)], b.c5);
+  top_mac64(p, rc.w[rec_b(6)], b.c6);
+  Top32 f = top_init(rc.w[rec_e(0)]);
+  top_mac(f, rc.w[rec_e(1)], b.c1);
+  top_mac(f, rc.w[rec_e(2)], b.c2);
+  top_mac(f, rc.w[rec_e(3)], b.c3);
+  top_mac(f, rc.w[rec_e(4)], b.c4);
+  top_mac(f, rc.w[rec_e(5)], b.c5);
+  Top32 g = top_init(rc.w[rec_g(0)]);
+  top_mac(g, rc.w[rec_g(1)], b.c1);
+  top_mac(g, rc.w[rec_g(2)], b.c2);
+  top_mac(g, rc.w[rec_g(3)], b.c3);
+  top_mac(g, rc.w[rec_g(4)], b.c4);
+  Top32 h = top_init(rc.w[rec_h(0)]);
+  top_mac(h, rc.w[rec_h(1)], b.c1);
+  top_mac(h, rc.w[rec_h(2)], b.c2);
+  top_mac(h, rc.w[rec_h(3)], b.c3);
   r.p = top_get(p);
   r.f = top_get(f);
   r.g = top_get(g);
@@ -265,59 +265,59 @@ __device__ __forceinline__ RunPoly poly_state(const TileRec& rc, const RunBin& b
 
 // poly_state for a degree-6 chirp whose h is known to round to 0 (TONE_FLAT3): no H polynomial.
 __device__ __forceinline__ RunPoly poly_state_flat3(const TileRec& rc, const RunBin& b) {
-  Top32 p = top_init(rc.B[0]);
-  top_mac(p, rc.B[1], b.c1);
-  top_mac(p, rc.B[2], b.c2);
-  top_mac(p, rc.B[3], b.c3);
-  top_mac(p, rc.B[4], b.c4);
-  top_mac(p, rc.B[5], b.c5);
-  top_mac64(p, rc.B[6], b.c6);
-  Top32 f = top_init(rc.E[0]);
-  top_mac(f, rc.E[1], b.c1);
-  top_mac(f, rc.E[2], b.c2);
-  top_mac(f, rc.E[3], b.c3);
-  top_mac(f, rc.E[4], b.c4);
-  top_mac(f, rc.E[5], b.c5);
-  Top32 g = top_init(rc.G[0]);
-  top_mac(g, rc.G[1], b.c1);
-  top_mac(g, rc.G[2], b.c2);
-  top_mac(g, rc.G[3], b.c3);
-  top_mac(g, rc.G[4], b.c4);
+  Top32 p = top_init(rc.w[rec_b(0)]);
+  top_mac(p, rc.w[rec_b(1)], b.c1);
+  top_mac(p, rc.w[rec_b(2)], b.c2);
+  top_mac(p, rc.w[rec_b(3)], b.c3);
+  top_mac(p, rc.w[rec_b(4)], b.c4);
+  top_mac(p, rc.w[rec_b(5)], b.c5);
+  top_mac64(p, rc.w[rec_b(6)], b.c6);
+  Top32 f = top_init(rc.w[rec_e(0)]);
+  top_mac(f, rc.w[rec_e(1)], b.c1);
+  top_mac(f, rc.w[rec_e(2)], b.c2);
+  top_mac(f, rc.w[rec_e(3)], b.c3);
+  top_mac(f, rc.w[rec_e(4)], b.c4);
+  top_mac(f, rc.w[rec_e(5)], b.c5);
+  Top32 g = top_init(rc.w[rec_g(0)]);
+  top_mac(g, rc.w[rec_g(1)], b.c1);
+  top_mac(g, rc.w[rec_g(2)], b.c2);
+  top_mac(g, rc.w[rec_g(3)], b.c3);
+  top_mac(g, rc.w[rec_g(4)], b.c4);
   return RunPoly{top_get(p), top_get(f), top_get(g), 0u};
 }
 
 // poly_state for a TONE_LOW6 chirp: FLAT3, and the set-up bounds B_6, E_5 and G_2..G_4 below 64
 // units of 2^-32 turn of phase over a run, so they are left out.
 __device__ __forceinline__ RunPoly poly_state_low6(const TileRec& rc, const RunBin& b) {
-  Top32 p = top_init(rc.B[0]);
-  top_mac(p, rc.B[1], b.c1);
-  top_mac(p, rc.B[2], b.c2);
-  top_mac(p, rc.B[3], b.c3);
-  top_mac(p, rc.B[4], b.c4);
-  top_mac(p, rc.B[5], b.c5);
-  Top32 f = top_init(rc.E[0]);
-  top_mac(f, rc.E[1], b.c1);
-  top_mac(f, rc.E[2], b.c2);
-  top_mac(f, rc.E[3], b.c3);
-  top_mac(f, rc.E[4], b.c4);
-  Top32 g = top_init(rc.G[0]);
-  top_mac(g, rc.G[1], b.c1);
+  Top32 p = top_init(rc.w[rec_b(0)]);
+  top_mac(p, rc.w[rec_b(1)], b.c1);
+  top_mac(p, rc.w[rec_b(2)], b.c2);
+  top_mac(p, rc.w[rec_b(3)], b.c3);
+  top_mac(p, rc.w[rec_b(4)], b.c4);
+  top_mac(p, rc.w[rec_b(5)], b.c5);
+  Top32 f = top_init(rc.w[rec_e(0)]);
+  top_mac(f, rc.w[rec_e(1)], b.c1);
+  top_mac(f, rc.w[rec_e(2)], b.c2);
+  top_mac(f, rc.w[rec_e(3)], b.c3);
+  top_mac(f, rc.w[rec_e(4)], b.c4);
+  Top32 g = top_init(rc.w[rec_g(0)]);
+  top_mac(g, rc.w[rec_g(1)], b.c1);
   return RunPoly{top_get(p), top_get(f), top_get(g), 0u};
 }
 
 // poly_state for a TONE_LOW3 chirp: LOW6, and B_5, E_3, E_4 left out as well (the set-up bounds all
 // left-out terms below 256 units of 2^-32 turn over a two-run cascade).
 __device__ __forceinline__ RunPoly poly_state_low3(const TileRec& rc, const RunBin& b) {
-  Top32 p = top_init(rc.B[0]);
-  top_mac(p, rc.B[1], b.c1);
-  top_mac(p, rc.B[2], b.c2);
-  top_mac(p, rc.B[3], b.c3);
-  top_mac(p, rc.B[4], b.c4);
-  Top32 f = top_init(rc.E[0]);
-  top_mac(f, rc.E[1], b.c1);
-  top_mac(f, rc.E[2], b.c2);
-  Top32 g = top_init(rc.G[0]);
-  top_mac(g, rc.G[1], b.c1);
+  Top32 p = top_init(rc.w[rec_b(0)]);
+  top_mac(p, rc.w[rec_b(1)], b.c1);
+  top_mac(p, rc.w[rec_b(2)], b.c2);
+  top_mac(p, rc.w[rec_b(3)], b.c3);
+  top_mac(p, rc.w[rec_b(4)], b.c4);
+  Top32 f = top_init(rc.w[rec_e(0)]);
+  top_mac(f, rc.w[rec_e(1)], b.c1);
+  top_mac(f, rc.w[rec_e(2)], b.c2);
+  Top32 g = top_init(rc.w[rec_g(0)]);
+  top_mac(g, rc.w[rec_g(1)], b.c1);
   return RunPoly{top_get(p), top_get(f), top_get(g), 0u};
 }
 
@@ -445,43 +445,33 @@ __device__ __forceinline__ uint64_t round_q64(unsigned __int128 v) {
 }
 
 // The stride-RUN records of a tile from the unit-stride forward differences h[1..DEG] of the
-// chirp phase at the tile start (Q64.64 words, mod 2^128) and its phase word B0.  The order-0
-// words take the run set-up's rounding offsets (poly_state): B_0 + 2^40 + 2^63, E_0, G_0 and
-// H_0 + 2^31.
-template <int DEG, class Args>
+// chirp phase at the tile start (Q64.64 words, mod 2^128) and its phase word B0: the first WORDS
+// words of the record.  The order-0 words take the run set-up's rounding offsets (poly_state):
+// B_0 + 2^40 + 2^63, E_0, G_0 and H_0 + 2^31.
+template <int DEG, int WORDS, class Args>
 __device__ __forceinline__ void stride_records(const unsigned __int128* h, uint64_t B0, const Args& a,
                                                TileRec& out) {
-#pragma unroll
-  for (int q = 0; q < 7; ++q) {
+  // sum over i >= q of h[i + k] W[q][i]: order q of the k-th unit difference
+  auto word = [&](int q, int k) -> uint64_t {
+    if (q + k > DEG) return 0;
     unsigned __int128 s = 0;
 #pragma unroll
-    for (int i = q; i <= DEG; ++i) s += h[i] * (unsigned __int128)a.W[q][i];
-    out.B[q] = (q == 0) ? B0 + B0_OFFSET : (q <= DEG ? round_q64(s) : 0);
-  }
+    for (int i = 0; i <= 6; ++i)
+      if (i >= q && i + k <= DEG) s += h[i + k] * (unsigned __int128)a.W[q][i];
+    return round_q64(s);
+  };
 #pragma unroll
-  for (int q = 0; q < 6; ++q) {
-    unsigned __int128 s = 0;
+  for (int q = 0; q < 7; ++q)
+    if (rec_b(q) < WORDS) out.w[rec_b(q)] = q == 0 ? B0 + B0_OFFSET : word(q, 0);
 #pragma unroll
-    for (int i = q; i + 1 <= DEG; ++i) s += h[i + 1] * (unsigned __int128)a.W[q][i];
-    out.E[q] = (q + 1 <= DEG) ? round_q64(s) : 0;
-    if (q == 0) out.E[0] += HALF32_OFF;
-  }
+  for (int q = 0; q < 6; ++q)
+    if (rec_e(q) < WORDS) out.w[rec_e(q)] = word(q, 1) + (q == 0 ? HALF32_OFF : 0);
 #pragma unroll
-  for (int q = 0; q < 5; ++q) {
-    unsigned __int128 s = 0;
+  for (int q = 0; q < 5; ++q)
+    if (rec_g(q) < WORDS) out.w[rec_g(q)] = word(q, 2) + (q == 0 ? HALF32_OFF : 0);
 #pragma unroll
-    for (int i = q; i + 2 <= DEG; ++i) s += h[i + 2] * (unsigned __int128)a.W[q][i];
-    out.G[q] = (q + 2 <= DEG) ? round_q64(s) : 0;
-    if (q == 0) out.G[0] += HALF32_OFF;
-  }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    unsigned __int128 s = 0;
-#pragma unroll
-    for (int i = q; i + 3 <= DEG; ++i) s += h[i + 3] * (unsigned __int128)a.W[q][i];
-    out.H[q] = (q + 3 <= DEG) ? round_q64(s) : 0;
-    if (q == 0) out.H[0] += HALF32_OFF;
-  }
+  for (int q = 0; q < 4; ++q)
+    if (rec_h(q) < WORDS) out.w[rec_h(q)] = word(q, 3) + (q == 0 ? HALF32_OFF : 0);
 }
 
 // d c mod 2^192 for a multiplier c whose 64-bit limbs above the first L are zero: the partial
@@ -568,7 +558,7 @@ __device__ __forceinline__ void newton_shift_signed(const ChirpRec& c, int64_t m
   }
 }
 
-template <int DEG, class Args>
+template <int DEG, int WORDS, class Args>
 __device__ __forceinline__ void prep_one(const ChirpRec& c, int64_t m, const Args& a, TileRec& out) {
   U192 acc[DEG + 1];
   if (m >= 0 && m < ((int64_t)1 << 29)) {
@@ -581,14 +571,14 @@ __device__ __forceinline__ void prep_one(const ChirpRec& c, int64_t m, const Arg
   unsigned __int128 h[DEG + 1];
 #pragma unroll
   for (int k = 0; k <= DEG; ++k) h[k] = hi128(acc[k]);
-  stride_records<DEG>(h, c.phi_start + acc[0].w2, a, out);   // acc_0 holds 2^127
+  stride_records<DEG, WORDS>(h, c.phi_start + acc[0].w2, a, out);   // acc_0 holds 2^127
 }
 
 // Exponential chirps: the unit forward differences of R(m) = C (e^(alpha m) - 1) at the tile
 // start are C e^(alpha m) q^k (k >= 1, q = e^alpha - 1), in FP64 (a few 1e-10 turn), cut after
 // order 6: the set-up gives a chirp a per-sample table instead when the dropped orders could
 // reach 2^-26 turn over a tile.
-template <class Args>
+template <int WORDS, class Args>
 __device__ __forceinline__ void prep_exp(const ChirpRec& c, int64_t m, const Args& a, TileRec& out) {
   const double alpha = __longlong_as_double((long long)c.d[2]);
   const double C = __longlong_as_double((long long)c.d[3]);
@@ -602,7 +592,7 @@ __device__ __forceinline__ void prep_exp(const ChirpRec& c, int64_t m, const Arg
     h[k] = q64_of(g);
     g *= q;
   }
-  stride_records<6>(h, c.phi_start + (uint64_t)((h[0] + ((unsigned __int128)1 << 63)) >> 64), a, out);
+  stride_records<6, WORDS>(h, c.phi_start + (uint64_t)((h[0] + ((unsigned __int128)1 << 63)) >> 64), a, out);
 }
 
 // Programmatic dependent launch (pipelined chunk sequences): the next kernel in the stream may
@@ -623,6 +613,24 @@ __device__ bool wait_counter(const unsigned long long* ctr, unsigned long long t
   return true;
 }
 
+// Words of a record that the render reads: the run set-up of a linear chirp takes 6 in every tile;
+// one in LOW3 form takes 10 in the tiles that it covers without an amplitude ramp (tile_kind,
+// kind_state); every other takes all.
+__device__ __forceinline__ int rec_words(const ChirpRec& c, const ToneRec& t, int64_t T0) {
+  if (c.flags & TONE_LINEAR) return REC_WORDS_LINEAR;
+  const bool ramp = (t.flags & TONE_AMP_RAMP) && T0 + TILE - 1 > t.a_ns && T0 < t.a_ns + t.a_L;
+  const bool inside = T0 >= c.n_s && T0 + TILE - 1 <= c.n_s + c.L;
+  return (c.flags & TONE_LOW3) && inside && !ramp ? REC_WORDS_LOW3 : REC_WORDS;
+}
+template <int WORDS>
+__device__ __forceinline__ void store_record(TileRec* out, const TileRec& r) {
+  static_assert(WORDS % 2 == 0, "16-byte stores");
+  uint4* o = reinterpret_cast<uint4*>(out);
+#pragma unroll
+  for (int i = 0; i < WORDS / 2; ++i)
+    o[i] = make_uint4((uint32_t)r.w[2 * i], (uint32_t)(r.w[2 * i] >> 32), (uint32_t)r.w[2 * i + 1], (uint32_t)(r.w[2 * i + 1] >> 32));
+}
+
 template <class Args>
 __global__ void __launch_bounds__(128, 5) prep_kernel(const __grid_constant__ Args a) {
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -634,87 +642,133 @@ __global__ void __launch_bounds__(128, 5) prep_kernel(const __grid_constant__ Ar
   const ChirpRec& c = a.chirps[slot];
   if (t == 0) a.act_of_slot[slot] = a.act_base + ai;
   const int64_t T0 = (a.tile0 + t) * (int64_t)TILE;
-  TileRec out;
-  if (c.flags & TONE_LINEAR) prep_one<2>(c, T0 - c.n_s, a, out);
-  else if (c.flags & TONE_EXP) prep_exp(c, T0 - c.n_s, a, out);
-  else prep_one<6>(c, T0 - c.n_s, a, out);
-  a.recs[(int64_t)(a.act_base + ai) * a.n_tiles + t] = out;
+  const int words = rec_words(c, a.tones[c.tone], T0);
+  TileRec* out = a.recs + (int64_t)t * a.rec_stride + a.act_base + ai;
+  TileRec r;
+  if (words == REC_WORDS_LINEAR) {
+    prep_one<2, REC_WORDS_LINEAR>(c, T0 - c.n_s, a, r);
+    store_record<REC_WORDS_LINEAR>(out, r);
+  } else if (words == REC_WORDS_LOW3) {
+    if (c.flags & TONE_EXP) prep_exp<REC_WORDS_LOW3>(c, T0 - c.n_s, a, r);
+    else prep_one<6, REC_WORDS_LOW3>(c, T0 - c.n_s, a, r);
+    store_record<REC_WORDS_LOW3>(out, r);
+  } else {
+    if (c.flags & TONE_EXP) prep_exp<REC_WORDS>(c, T0 - c.n_s, a, r);
+    else prep_one<6, REC_WORDS>(c, T0 - c.n_s, a, r);
+    store_record<REC_WORDS>(out, r);
+  }
 }
 
 // ------------------------------------------------------------------------------------------
 // render
 // ------------------------------------------------------------------------------------------
-// Accumulators: a thread's RUN partial sums as RUN / 2 pairs of consecutive samples (float2).
-// The static and chirp loops compute the sine arguments and the multiply-adds of two samples as
-// packed FP32 pairs (each component rounds as fmaf, so the sums are the same bits as with scalar
-// fmaf): one instruction per tone-sample fewer (8.5 -> 7.5 on the 1000-chirp record).
-typedef float2 Acc[RUN / 2];
+// Geometry of a render CTA: RT = 128 threads take SPT consecutive samples each, RT x SPT samples of
+// one tile: the whole tile (SPT 32) or one of PARTS = RUN / SPT equal parts of it.  A run of RUN
+// samples belongs to PARTS neighbouring lanes; the run cascade is an exact integer recurrence, so
+// a lane that starts r0 samples into its run advances the run's state by r0 in closed form and
+// takes the same integers.  Parts cut the work of a window finer without a change in any sum:
+// see render_parts in the host code for where each form is used.
+template <int SPT>
+struct Geo {
+  static constexpr int PARTS = RUN / SPT;
+  static constexpr int PSAMP = RT * SPT;       // samples of a part
+  static constexpr int PRUNS = RUNS / PARTS;   // runs of a part
+  static constexpr int RW = 32 / PARTS;        // runs of a warp
+};
+
+// Accumulators: a thread's SPT partial sums as SPT / 2 pairs of consecutive samples (float2).
+// The loops compute the sine arguments and the multiply-adds of two samples as packed FP32 pairs
+// (each component rounds as fmaf, so the sums are the same bits as with scalar fmaf).
+template <int SPT>
+using Acc = float2[SPT / 2];
 
 constexpr float TWO_PI_F = 6.28318530717958647692f;
 constexpr float THREE_PI_F = 9.42477796076937971538f;
 
-// acc += (A0 sin(p0), A1 sin(p1)) for two phases already offset by half a turn (see sin_centred)
-__device__ __forceinline__ void acc_pair(float2& acc, float A0, float A1, uint32_t p0, uint32_t p1) {
-  acc.x = fmaf(A0, sin_centred(p0), acc.x);
-  acc.y = fmaf(A1, sin_centred(p1), acc.y);
-}
-// the same for one amplitude, as packed FP32 pairs
-__device__ __forceinline__ void acc_pair_packed(float2& acc, float A, uint32_t p0, uint32_t p1) {
+// the sines of two phases already offset by half a turn (see sin_centred)
+__device__ __forceinline__ float2 sin_pair(uint32_t p0, uint32_t p1) {
   const float2 v = make_float2(mantissa_float(p0), mantissa_float(p1));
   const float2 x = __ffma2_rn(v, make_float2(TWO_PI_F, TWO_PI_F), make_float2(-THREE_PI_F, -THREE_PI_F));
-  acc = __ffma2_rn(make_float2(A, A), make_float2(__sinf(x.x), __sinf(x.y)), acc);
+  return make_float2(__sinf(x.x), __sinf(x.y));
 }
-// acc += (A0 s0, A1 s1) for sines already computed
-__device__ __forceinline__ void acc_pair_s(float2& acc, float A0, float A1, float s0, float s1) {
-  acc.x = fmaf(A0, s0, acc.x);
-  acc.y = fmaf(A1, s1, acc.y);
+// acc += A (sin(p0), sin(p1))
+__device__ __forceinline__ void acc_pair(float2& acc, float A, uint32_t p0, uint32_t p1) {
+  acc = __ffma2_rn(make_float2(A, A), sin_pair(p0, p1), acc);
 }
 
-// Static segment over N samples from acc pair B: p += f per sample.
-template <int B, int N>
-__device__ __forceinline__ void static_loop(uint32_t p, uint32_t f, float A, Acc& acc) {
+// Static segment: p += f per sample.
+template <int SPT>
+__device__ __forceinline__ void static_loop(uint32_t p, uint32_t f, float A, Acc<SPT>& acc) {
 #pragma unroll
-  for (int r = 0; r < N; r += 2) {
+  for (int r = 0; r < SPT; r += 2) {
     const uint32_t p1 = p + f;
-    acc_pair_packed(acc[B + r / 2], A, p, p1);
+    acc_pair(acc[r / 2], A, p, p1);
     p = p1 + f;
   }
 }
 
-// Chirp cascade over N samples from acc pair B: p += f, f += g (and g += h with WITH_H).
-template <int B, int N, bool WITH_H>
-__device__ __forceinline__ void cascade(const RunPoly& q, float A, Acc& acc) {
+// Chirp cascade p += f, f += g (and g += h with WITH_H).  Without h the phases go in blocks of
+// four, p_{k+1} = p_k + f + k g with the multiples of g formed once: one three-input add per
+// sample (16 samples per thread, the loop alone: 4.09 -> 4.40e12 sines/s; 32 samples: 4.40 ->
+// 4.43e12).
+template <int SPT, bool WITH_H>
+__device__ __forceinline__ void cascade(const RunPoly& q, float A, Acc<SPT>& acc) {
   uint32_t p = q.p, f = q.f, g = q.g;
-  const uint32_t h = q.h;
+  if constexpr (WITH_H) {
+    const uint32_t h = q.h;
 #pragma unroll
-  for (int r = 0; r < N; r += 2) {
-    const uint32_t p1 = p + f;
-    uint32_t f1 = f + g;
-    if (WITH_H) g += h;
-    acc_pair_packed(acc[B + r / 2], A, p, p1);
-    p = p1 + f1;
-    f = f1 + g;
-    if (WITH_H) g += h;
+    for (int r = 0; r < SPT; r += 2) {
+      const uint32_t p1 = p + f;
+      const uint32_t f1 = f + g;
+      g += h;
+      acc_pair(acc[r / 2], A, p, p1);
+      p = p1 + f1;
+      f = f1 + g;
+      g += h;
+    }
+  } else {
+    const uint32_t g2 = 2u * g, g3 = 3u * g, g4 = 4u * g;
+#pragma unroll
+    for (int r = 0; r < SPT; r += 4) {
+      const uint32_t p1 = p + f, p2 = p1 + f + g, p3 = p2 + f + g2;
+      acc_pair(acc[r / 2], A, p, p1);
+      acc_pair(acc[r / 2 + 1], A, p2, p3);
+      p = p3 + f + g3;
+      f += g4;
+    }
   }
 }
 
-// Per (tone, run) contribution of one staged tone, added into the thread's partial sums.
+// The state r0 samples later (exact mod 2^32).
+__device__ __forceinline__ RunPoly advance(const RunPoly& q, uint32_t r0) {
+  const uint32_t c2 = r0 * (r0 - 1) / 2, c3 = r0 >= 3 ? r0 * (r0 - 1) * (r0 - 2) / 6 : 0u;
+  RunPoly n;
+  n.p = q.p + r0 * q.f + c2 * q.g + c3 * q.h;
+  n.f = q.f + r0 * q.g + c2 * q.h;
+  n.g = q.g + r0 * q.h;
+  n.h = q.h;
+  return n;
+}
+
+// The same with h = 0.
+__device__ __forceinline__ RunPoly advance3(const RunPoly& q, uint32_t r0) {
+  return RunPoly{q.p + r0 * q.f + (r0 * (r0 - 1) / 2) * q.g, q.f + r0 * q.g, q.g, 0u};
+}
+
 // Amplitude a(n) of a ramping tone (TONE_AMP_RAMP): A before a_ns, A_end from a_ns + a_L on, and
 // A + (A_end - A) s(tau) between, tau = (n - a_ns) / a_L, s linear or minimum-jerk
 // (10 tau^3 - 15 tau^4 + 6 tau^5).  FP32 (tau as m times the rounded 1 / a_L); error
 // <= 6e-7 |A_end - A|.
-// Per run: the offset of the run start into the ramp and 1 / a_L; ramp_amp_at(rr, r) is a(n0 + r),
-// with tau = m (1 / a_L) in FP32 (a function of the absolute sample only, whatever the window).
-struct RampRun {
-  int64_t m0;       // n0 - a_ns
-  int64_t L;
+struct Ramp {
+  int32_t m0;       // the thread's first sample - a_ns, clamped to -RUN .. a_L (beyond, a is constant)
+  int32_t L;
   float inv_L, A, A_end, dA;
   bool minjerk;
 };
-__device__ __forceinline__ RampRun ramp_run_setup(const ToneRec& t, int64_t n0) {
-  RampRun rr;
-  rr.m0 = n0 - t.a_ns;
+__device__ __forceinline__ Ramp ramp_setup(const ToneRec& t, int64_t n) {
+  Ramp rr;
   rr.L = t.a_L;
+  rr.m0 = (int32_t)max((int64_t)-RUN, min((int64_t)t.a_L, n - t.a_ns));
   rr.inv_L = 1.0f / (float)t.a_L;
   rr.A = t.A;
   rr.A_end = t.A_end;
@@ -722,136 +776,86 @@ __device__ __forceinline__ RampRun ramp_run_setup(const ToneRec& t, int64_t n0) 
   rr.minjerk = (t.flags & TONE_AMP_MINJERK) != 0;
   return rr;
 }
-__device__ __forceinline__ float ramp_amp_at(const RampRun& rr, int r) {
-  const int64_t m = rr.m0 + r;
-  if (m <= 0) return rr.A;
-  if (m >= rr.L) return rr.A_end;
-  const float tau = (float)m * rr.inv_L;
-  const float s = rr.minjerk ? tau * tau * tau * fmaf(tau, fmaf(6.f, tau, -15.f), 10.f) : tau;
-  return fmaf(rr.dA, s, rr.A);
+// a(n) at the offsets m (mf: m as floats), two samples as packed pairs
+__device__ __forceinline__ float2 ramp_curve(const Ramp& rr, float2 mf, bool minjerk) {
+  const float2 tau = __fmul2_rn(mf, make_float2(rr.inv_L, rr.inv_L));
+  float2 s = tau;
+  if (minjerk) {
+    const float2 poly = __ffma2_rn(tau, __ffma2_rn(make_float2(6.f, 6.f), tau, make_float2(-15.f, -15.f)),
+                                   make_float2(10.f, 10.f));
+    s = __fmul2_rn(__fmul2_rn(__fmul2_rn(tau, tau), tau), poly);
+  }
+  return __ffma2_rn(make_float2(rr.dA, rr.dA), s, make_float2(rr.A, rr.A));
+}
+__device__ __forceinline__ float2 ramp_amp_pair(const Ramp& rr, int r) {
+  const int m = rr.m0 + r;
+  float2 a = ramp_curve(rr, make_float2((float)m, (float)(m + 1)), rr.minjerk);
+  a.x = m <= 0 ? rr.A : (m >= rr.L ? rr.A_end : a.x);
+  a.y = m + 1 <= 0 ? rr.A : (m + 1 >= rr.L ? rr.A_end : a.y);
+  return a;
 }
 
-// The general paths for the thread's run (samples n0 .. n0 + RUN - 1), used where a tile holds a
-// chirp boundary, an amplitude ramp or a per-sample phase table; col holds the run's RUN sines,
-// sample r at col[r * cs] (a column of the cluster render's shared tile buffer, stride RUNS, or a
-// local array, stride 1).
-__device__ __forceinline__ void tone_run(const ToneRec& tr, const TileRec* rec, const RunBin& rb, float* col,
-                                         Acc& acc, int64_t T0, int64_t n0, const uint32_t* exact_tab, int cs) {
-  constexpr int B = 0;
-  const bool ramp = (tr.flags & TONE_AMP_RAMP) != 0;
-  const bool ramp_run = ramp && n0 + RUN - 1 > tr.a_ns && n0 < tr.a_ns + tr.a_L;   // a(n) varies in the run
-  const float A = (ramp && n0 >= tr.a_ns + tr.a_L) ? tr.A_end : tr.A;
-  const int tcls = classify_tile(tr, T0);
-  int mode;   // 0 static before the chirp, 1 static after, 2 chirp polynomial, 3 general
-  if (tcls == TILE_PRE) {
-    mode = 0;
-  } else if (tcls == TILE_POST) {
-    mode = 1;
-  } else {
-    const int64_t last = n0 + RUN - 1;
-    if (last < tr.n_s) mode = 0;
-    else if (n0 > tr.n_e) mode = 1;
-    else if (n0 >= tr.n_s && last <= tr.n_e && !(tr.flags & TONE_EXACT)) mode = 2;
-    else mode = 3;
-  }
-  if (!ramp && !(tr.flags & TONE_EXACT)) {
-    // no ramp and no table (tile TILE_CHIRP, record present): one loop per warp.  The same
-    // integers as the per-thread paths below, without running three of them one after another
-    // in the warp that holds a chirp boundary.
-    if (__all_sync(0xffffffffu, mode <= 1)) {
-      const uint64_t phi = mode == 0 ? tr.phi_ref : tr.phi_post_ref;
-      const uint64_t F = mode == 0 ? tr.F : tr.F_end;
-      static_loop<B, RUN>(static_p0(phi, F, n0) + HALF_TURN, static_f(F), A, acc);
-      return;
-    }
-    const RunPoly st = poly_state(*rec, rb, (tr.flags & TONE_LINEAR) != 0);
-    if (__all_sync(0xffffffffu, mode == 2)) {
-      if (__all_sync(0xffffffffu, st.h == 0)) cascade<B, RUN, false>(st, A, acc);
-      else cascade<B, RUN, true>(st, A, acc);
-      return;
-    }
-    // a boundary in the warp: sample r takes the static phase before the chirp (r < i1), the
-    // one after it (r > i2), else the chirp cascade; i1, i2 clamped to [-1, RUN]
-    const int i1 = (int)max((int64_t)-1, min((int64_t)RUN, tr.n_s - n0));
-    const int i2 = (int)max((int64_t)-1, min((int64_t)RUN, tr.n_e - n0));
-    uint32_t qa = static_p0(tr.phi_ref, tr.F, n0) + HALF_TURN, qb = static_p0(tr.phi_post_ref, tr.F_end, n0) + HALF_TURN;
-    const uint32_t fa = static_f(tr.F), fb = static_f(tr.F_end);
-    uint32_t pp = st.p, ff = st.f, gg = st.g;
-    const uint32_t hh = st.h;
-#pragma unroll
-    for (int r = 0; r < RUN; r += 2) {
-      const uint32_t ph0 = r < i1 ? qa : (r > i2 ? qb : pp);
-      qa += fa;
-      qb += fb;
-      pp += ff;
-      ff += gg;
-      gg += hh;
-      const uint32_t ph1 = r + 1 < i1 ? qa : (r + 1 > i2 ? qb : pp);
-      qa += fa;
-      qb += fb;
-      pp += ff;
-      ff += gg;
-      gg += hh;
-      acc_pair(acc[B + r / 2], A, A, ph0, ph1);
-    }
+// A ramping tone whose phase follows one cascade over the thread's samples (CHIRP: a chirp, else a
+// static segment).  Where the ramp covers all the samples of the warp and m < 2^24, the sample
+// offsets are stepped in FP32 (exact integers, so the same tau, s and a) and the amplitudes come in
+// packed pairs without selects: 3 (linear) or 8 instructions per two samples.  A warp whose
+// amplitudes are constant takes the plain loop.  (Per sample before: 64-bit compares, a 64-bit
+// conversion and a branch: 600 tones, 500 of them ramping, 200,000 samples took 255 us.)
+template <int SPT, bool CHIRP>
+__device__ __forceinline__ void ramp_loop(RunPoly q, const Ramp& rr, Acc<SPT>& acc) {
+  const bool before = rr.m0 + (SPT - 1) <= 0, after = rr.m0 >= rr.L;
+  if (__all_sync(0xffffffffu, before || after)) {
+    const float A = before ? rr.A : rr.A_end;
+    if constexpr (CHIRP) cascade<SPT, true>(q, A, acc);
+    else static_loop<SPT>(q.p, q.f, A, acc);
     return;
   }
-  if (ramp_run && mode <= 1) {
-    // a ramp on a static segment: stepped phase, the amplitude of ramp_amp per sample
-    const uint64_t phi = mode == 0 ? tr.phi_ref : tr.phi_post_ref;
-    const uint64_t F = mode == 0 ? tr.F : tr.F_end;
-    uint32_t p = static_p0(phi, F, n0) + HALF_TURN;
-    const uint32_t f = static_f(F);
-    const RampRun rr = ramp_run_setup(tr, n0);
-#pragma unroll
-    for (int r = 0; r < RUN; r += 2) {
-      acc_pair(acc[B + r / 2], ramp_amp_at(rr, r), ramp_amp_at(rr, r + 1), p, p + f);
-      p += 2 * f;
-    }
-  } else if (ramp_run) {
-    mode = 3;
-  }
-  if (ramp_run) {
-    if (mode <= 1) return;
-  } else if (mode <= 1) {
-    const uint64_t phi = mode == 0 ? tr.phi_ref : tr.phi_post_ref;
-    const uint64_t F = mode == 0 ? tr.F : tr.F_end;
-    static_loop<B, RUN>(static_p0(phi, F, n0) + HALF_TURN, static_f(F), A, acc);
-    return;
-  }
-  if (mode == 2) {
-    cascade<B, RUN, true>(poly_state(*rec, rb, (tr.flags & TONE_LINEAR) != 0), A, acc);
-  } else {
-    // a segment boundary inside this run, or a table chirp: choose the segment per sample; the
-    // sines go to col, then into the accumulators
-    const uint32_t p_pre = static_p0(tr.phi_ref, tr.F, n0) + HALF_TURN, f_pre = static_f(tr.F);
-    const uint32_t p_post = static_p0(tr.phi_post_ref, tr.F_end, n0) + HALF_TURN, f_post = static_f(tr.F_end);
-    const bool exact = (tr.flags & TONE_EXACT) != 0;
-    RunPoly st = {0, 0, 0, 0};
-    if (!exact && tcls == TILE_CHIRP) st = poly_state(*rec, rb, (tr.flags & TONE_LINEAR) != 0);
-    const int64_t r1 = tr.n_s - n0, r2 = tr.n_e - n0;
-    uint32_t pp = st.p, ff = st.f, gg = st.g;
-    for (int r = 0; r < RUN; ++r) {
-      uint32_t ph;
-      if (r < r1) ph = p_pre + (uint32_t)r * f_pre;
-      else if (r > r2) ph = p_post + (uint32_t)r * f_post;
-      else ph = exact ? exact_tab[tr.tab_off + (int32_t)(r - r1)] + HALF_TURN : pp;
-      col[r * cs] = sin_centred(ph);
-      pp += ff;
-      ff += gg;
-      gg += st.h;
-    }
-    if (ramp_run) {
-      const RampRun rr = ramp_run_setup(tr, n0);
-#pragma unroll
-      for (int r = 0; r < RUN; r += 2)
-        acc_pair_s(acc[B + r / 2], ramp_amp_at(rr, r), ramp_amp_at(rr, r + 1), col[r * cs], col[(r + 1) * cs]);
+  auto step = [&](uint32_t& p0, uint32_t& p1) {   // the next two phases
+    p0 = q.p;
+    p1 = q.p + q.f;
+    if constexpr (CHIRP) {
+      const uint32_t f1 = q.f + q.g;
+      q.g += q.h;
+      q.p = p1 + f1;
+      q.f = f1 + q.g;
+      q.g += q.h;
     } else {
-#pragma unroll
-      for (int r = 0; r < RUN; r += 2) acc_pair_s(acc[B + r / 2], A, A, col[r * cs], col[(r + 1) * cs]);
+      q.p = p1 + q.f;
     }
+  };
+  const bool inside = rr.m0 > 0 && rr.m0 + (SPT - 1) < rr.L && rr.L <= (1 << 24);
+  uint32_t p0, p1;
+  if (!__all_sync(0xffffffffu, inside)) {
+#pragma unroll
+    for (int r = 0; r < SPT; r += 2) {
+      step(p0, p1);
+      acc[r / 2] = __ffma2_rn(ramp_amp_pair(rr, r), sin_pair(p0, p1), acc[r / 2]);
+    }
+    return;
   }
+  const float mf = (float)rr.m0;
+  auto run = [&](bool minjerk) {
+#pragma unroll
+    for (int r = 0; r < SPT; r += 2) {
+      step(p0, p1);
+      const float2 m = __fadd2_rn(make_float2(mf, mf), make_float2((float)r, (float)(r + 1)));
+      acc[r / 2] = __ffma2_rn(ramp_curve(rr, m, minjerk), sin_pair(p0, p1), acc[r / 2]);
+    }
+  };
+  if (rr.minjerk) run(true);
+  else run(false);
 }
+
+// Tile kinds of a tone.  The chirp kinds cover the tile from start to end.
+enum { DESC_STATIC = 0, DESC_STATIC_ROT = 1,
+       DESC_RAMP_STATIC = 2,    // a static segment with an amplitude ramp in the tile
+       DESC_RAMP_CHIRP = 3,     // a chirp that covers the tile, with an amplitude ramp in it
+       DESC_MIXED = 4,          // a chirp boundary or a per-sample phase table in the tile
+       DESC_SKIP = 5,           // a static segment the tensor-core engine sums
+       DESC_LINEAR = 8, DESC_MINJERK = 9,
+       DESC_FLAT3 = 10,         // a degree-6 chirp whose h is 0 in every run (TONE_FLAT3)
+       DESC_LOW6 = 11,          // FLAT3 without the negligible high orders (TONE_LOW6)
+       DESC_LOW3 = 12 };        // LOW6 without B_5, E_3, E_4 (TONE_LOW3)
 
 // Per-stage tone descriptor, built by warp 0 once per (tone, tile) so that the other threads
 // skip the classification and the 64-bit phase set-up of static segments.
@@ -859,13 +863,9 @@ struct alignas(16) Desc {
   uint64_t p0;    // static: phase word at the tile start of the segment covering the tile
   uint64_t F;     // static: its frequency word
   float A;
-  int32_t kind;
+  int32_t rec;    // the tone's record in the stage (chirp kinds, DESC_RAMP_CHIRP, DESC_MIXED)
   float c, s;     // DESC_STATIC_ROT: cos and sin of the per-sample phase step
 };
-enum { DESC_STATIC = 0, DESC_LINEAR = 1, DESC_MINJERK = 2, DESC_MIXED = 3, DESC_STATIC_ROT = 4, DESC_SKIP = 5,
-       DESC_FLAT3 = 6,     // FLAT3: a degree-6 chirp whose h is 0 in every run (TONE_FLAT3)
-       DESC_LOW6 = 7,      // LOW6: FLAT3 without the negligible high orders (TONE_LOW6)
-       DESC_LOW3 = 8 };    // LOW3: LOW6 without B_5, E_3, E_4 (TONE_LOW3)
 
 // Kind of a chirp tile that the chirp covers from start to end (no table, no ramp in the tile).
 __device__ __forceinline__ int chirp_inside_kind(int32_t flags) {
@@ -873,22 +873,16 @@ __device__ __forceinline__ int chirp_inside_kind(int32_t flags) {
          : (flags & TONE_FLAT3) ? DESC_FLAT3 : DESC_MINJERK;
 }
 
-// Descriptor kind of a tone in the tile [T0, T0 + TILE): DESC_STATIC for a static segment (the
-// stage turns it into DESC_STATIC_ROT under the rotator sine), a chirp kind for a chirp that covers
-// the tile without a table, DESC_MIXED for a chirp boundary, a table or an amplitude ramp in the
-// tile, DESC_SKIP for a static segment the tensor-core engine sums.
+// Descriptor kind of a tone in the tile [T0, T0 + TILE) (the stage turns DESC_STATIC into
+// DESC_STATIC_ROT under the rotator sine).
 __device__ __forceinline__ int tile_kind(const ToneRec& tr, int64_t T0, bool skip_static) {
+  if (skip_static && tile_static(tr, T0)) return DESC_SKIP;
   const int tcls = classify_tile(tr, T0);
-  int kind;
-  if (tcls == TILE_PRE || tcls == TILE_POST) {
-    kind = DESC_STATIC;
-  } else {
-    const bool inside = T0 >= tr.n_s && T0 + TILE - 1 <= tr.n_e;
-    kind = (inside && !(tr.flags & TONE_EXACT)) ? chirp_inside_kind(tr.flags) : DESC_MIXED;
-  }
-  if ((tr.flags & TONE_AMP_RAMP) && T0 + TILE - 1 > tr.a_ns && T0 < tr.a_ns + tr.a_L) kind = DESC_MIXED;
-  if (skip_static && tile_static(tr, T0)) kind = DESC_SKIP;
-  return kind;
+  const bool ramp = (tr.flags & TONE_AMP_RAMP) && T0 + TILE - 1 > tr.a_ns && T0 < tr.a_ns + tr.a_L;
+  if (tcls != TILE_CHIRP) return ramp ? DESC_RAMP_STATIC : DESC_STATIC;
+  const bool inside = T0 >= tr.n_s && T0 + TILE - 1 <= tr.n_e;
+  if (!inside || (tr.flags & TONE_EXACT)) return DESC_MIXED;
+  return ramp ? DESC_RAMP_CHIRP : chirp_inside_kind(tr.flags);
 }
 
 // Visit group of a stage's tone: chirps in linear form that may share their run set-up (TONE_PAIR),
@@ -906,11 +900,11 @@ __device__ __forceinline__ int visit_group(int kind, bool listed, bool pair) {
 }
 
 // Run set-up shared by a lane pair.  Lanes 2m and 2m + 1 (runs j and j + 1) take two tones of a
-// group: each evaluates one tone's set-up exactly (the even lane the first tone's, the odd lane the
-// second's) and takes the other tone's from its partner, moved by one run with the cascade's own
-// integer steps (h = 0): forward from run j - 1, p + 32 f + 496 g and f + 32 g (the state the
-// partner's cascade reaches after 32 samples); backward from run j + 1, p - 32 f + 528 g and
-// f - 32 g (C(-32, 2) = 528).  The moved state's error is the cascade's over up to 63 steps
+// group: each evaluates one tone's set-up exactly (the even run's lane the first tone's, the odd
+// run's the second's) and takes the other tone's from its partner, moved by one run with the
+// cascade's own integer steps (h = 0): forward from run j - 1, p + 32 f + 496 g and f + 32 g (the
+// state the partner's cascade reaches after 32 samples); backward from run j + 1, p - 32 f + 528 g
+// and f - 32 g (C(-32, 2) = 528).  The moved state's error is the cascade's over up to 63 steps
 // (pair_setup_ok on the host bounds it).  Every lane of the warp takes part.
 __device__ __forceinline__ RunPoly partner_state(const RunPoly& own, bool odd) {
   const uint32_t p = __shfl_xor_sync(0xffffffffu, own.p, 1);
@@ -927,6 +921,84 @@ __device__ __forceinline__ RunPoly partner_state(const RunPoly& own, bool odd) {
   q.g = g;
   q.h = 0;
   return q;
+}
+
+// A tile with a chirp boundary or a per-sample table (DESC_MIXED): the thread's samples n0s ..
+// n0s + SPT - 1, the first of them r0 samples into the run that starts at n0.  Sample r takes the
+// static phase before the chirp (r < n_s - n0), the one after it (r > n_e - n0), else the chirp's
+// cascade (or its table entry); the amplitude is the ramp's where one is under way.
+template <int SPT>
+__device__ __forceinline__ void mixed_run(const ToneRec& tr, const TileRec* rec, const RunBin& rb, Acc<SPT>& acc,
+                                          int64_t n0, int r0, const uint32_t* exact_tab) {
+  const int64_t n0s = n0 + r0, last = n0s + SPT - 1;
+  const bool ramp = (tr.flags & TONE_AMP_RAMP) != 0;
+  const bool exact = (tr.flags & TONE_EXACT) != 0;
+  const bool ramp_run = ramp && last > tr.a_ns && n0s < tr.a_ns + tr.a_L;   // a(n) varies here
+  const float A = (ramp && n0s >= tr.a_ns + tr.a_L) ? tr.A_end : tr.A;
+  const bool pre = last < tr.n_s, post = n0s > tr.n_e;
+  const uint32_t ur0 = (uint32_t)r0;
+  if (__all_sync(0xffffffffu, (pre || post) && !ramp_run)) {
+    const uint64_t phi = pre ? tr.phi_ref : tr.phi_post_ref;
+    const uint64_t F = pre ? tr.F : tr.F_end;
+    const uint32_t f = static_f(F);
+    static_loop<SPT>(static_p0(phi, F, n0) + HALF_TURN + ur0 * f, f, A, acc);
+    return;
+  }
+  RunPoly st = {0, 0, 0, 0};
+  if (!exact) st = advance(poly_state(*rec, rb, (tr.flags & TONE_LINEAR) != 0), ur0);
+  if (__all_sync(0xffffffffu, !exact && !ramp_run && n0s >= tr.n_s && last <= tr.n_e)) {
+    if (__all_sync(0xffffffffu, st.h == 0)) cascade<SPT, false>(st, A, acc);
+    else cascade<SPT, true>(st, A, acc);
+    return;
+  }
+  // i1, i2: the chirp's samples i1 <= r <= i2 of the thread, clamped to [-1, SPT]
+  const int i1 = (int)max((int64_t)-1, min((int64_t)SPT, tr.n_s - n0s));
+  const int i2 = (int)max((int64_t)-1, min((int64_t)SPT, tr.n_e - n0s));
+  const uint32_t fa = static_f(tr.F), fb = static_f(tr.F_end);
+  uint32_t qa = static_p0(tr.phi_ref, tr.F, n0) + HALF_TURN + ur0 * fa;
+  uint32_t qb = static_p0(tr.phi_post_ref, tr.F_end, n0) + HALF_TURN + ur0 * fb;
+  if (!__any_sync(0xffffffffu, exact || ramp_run)) {
+    auto next = [&](int r) {
+      const uint32_t ph = r < i1 ? qa : (r > i2 ? qb : st.p);
+      qa += fa;
+      qb += fb;
+      st.p += st.f;
+      st.f += st.g;
+      st.g += st.h;
+      return ph;
+    };
+#pragma unroll
+    for (int r = 0; r < SPT; r += 2) {
+      const uint32_t ph0 = next(r);
+      const uint32_t ph1 = next(r + 1);
+      acc_pair(acc[r / 2], A, ph0, ph1);
+    }
+    return;
+  }
+  // table chirps and ramps: the phases one by one into local memory, then the sums
+  const Ramp rr = ramp_setup(tr, n0s);
+  uint32_t col[SPT];
+  const uint32_t* tab = exact ? exact_tab + tr.tab_off : nullptr;
+  const int32_t t0 = (int32_t)(n0s - tr.n_s);   // table index of sample 0 (negative before the chirp)
+#pragma unroll 4
+  for (int r = 0; r < SPT; ++r) {
+    uint32_t ph;
+    if (r < i1) ph = qa + (uint32_t)r * fa;
+    else if (r > i2) ph = qb + (uint32_t)r * fb;
+    else ph = exact ? tab[t0 + r] + HALF_TURN : st.p;
+    col[r] = ph;
+    st.p += st.f;
+    st.f += st.g;
+    st.g += st.h;
+  }
+  if (ramp_run) {
+#pragma unroll
+    for (int r = 0; r < SPT; r += 2)
+      acc[r / 2] = __ffma2_rn(ramp_amp_pair(rr, r), sin_pair(col[r], col[r + 1]), acc[r / 2]);
+  } else {
+#pragma unroll
+    for (int r = 0; r < SPT; r += 2) acc_pair(acc[r / 2], A, col[r], col[r + 1]);
+  }
 }
 
 // Scale, round half to even, clamp and store sample n (inside the window), after adding the
@@ -978,67 +1050,86 @@ __device__ __forceinline__ void store_group(const RenderArgs& a, int64_t n, cons
   for (int u = 0; u < 8; ++u) store_sample(a, n + u, xv[u]);
 }
 
-// Sum over the split without clusters.  Thread t holds samples RUN t .. RUN t + RUN - 1 of the
-// tile in acc.  With split 1 it stores them; otherwise the CTA writes them to its partial tile
-// a.part[(tile split + crank) TILE ...] and counts itself in on a.tile_ctr[tile]; the CTA that
-// brings the count to split - 1 (mod split) is the last of the tile: it sums the split's partials
-// in rank order (as the cluster reduction does: the same FP32 sums) and stores all 4096 samples,
-// thread t taking the 8-sample groups t, t + RT, ... (coalesced 16-byte stores).
+// Sum over the split without clusters.  The thread holds samples at .. at + SPT - 1 of the part
+// in acc.  With split 1 it stores them; otherwise the CTA writes them to its partial part
+// a.part[(unit split + crank) PSAMP ...] (unit: the part's index in the launch) and counts itself in
+// on a.tile_ctr[unit]; the CTA that brings the count to split - 1 (mod split) is the last of the
+// part: it sums the split's partials in rank order (as the cluster reduction does: the same FP32
+// sums) and stores the part, thread t taking the 8-sample groups t, t + RT, ... (coalesced
+// 16-byte stores).  The loads of several ranks are in flight at a time: one rank at a time left
+// the last CTA of a tile waiting for the L2 `split` times in a row (12 us at split 11).
 // In a pipelined sequence (pdl 2) the scratch of this launch was used two launches back: waiting
 // for the preceding launch to complete (which waited for the one before) makes it free.
-__device__ __forceinline__ void tile_epilogue_split(const RenderArgs& a, int tile, int crank, int split, int64_t T0,
-                                                    const Acc& acc) {
+template <int SPT>
+__device__ __forceinline__ void tile_epilogue_split(const RenderArgs& a, int unit, int crank, int split, int64_t P0,
+                                                    int at, const Acc<SPT>& acc) {
+  constexpr int PSAMP = Geo<SPT>::PSAMP;
   const int tid = threadIdx.x;
   __shared__ int s_last;
   const bool vec = q_vec_ok(a) && f_vec_ok(a);
   if (split == 1) {
 #pragma unroll
-    for (int g = 0; g < RUN / 8; ++g) {
+    for (int g = 0; g < SPT / 8; ++g) {
       float xv[8];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         xv[2 * u] = 0.f + acc[4 * g + u].x;
         xv[2 * u + 1] = 0.f + acc[4 * g + u].y;
       }
-      store_group(a, T0 + (int64_t)tid * RUN + 8 * g, xv, vec);
+      store_group(a, P0 + at + 8 * g, xv, vec);
     }
   } else {
     if (a.pdl == 2) pdl_wait();
-    float4* dst = reinterpret_cast<float4*>(a.part + ((int64_t)tile * split + crank) * TILE + tid * RUN);
+    float4* dst = reinterpret_cast<float4*>(a.part + ((int64_t)unit * split + crank) * PSAMP + at);
 #pragma unroll
-    for (int j = 0; j < RUN / 4; ++j)
+    for (int j = 0; j < SPT / 4; ++j)
       __stcg(dst + j, make_float4(acc[2 * j].x, acc[2 * j].y, acc[2 * j + 1].x, acc[2 * j + 1].y));
     __threadfence();
     __syncthreads();
-    if (tid == 0) s_last = atomicAdd(&a.tile_ctr[tile], 1ull) % (unsigned long long)split == (unsigned long long)(split - 1);
+    if (tid == 0) s_last = atomicAdd(&a.tile_ctr[unit], 1ull) % (unsigned long long)split == (unsigned long long)(split - 1);
     __syncthreads();
     if (s_last) {
       __threadfence();
-      // rank by rank, the thread's 8-sample groups tid + RT v, 16-byte loads in flight
-      constexpr int G = TILE / 8 / RT;   // 8-sample groups per thread
-      const float4* src = reinterpret_cast<const float4*>(a.part + (int64_t)tile * split * TILE) + 2 * tid;
-      float xs[G][8];
+      constexpr int G = SPT / 8;             // 8-sample groups per thread
+      constexpr int H = G > 2 ? 2 : G;       // groups summed at a time
+      constexpr int CU = 4 / H;              // ranks in flight
+      const float4* src = reinterpret_cast<const float4*>(a.part + (int64_t)unit * split * PSAMP) + 2 * tid;
 #pragma unroll
-      for (int v = 0; v < G; ++v)
+      for (int v0 = 0; v0 < G; v0 += H) {
+        float xs[H][8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) xs[v][u] = 0.f;
-      for (int c = 0; c < split; ++c) {
+        for (int v = 0; v < H; ++v)
 #pragma unroll
-        for (int v = 0; v < G; ++v) {
-          const float4 lo = __ldcg(src + (int64_t)c * (TILE / 4) + 2 * RT * v);
-          const float4 hi = __ldcg(src + (int64_t)c * (TILE / 4) + 2 * RT * v + 1);
-          xs[v][0] += lo.x;
-          xs[v][1] += lo.y;
-          xs[v][2] += lo.z;
-          xs[v][3] += lo.w;
-          xs[v][4] += hi.x;
-          xs[v][5] += hi.y;
-          xs[v][6] += hi.z;
-          xs[v][7] += hi.w;
+          for (int u = 0; u < 8; ++u) xs[v][u] = 0.f;
+        for (int c = 0; c < split; c += CU) {
+          float4 lo[CU][H], hi[CU][H];
+#pragma unroll
+          for (int k = 0; k < CU; ++k)
+#pragma unroll
+            for (int v = 0; v < H; ++v)
+              if (c + k < split) {
+                lo[k][v] = __ldcg(src + (int64_t)(c + k) * (PSAMP / 4) + 2 * RT * (v0 + v));
+                hi[k][v] = __ldcg(src + (int64_t)(c + k) * (PSAMP / 4) + 2 * RT * (v0 + v) + 1);
+              }
+#pragma unroll
+          for (int k = 0; k < CU; ++k)
+            if (c + k < split) {
+#pragma unroll
+              for (int v = 0; v < H; ++v) {
+                xs[v][0] += lo[k][v].x;
+                xs[v][1] += lo[k][v].y;
+                xs[v][2] += lo[k][v].z;
+                xs[v][3] += lo[k][v].w;
+                xs[v][4] += hi[k][v].x;
+                xs[v][5] += hi[k][v].y;
+                xs[v][6] += hi[k][v].z;
+                xs[v][7] += hi[k][v].w;
+              }
+            }
         }
-      }
 #pragma unroll
-      for (int v = 0; v < G; ++v) store_group(a, T0 + 8 * ((int64_t)tid + RT * v), xs[v], vec);
+        for (int v = 0; v < H; ++v) store_group(a, P0 + 8 * ((int64_t)tid + RT * (v0 + v)), xs[v], vec);
+      }
     }
   }
   if (a.exit_ctr) {   // this CTA's samples (if any) are stored and visible
@@ -1048,31 +1139,39 @@ __device__ __forceinline__ void tile_epilogue_split(const RenderArgs& a, int til
   }
 }
 
-// One CTA's share of one tile: tones [K crank / split, K (crank+1) / split) of window tile `tile`
-// of the render described by `a` (or the listed tones of its bounds), then the sum over the split
-// and the store.  CLUSTER: the split's CTAs form a thread-block cluster, sum through distributed
-// shared memory in rank order and each stores a slice.  Otherwise each CTA writes its partial
-// tile to a.part and the last of the split to finish (a counter per tile) sums the partials in
-// rank order and stores the whole tile: the same sums, and no CTA waits for the others.
-template <bool CLUSTER>
-__device__ __forceinline__ void render_tile(const RenderArgs& a, const int tile, const int crank, const int split) {
+// One CTA's share of one part of a tile: tones [K crank / split, K (crank+1) / split) of window tile
+// unit / PARTS of the render described by `a` (or the listed tones of its bounds), then the sum over
+// the split and the store.  CLUSTER: the split's CTAs form a thread-block cluster, sum through
+// distributed shared memory in rank order and each stores a slice.  Otherwise each CTA writes its
+// partial sums to a.part and the last of the split to finish (a counter per part) sums the partials
+// in rank order and stores the whole part: the same sums, and no CTA waits for the others.
+//
+// The tones go through in stages of STAGE, in the stage's visit order: the groups of visit_group, each
+// in a loop of its own without a per-tone dispatch, then the rest.
+template <int SPT, bool CLUSTER>
+__device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit, const int crank, const int split) {
+  using G = Geo<SPT>;
+  constexpr int PARTS = G::PARTS, RW = G::RW;
+  static_assert(!CLUSTER || SPT == RUN, "cluster sums take whole tiles");
   __shared__ alignas(16) ToneRec s_tone[2][STAGE];
   __shared__ alignas(16) TileRec s_rec[2][STAGE];
   __shared__ alignas(16) Desc s_desc[2][STAGE];
-  __shared__ uint8_t s_order[2][STAGE];          // visit order: linear chirps, LOW6 chirps, the rest
-  __shared__ int s_ngrp[2][N_GRP - 1];            // ends of the visit groups before the last
-  // cluster sums through distributed shared memory: [i][thread]; without clusters the general
-  // per-sample path keeps its run's sines in a local array (lcol) instead, so that the CTA's
-  // shared memory (20 KB) leaves room for AWG_RENDER_SPLIT_MIN_BLOCKS CTAs per SM
+  __shared__ uint8_t s_order[2][STAGE];          // visit order
+  __shared__ uint8_t s_kind[2][STAGE];           // kinds, in visit order
+  __shared__ int s_ngrp[2][N_GRP];                // ends of the visit groups
+  // cluster sums through distributed shared memory: [i][thread]
   __shared__ alignas(16) float s_red[CLUSTER ? TILE : 4];
-  float lcol[RUN];
   __shared__ alignas(8) uint64_t s_bar[4];        // tones[0], tones[1], records[0], records[1]
 
   cg::cluster_group cluster = cg::this_cluster();
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tile = unit / PARTS, part = unit % PARTS;
   const int64_t T0 = (a.tile0 + tile) * (int64_t)TILE;
-  const int64_t n0 = T0 + (int64_t)tid * RUN;       // the thread's run
-  const uint32_t run_off = (uint32_t)(tid * RUN);
+  const int64_t P0 = T0 + (int64_t)part * G::PSAMP;   // the part's first sample
+  // the thread's run of the tile and its first sample in the run (lanes l, l + RW, ... of a warp
+  // share a run, neighbouring lanes have neighbouring runs)
+  const int run = part * G::PRUNS + warp * RW + lane % RW;
+  const uint32_t r0 = (uint32_t)(lane / RW * SPT);
   // positions [l_begin, l_end) of the visit: the CTA's range of tones, or of the tone list
   int l_begin = (int)((int64_t)a.K * crank / split);
   int l_end = (int)((int64_t)a.K * (crank + 1) / split);
@@ -1092,9 +1191,9 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int tile,
   }
   const int n_stages = (l_end - l_begin + STAGE - 1) / STAGE;
 
-  Acc acc;
+  Acc<SPT> acc;
 #pragma unroll
-  for (int r = 0; r < RUN / 2; ++r) acc[r] = make_float2(0.f, 0.f);
+  for (int r = 0; r < SPT / 2; ++r) acc[r] = make_float2(0.f, 0.f);
 
   if (a.pdl == 1) {   // pipelined sequence: the records' set-up (the preceding kernel) is complete
     pdl_wait();         // before the next render may start (it relies on the same set-up)
@@ -1109,7 +1208,7 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int tile,
   }
   __syncthreads();
 
-  // thread 0 issues the tone copies and counts the issues per barrier (for a bounded drain)
+  // thread 0 issues the copies and counts the issues per barrier (for a bounded drain)
   uint32_t issued = 0;   // 8-bit issue count per barrier
   // warp 0: one bulk copy of the stage's contiguous tone records, or one per listed tone
   auto issue_tones = [&](int st) {
@@ -1127,22 +1226,26 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int tile,
       bulk_g2s(&s_tone[st & 1][tid], a.tones + a.tone_list[lb + tid], (uint32_t)sizeof(ToneRec), &s_bar[st & 1]);
     }
   };
-  // warp 0, once the stage's tones have landed: descriptors, and the records of tones that
-  // chirp inside this tile
+  // warp 0, once the stage's tones have landed: descriptors, visit order, and the records of tones
+  // that chirp inside this tile: the window's active chirps are numbered in tone order, so the
+  // stage's records lie one after another and come in one bulk copy
   auto prepare_stage = [&](int st) {
     const int b = st & 1;
     const int cnt = min(STAGE, l_end - (l_begin + st * STAGE));
     bool need = false, pairable = false;
-    const TileRec* src = nullptr;
-    int kind = -1;
+    int kind = DESC_SKIP, act = 0;
     if (tid < cnt) {
       const ToneRec& tr = s_tone[b][tid];
+      const int tcls = classify_tile(tr, T0);
+      need = tcls == TILE_CHIRP && !(tr.flags & TONE_EXACT);
+      if (need) act = a.act_of_slot[tr.slot];
       Desc d;
       const bool ramp = (tr.flags & TONE_AMP_RAMP) != 0;
       d.A = (ramp && T0 >= tr.a_ns + tr.a_L) ? tr.A_end : tr.A;
       d.c = d.s = 0.f;
-      const int tcls = classify_tile(tr, T0);
-      const bool exact = (tr.flags & TONE_EXACT) != 0;
+      d.F = 0;
+      d.p0 = 0;
+      d.rec = 0;
       if (tcls == TILE_PRE || tcls == TILE_POST) {
         const bool pre = tcls == TILE_PRE;
         d.F = pre ? tr.F : tr.F_end;
@@ -1151,46 +1254,44 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int tile,
           d.c = pre ? tr.rot_c : tr.rot_c_end;
           d.s = pre ? tr.rot_s : tr.rot_s_end;
         }
-      } else {
-        d.F = 0;
-        d.p0 = 0;
-        if (!exact) {
-          need = true;
-          src = a.recs + (int64_t)a.act_of_slot[tr.slot] * (a.rec_stride ? a.rec_stride : a.n_tiles) + a.rec_tile0 + tile;
-        }
       }
-      // a ramp inside the tile takes the general per-sample path; static segments the engine sums
-      // are skipped
-      d.kind = tile_kind(tr, T0, a.skip_static != 0);
-      if (d.kind == DESC_STATIC && a.sine_mode == SINE_ROTATOR) d.kind = DESC_STATIC_ROT;
+      kind = tile_kind(tr, T0, a.skip_static != 0);
+      if (kind == DESC_STATIC && a.sine_mode == SINE_ROTATOR) kind = DESC_STATIC_ROT;
       s_desc[b][tid] = d;
-      kind = d.kind;
       pairable = (tr.flags & TONE_PAIR) && !a.skip_static;
     }
-    // visit order: the chirps that cover the tile in linear form, those in LOW6 form, the static
-    // tones (SFU or rotator), then the rest; tone order within each group.  The first three
-    // groups run in loops without a per-tone dispatch.  The order of the FP32 sums then depends
-    // on which tones share a stage; with a tone list (the window's listed tones) that changes with
-    // the window, so listed renders keep plain tone order, and every window cut gives the same bits.
-    const int grp = visit_group(kind, a.tone_list != nullptr, pairable);
+    // visit order: the chirps that cover the tile in linear form, those in LOW3 and LOW6 form, the
+    // static tones (SFU or rotator), then the rest; tone order within each group.  The order of the
+    // FP32 sums then depends on which tones share a stage; with a tone list (the window's listed
+    // tones) that changes with the window, so listed renders keep plain tone order, and every window
+    // cut gives the same bits.  Skipped tones are left out.
+    const int grp = kind == DESC_SKIP ? -1 : visit_group(kind, a.tone_list != nullptr, pairable);
     const unsigned below = (1u << tid) - 1u;
     int pos = 0, end = 0;
 #pragma unroll
     for (int g = 0; g < N_GRP; ++g) {
-      const unsigned m = __ballot_sync(0xffffffffu, tid < cnt && grp == g);
+      const unsigned m = __ballot_sync(0xffffffffu, grp == g);
       if (grp == g) pos = end + __popc(m & below);
       end += __popc(m);
-      if (tid == 0 && g < N_GRP - 1) s_ngrp[b][g] = end;
+      if (tid == 0) s_ngrp[b][g] = end;
     }
-    if (tid < cnt) s_order[b][pos] = (uint8_t)tid;
+    if (grp >= 0) {
+      s_order[b][pos] = (uint8_t)tid;
+      s_kind[b][pos] = (uint8_t)kind;
+    }
     const unsigned mask = __ballot_sync(0xffffffffu, need);
+    const int first = __shfl_sync(0xffffffffu, act, mask ? __ffs(mask) - 1 : 0);
+    const int last = __shfl_sync(0xffffffffu, act, mask ? 31 - __clz(mask) : 0);
+    if (need) s_desc[b][tid].rec = act - first;
     if (tid == 0) {
+      const uint32_t bytes = mask ? (uint32_t)(last - first + 1) * (uint32_t)sizeof(TileRec) : 0u;
       fence_proxy_async();
-      mbar_arrive_expect_tx(&s_bar[2 + b], (uint32_t)__popc(mask) * (uint32_t)sizeof(TileRec));
+      mbar_arrive_expect_tx(&s_bar[2 + b], bytes);
       issued += 1u << (8 * (2 + b));
+      if (bytes)
+        bulk_g2s(&s_rec[b][0], a.recs + (int64_t)(a.rec_tile0 + tile) * a.rec_stride + first, bytes, &s_bar[2 + b]);
     }
     __syncwarp();
-    if (need) bulk_g2s(&s_rec[b][tid], src, (uint32_t)sizeof(TileRec), &s_bar[2 + b]);
   };
 
   bool ok = true;
@@ -1198,15 +1299,13 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int tile,
     if (tid < 32) {
       issue_tones(0);
       if (n_stages > 1) issue_tones(1);
-    }
-    if (tid < 32) {
       ok &= mbar_wait(&s_bar[0], 0);
       prepare_stage(0);
     }
     __syncthreads();   // stage-0 descriptors visible
   }
   int fail_stage = -1;
-  const RunBin rb0 = run_binomials(tid);
+  const RunBin rb = run_binomials(run);
   for (int st = 0; st < n_stages; ++st) {
     const int b = st & 1;
     const uint32_t par = (uint32_t)((st >> 1) & 1);
@@ -1219,75 +1318,101 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int tile,
     // the same decision in every lane of the warp: the loops below exchange values between lanes
     ok = __all_sync(0xffffffffu, ok);
     if (ok) {
-      const int cnt = min(STAGE, l_end - (l_begin + st * STAGE));
       const int e_lp = s_ngrp[b][GRP_LIN_PAIR], e_lin = s_ngrp[b][GRP_LIN], e_l3p = s_ngrp[b][GRP_LOW3_PAIR],
-                e_l6p = s_ngrp[b][GRP_LOW6_PAIR], e_low6 = s_ngrp[b][GRP_LOW6], e_static = s_ngrp[b][GRP_STATIC];
-      auto linear = [&](int i) { cascade<0, RUN, false>(poly_state(s_rec[b][i], rb0, true), s_desc[b][i].A, acc); };
-      // LOW6, FLAT3: the third difference rounds to 0 everywhere (set-up bound), g is constant
-      auto low6 = [&](int i) { cascade<0, RUN, false>(poly_state_low6(s_rec[b][i], rb0), s_desc[b][i].A, acc); };
-      auto low3 = [&](int i) { cascade<0, RUN, false>(poly_state_low3(s_rec[b][i], rb0), s_desc[b][i].A, acc); };
-      auto flat3 = [&](int i) { cascade<0, RUN, false>(poly_state_flat3(s_rec[b][i], rb0), s_desc[b][i].A, acc); };
-      auto static_sfu = [&](int i) {
-        const Desc& d = s_desc[b][i];
-        static_loop<0, RUN>((uint32_t)((mac_u32(d.p0 + P_OFFSET, d.F, run_off)) >> 32) + HALF_TURN, static_f(d.F), d.A, acc);
+                e_l6p = s_ngrp[b][GRP_LOW6_PAIR], e_low6 = s_ngrp[b][GRP_LOW6], e_static = s_ngrp[b][GRP_STATIC],
+                n_vis = s_ngrp[b][GRP_REST];
+      auto record = [&](int i) -> const TileRec& { return s_rec[b][s_desc[b][i].rec]; };
+      // a chirp run with h = 0 from its run state
+      auto chirp = [&](const RunPoly& q, int i) {
+        cascade<SPT, false>(PARTS > 1 ? advance3(q, r0) : q, s_desc[b][i].A, acc);
       };
-      auto static_rot = [&](int i) {
-        // the exact phase word at the run start, SFU sine and cosine once, then 31 rotations by
-        // the per-sample step on the FP32 pipe (amplitude folded into the phasor)
-        const Desc& d = s_desc[b][i];
-        const float c = d.c, s = d.s;
-        const uint64_t w = d.p0 + (uint64_t)run_off * d.F;
+      auto linear = [&](int i) { chirp(poly_state(record(i), rb, true), i); };
+      auto low6 = [&](int i) { chirp(poly_state_low6(record(i), rb), i); };
+      auto low3 = [&](int i) { chirp(poly_state_low3(record(i), rb), i); };
+      auto flat3 = [&](int i) { chirp(poly_state_flat3(record(i), rb), i); };
+      auto static_state = [&](const Desc& d) {   // the thread's first sample
+        const uint32_t f = static_f(d.F);
+        const uint32_t p = (uint32_t)((mac_u32(d.p0 + P_OFFSET, d.F, (uint32_t)(run * RUN))) >> 32) + HALF_TURN;
+        return RunPoly{PARTS > 1 ? p + r0 * f : p, f, 0u, 0u};
+      };
+      auto static_sfu = [&](int i) {
+        const RunPoly q = static_state(s_desc[b][i]);
+        static_loop<SPT>(q.p, q.f, s_desc[b][i].A, acc);
+      };
+      // the exact phase word at the run start, SFU sine and cosine once, then 31 rotations by the
+      // per-sample step on the FP32 pipe (amplitude folded into the phasor)
+      auto phasor = [&](const Desc& d, float& re, float& im) {
+        const uint64_t w = d.p0 + (uint64_t)(uint32_t)(run * RUN) * d.F;
         float sn, cs;
         __sincosf((float)(int32_t)(w >> 32) * 1.46291807926715968e-9f, &sn, &cs);   // 2 pi / 2^32
-        float im = d.A * sn, re = d.A * cs;
+        im = d.A * sn;
+        re = d.A * cs;
+      };
+      auto rotate = [](float& re, float& im, float c, float s) {
+        const float t = fmaf(re, c, -im * s);
+        im = fmaf(re, s, im * c);
+        re = t;
+      };
+      auto static_rot = [&](int i) {
+        const Desc& d = s_desc[b][i];
+        float re, im;
+        phasor(d, re, im);
+        const float c = d.c, s = d.s;
+        if (PARTS > 1)
+          for (uint32_t r = 0; r < r0; ++r) rotate(re, im, c, s);
 #pragma unroll
-        for (int r = 0; r < RUN; ++r) {
+        for (int r = 0; r < SPT; ++r) {
           if (r & 1) acc[r / 2].y += im;
           else acc[r / 2].x += im;
-          const float t = fmaf(re, c, -im * s);
-          im = fmaf(re, s, im * c);
-          re = t;
+          rotate(re, im, c, s);
         }
       };
       // the sharing groups two tones at a time: one set-up per lane, the other tone's state from the
       // partner lane (partner_state); per sample the first tone's multiply-add, then the second's,
       // as in two single loops; an odd group's last tone alone
-      const bool odd = (tid & 1) != 0;
+      const bool odd = (run & 1) != 0;
+      auto pair = [&](const RunPoly& own, int i, int k) {
+        const RunPoly oth = partner_state(own, odd);
+        chirp(odd ? oth : own, i);
+        chirp(odd ? own : oth, k);
+      };
       for (int o = 0; o + 1 < e_lp; o += 2) {
         const int i = s_order[b][o], k = s_order[b][o + 1];
-        const RunPoly own = poly_state(s_rec[b][odd ? k : i], rb0, true);
-        const RunPoly oth = partner_state(own, odd);
-        cascade<0, RUN, false>(odd ? oth : own, s_desc[b][i].A, acc);
-        cascade<0, RUN, false>(odd ? own : oth, s_desc[b][k].A, acc);
+        pair(poly_state(record(odd ? k : i), rb, true), i, k);
       }
       for (int o = e_lp & ~1; o < e_lin; ++o) linear(s_order[b][o]);
       for (int o = e_lin; o + 1 < e_l3p; o += 2) {
         const int i = s_order[b][o], k = s_order[b][o + 1];
-        const RunPoly own = poly_state_low3(s_rec[b][odd ? k : i], rb0);
-        const RunPoly oth = partner_state(own, odd);
-        cascade<0, RUN, false>(odd ? oth : own, s_desc[b][i].A, acc);
-        cascade<0, RUN, false>(odd ? own : oth, s_desc[b][k].A, acc);
+        pair(poly_state_low3(record(odd ? k : i), rb), i, k);
       }
       if ((e_l3p - e_lin) & 1) low3(s_order[b][e_l3p - 1]);
       for (int o = e_l3p; o + 1 < e_l6p; o += 2) {
         const int i = s_order[b][o], k = s_order[b][o + 1];
-        const RunPoly own = poly_state_low6(s_rec[b][odd ? k : i], rb0);
-        const RunPoly oth = partner_state(own, odd);
-        cascade<0, RUN, false>(odd ? oth : own, s_desc[b][i].A, acc);
-        cascade<0, RUN, false>(odd ? own : oth, s_desc[b][k].A, acc);
+        pair(poly_state_low6(record(odd ? k : i), rb), i, k);
       }
       for (int o = e_l3p + ((e_l6p - e_l3p) & ~1); o < e_low6; ++o) low6(s_order[b][o]);
       if (a.sine_mode == SINE_ROTATOR) {
         for (int o = e_low6; o < e_static; ++o) static_rot(s_order[b][o]);
       } else {
-        for (int o = e_low6; o < e_static; ++o) static_sfu(s_order[b][o]);
+        // the next tone's set-up before this tone's loop
+        RunPoly nx = {0, 0, 0, 0};
+        float nA = 0.f;
+        if (e_low6 < e_static) {
+          const Desc& d = s_desc[b][s_order[b][e_low6]];
+          nx = static_state(d);
+          nA = d.A;
+        }
+        for (int o = e_low6; o < e_static; ++o) {
+          const RunPoly q = nx;
+          const float A = nA;
+          const Desc& d = s_desc[b][s_order[b][min(o + 1, e_static - 1)]];
+          nx = static_state(d);
+          nA = d.A;
+          static_loop<SPT>(q.p, q.f, A, acc);
+        }
       }
-      for (int o = e_static; o < cnt; ++o) {
-        const int i = s_order[b][o];
-        const Desc& d = s_desc[b][i];
-        const int kind = d.kind;
-        const float A = d.A;
-        if (kind == DESC_SKIP) continue;
+      for (int o = e_static; o < n_vis; ++o) {
+        const int i = s_order[b][o], kind = s_kind[b][o];
         if (kind == DESC_STATIC) {
           static_sfu(i);
         } else if (kind == DESC_STATIC_ROT) {
@@ -1303,12 +1428,20 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int tile,
         } else if (kind == DESC_MINJERK) {
           // third difference below 2^-33 turn (long ramps): g is constant over the run, the same
           // integers as the loop with h
-          const RunPoly q0 = poly_state(s_rec[b][i], rb0, false);
-          if (__all_sync(0xffffffffu, q0.h == 0)) cascade<0, RUN, false>(q0, A, acc);
-          else cascade<0, RUN, true>(q0, A, acc);
+          const RunPoly q0 = poly_state(record(i), rb, false);
+          if (__all_sync(0xffffffffu, q0.h == 0)) chirp(q0, i);
+          else cascade<SPT, true>(PARTS > 1 ? advance(q0, r0) : q0, s_desc[b][i].A, acc);
         } else {
-          if constexpr (CLUSTER) tone_run(s_tone[b][i], &s_rec[b][i], rb0, &s_red[tid], acc, T0, n0, a.exact_tab, RUNS);
-          else tone_run(s_tone[b][i], &s_rec[b][i], rb0, lcol, acc, T0, n0, a.exact_tab, 1);
+          const ToneRec& tr = s_tone[b][i];
+          const int64_t n0 = T0 + (int64_t)run * RUN;
+          if (kind == DESC_RAMP_STATIC) {
+            ramp_loop<SPT, false>(static_state(s_desc[b][i]), ramp_setup(tr, n0 + r0), acc);
+          } else if (kind == DESC_RAMP_CHIRP) {
+            const RunPoly q = poly_state(record(i), rb, (tr.flags & TONE_LINEAR) != 0);
+            ramp_loop<SPT, true>(advance(q, r0), ramp_setup(tr, n0 + r0), acc);
+          } else {
+            mixed_run<SPT>(tr, &record(i), rb, acc, n0, (int)r0, a.exact_tab);
+          }
         }
       }
     }
@@ -1331,7 +1464,7 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int tile,
   }
 
   if constexpr (!CLUSTER) {
-    tile_epilogue_split(a, tile, crank, split, T0, acc);
+    tile_epilogue_split<SPT>(a, unit, crank, split, P0, (run - part * G::PRUNS) * RUN + (int)r0, acc);
   } else {
     // partial sums -> shared memory ([i][thread], sample RUN thread + i), then the cluster-wide
     // sum in rank order
@@ -1365,28 +1498,25 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int tile,
       const int sidx = s_first + u;
       if (u < per && sidx < hi) store_sample(a, T0 + sidx, xs[u]);
     }
-    if (a.exit_ctr) {   // this CTA's samples are stored and visible
-      __threadfence();
-      __syncthreads();
-      if (tid == 0) atomicAdd(a.exit_ctr, 1ull);
-    }
   }
 }
 
-// 96 registers: five CTAs of RT threads per SM (the cluster and batched renders)
+// Register budgets, by CTAs per SM.  Whole tiles: six (80 registers, 56 bytes of spill loads); the
+// 1000-chirp 35 ms record took 2636 us at six, 2703 at seven (72 registers), 2711 at five; the batched
+// and cluster renders keep five (no spills).  Parts need fewer accumulators: eight.
 #define AWG_RENDER_MIN_BLOCKS 5
-// The direct render: seven CTAs per SM (72 registers, some spills, 20 KB of shared memory each) ran
-// the 1000-chirp record 1.6 % faster than six and six 1.6 % faster than five; the batched render
-// of the served stream, whose spills grow more, stays at five.
-#define AWG_RENDER_SPLIT_MIN_BLOCKS 7
+#define AWG_RENDER_SPLIT_MIN_BLOCKS 6
+#define AWG_RENDER_PART_MIN_BLOCKS 8
 __global__ void __launch_bounds__(RT, AWG_RENDER_MIN_BLOCKS) render_kernel(const __grid_constant__ RenderArgs a) {
   cg::cluster_group cluster = cg::this_cluster();
-  render_tile<true>(a, blockIdx.x / a.split, (int)cluster.block_rank(), a.split);
+  render_tile<RUN, true>(a, blockIdx.x / a.split, (int)cluster.block_rank(), a.split);
 }
 
-// The same without clusters (a.part set): CTA blockIdx.x takes rank blockIdx.x % split.
-__global__ void __launch_bounds__(RT, AWG_RENDER_SPLIT_MIN_BLOCKS) render_split_kernel(const __grid_constant__ RenderArgs a) {
-  render_tile<false>(a, blockIdx.x / a.split, blockIdx.x % a.split, a.split);
+// The same without clusters (a.part set when split > 1): CTA blockIdx.x takes rank blockIdx.x % split.
+template <int SPT>
+__global__ void __launch_bounds__(RT, SPT == RUN ? AWG_RENDER_SPLIT_MIN_BLOCKS : AWG_RENDER_PART_MIN_BLOCKS)
+    render_split_kernel(const __grid_constant__ RenderArgs a) {
+  render_tile<SPT, false>(a, blockIdx.x / a.split, blockIdx.x % a.split, a.split);
 }
 
 // Several renders in one grid (continuous batching): CTA group i (split CTAs) renders window tile
@@ -1397,7 +1527,7 @@ __global__ void __launch_bounds__(RT, AWG_RENDER_MIN_BLOCKS) render_batch_split_
                                                                                        const int2* __restrict__ items,
                                                                                        int split) {
   const int2 it = items[blockIdx.x / split];
-  render_tile<false>(reqs[it.x], it.y, (int)(blockIdx.x % split), split);
+  render_tile<RUN, false>(reqs[it.x], it.y, (int)(blockIdx.x % split), split);
 }
 
 // The 32-bit phase the render feeds to the sine for sample s of the tile [T0, T0 + TILE) (any
@@ -1491,7 +1621,7 @@ __global__ void trace_kernel(const __grid_constant__ TraceArgs a) {
   const ToneRec t = a.tones[a.tone];
   const TileRec* rec = nullptr;
   if (classify_tile(t, T0) == TILE_CHIRP && !(t.flags & TONE_EXACT))
-    rec = a.recs + (int64_t)a.act_of_slot[t.slot] * a.n_tiles + (tile_abs - a.tile0);
+    rec = a.recs + (tile_abs - a.tile0);   // the one active chirp of the window
   a.out[i] = phase32_at(t, rec, a.chirps, T0, (int)(n - T0), a.inv_odd, pair_role(a, a.tone, T0));
 }
 
@@ -1512,7 +1642,9 @@ int device_sm_count() {
 cudaError_t render_setup_attributes() {
   cudaError_t e = cudaFuncSetAttribute(render_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   // shared memory before L1 for AWG_RENDER_SPLIT_MIN_BLOCKS CTAs
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(render_split_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(render_split_kernel<32>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(render_split_kernel<16>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(render_split_kernel<8>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   return e;
 }
 
@@ -1530,12 +1662,14 @@ cudaError_t launch_prep(const PrepArgs& a, cudaStream_t s) {
   if (a.n_active <= SMALL_PREP) {   // the small parameter form: fewer bytes copied with the launch
     PrepArgsT<SMALL_PREP> b;
     b.chirps = a.chirps;
+    b.tones = a.tones;
     b.recs = a.recs;
     b.act_of_slot = a.act_of_slot;
     b.tile0 = a.tile0;
     b.n_tiles = a.n_tiles;
     b.n_active = a.n_active;
     b.act_base = a.act_base;
+    b.rec_stride = a.rec_stride;
     for (int q = 0; q < 7; ++q)
       for (int i = 0; i < 7; ++i) b.W[q][i] = a.W[q][i];
     for (int q = 0; q < 3; ++q)
@@ -1606,7 +1740,8 @@ cudaError_t launch_join(const unsigned long long* exit_ctr, unsigned long long t
 cudaError_t launch_render(const RenderArgs& a, cudaStream_t s) {
   if (a.n_tiles == 0) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(a.n_tiles * a.split), 1, 1);
+  const int parts = a.cluster ? 1 : a.parts;
+  cfg.gridDim = dim3((unsigned)(a.n_tiles * parts * a.split), 1, 1);
   cfg.blockDim = dim3(RT, 1, 1);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = s;
@@ -1617,10 +1752,12 @@ cudaError_t launch_render(const RenderArgs& a, cudaStream_t s) {
   attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
-  if (a.part) {   // no cluster: the split sums through the scratch partials
+  if (!a.cluster) {   // the split sums through the scratch partials
     cfg.attrs = attr + 1;
     cfg.numAttrs = a.pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, render_split_kernel, a);
+    if (parts == 4) return cudaLaunchKernelEx(&cfg, render_split_kernel<8>, a);
+    if (parts == 2) return cudaLaunchKernelEx(&cfg, render_split_kernel<16>, a);
+    return cudaLaunchKernelEx(&cfg, render_split_kernel<32>, a);
   }
   cfg.attrs = attr;
   cfg.numAttrs = a.pdl ? 2 : 1;
@@ -1654,11 +1791,11 @@ __global__ void __launch_bounds__(RT, AWG_RENDER_MIN_BLOCKS) sfu_rate_kernel(flo
   uint32_t p = id * 0x9E3779B9u;
   const uint32_t f = (id * 0x85EBCA6Bu) | 1u;
   const float A = 1e-3f;
-  Acc acc;
+  Acc<RUN> acc;
 #pragma unroll
   for (int r = 0; r < RUN / 2; ++r) acc[r] = make_float2(0.f, 0.f);
   for (int k = 0; k < runs; ++k) {
-    static_loop<0, RUN>(p, f, A, acc);
+    static_loop<RUN>(p, f, A, acc);
     p += (uint32_t)RUN * f;
   }
   float t = 0.f;
@@ -1682,11 +1819,11 @@ __global__ void __launch_bounds__(RT, AWG_RENDER_MIN_BLOCKS) chirp_rate_kernel(f
   q.g = (id * 0xC2B2AE35u) >> 8;
   q.h = 0;
   const float A = 1e-3f;
-  Acc acc;
+  Acc<RUN> acc;
 #pragma unroll
   for (int r = 0; r < RUN / 2; ++r) acc[r] = make_float2(0.f, 0.f);
   for (int k = 0; k < runs; ++k) {
-    cascade<0, RUN, false>(q, A, acc);
+    cascade<RUN, false>(q, A, acc);
     q.p += 32u * q.f + 496u * q.g;   // the state after the run
     q.f += 32u * q.g;
   }
