@@ -278,8 +278,9 @@ int awg_render_phases(awg_t* h, int32_t tone, int64_t n0, int32_t count, uint32_
  * whose partial sums are added in rank order.  For information. */
 int32_t awg_tone_split(const awg_t* h);
 
-/* Sum of the device time (ms) of the last render's kernels, recorded with CUDA events; it is
- * valid once that render has completed (e.g. after synchronising its stream).  -1 if none. */
+/* Device time (ms) of the last render, from the start of its first kernel to the end of its last
+ * CTA (device clock); it is valid once that render has completed (e.g. after synchronising its
+ * stream).  -1 if none. */
 float awg_last_render_ms(awg_t* h);
 
 /* Profiling mode: while on, every render records CUDA events on its stream around its chirp

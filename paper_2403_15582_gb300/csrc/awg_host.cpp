@@ -597,7 +597,8 @@ struct awg {
   int32_t periodic_log2 = 0;
   int64_t periodic_start = -1;
   cudaStream_t priv = nullptr;
-  cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev_done = nullptr;
+  cudaEvent_t ev_done = nullptr;
+  unsigned long long* d_times = nullptr;   // device times of the last render's start and end
   // stream-ordered uploads of changed records (awg_set_chirps): pinned staging, copied on the
   // private stream after the last render issued (ev_done); later launches wait for ev_upload
   unsigned char* stage = nullptr;
@@ -1031,6 +1032,24 @@ std::vector<int32_t> active_slots(const awg_t* h, int64_t c, int64_t n, int64_t*
   return active;
 }
 
+// Arguments of the set-up launch of active chirps [b, b + MAX_ACTIVE_PER_LAUNCH) of a window (the
+// record buffers are the caller's).
+void prep_args(const awg_t* h, const std::vector<int32_t>& active, size_t b, int64_t tile0, int32_t n_tiles,
+               awgk::PrepArgs* pa) {
+  std::memset(pa, 0, offsetof(awgk::PrepArgs, slots));
+  pa->chirps = h->d_chirps;
+  pa->tones = h->d_tones;
+  pa->tile0 = tile0;
+  pa->n_tiles = n_tiles;
+  pa->n_active = (int32_t)std::min<size_t>(awgk::MAX_ACTIVE_PER_LAUNCH, active.size() - b);
+  pa->act_base = (int32_t)b;
+  pa->rec_stride = (int32_t)active.size();
+  std::memcpy(pa->W, h->W, sizeof(pa->W));
+  std::memcpy(pa->inv_odd, h->inv_odd, sizeof(pa->inv_odd));
+  pa->more = b + (size_t)pa->n_active < active.size();
+  std::memcpy(pa->slots, active.data() + b, (size_t)pa->n_active * sizeof(int32_t));
+}
+
 // Parts a tile's samples are cut into (RenderArgs::parts) for work of `tiles` tiles.  A CTA is one
 // rank of one part; c of them land on the busiest SM.  Halves and quarters repeat the run set-ups (per
 // SM 0.56 and 0.36 of a whole tile's time instead of 0.5 and 0.25), so they pay only where whole
@@ -1052,6 +1071,124 @@ int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
                   const float* base, int32_t skip_static, const int32_t* tone_list = nullptr, int32_t n_list = 0,
                   int32_t list_split = 0, const int32_t* list_bounds = nullptr);
 int render_engine(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream, int32_t q_stride);
+
+// One direct render of the window [cursor, cursor + n): the plan (buffers made large enough), the
+// chirp tile set-up and the render launches.  Every launch may start while the kernel before it in
+// the stream still runs (RenderArgs::pdl): a render's start, its set-up's arithmetic and the launch
+// gaps lie beside the end of the render before (no event is recorded between the kernels of a call
+// but in profiling mode).
+struct Window {
+  int64_t c, n, tile0;
+  int32_t n_tiles, per_launch;
+  int32_t split;              // CTAs per part of a tile (set by the caller)
+  bool first;                 // its first kernel starts the call (device time)
+  std::vector<int32_t> active;
+  cudaEvent_t pe[4] = {nullptr, nullptr, nullptr, nullptr};   // profiling
+  int64_t launches = 0;
+};
+
+int window_plan(awg_t* h, int64_t n, Window* w) {
+  w->c = h->cursor;
+  w->n = n;
+  const int64_t n_tiles = (w->c + n - 1) / awgk::TILE - w->c / awgk::TILE + 1;
+  if (n_tiles > (int64_t)(INT32_MAX / awgk::MAX_SPLIT)) return fail(AWG_EINVAL, "render window too long");
+  w->active = active_slots(h, w->c, n, &w->tile0, &w->n_tiles);
+  int st = ensure(&h->d_recs, &h->cap_recs, std::max<size_t>(1, w->active.size() * (size_t)w->n_tiles), h, "tile records");
+  if (st) return st;
+  // With a split, the window goes out in launches of at most SPLIT_LAUNCH_TILES tiles, on
+  // alternating scratch buffers.
+  w->per_launch = w->split > 1 ? std::min(w->n_tiles, SPLIT_LAUNCH_TILES) : w->n_tiles;
+  if (w->split > 1 && (st = ensure_split_scratch(h, w->per_launch, w->split))) return st;
+  if (h->profiling) {
+    while (h->prof_ev.size() < 4 * (h->prof_calls + 1)) {
+      cudaEvent_t ev;
+      const cudaError_t e = cudaEventCreate(&ev);
+      if (e != cudaSuccess) return cuda_fail(e, "profiling event");
+      h->prof_ev.push_back(ev);
+    }
+    for (int i = 0; i < 4; ++i) w->pe[i] = h->prof_ev[4 * h->prof_calls + (size_t)i];
+  }
+  return AWG_OK;
+}
+
+// The chirp tile set-up, in stream order right before the render.  (Running it on a second stream,
+// overlapped with the previous render, takes SM slots from the render and pushes its grid into a
+// second wave; measured slower.)  more: another window's set-up follows.
+int window_setup(awg_t* h, Window* w, bool more, cudaStream_t s) {
+  cudaError_t e;
+  if ((e = order_after_uploads(h, s)) != cudaSuccess) return cuda_fail(e, "upload ordering");
+  if (w->pe[0] && (e = cudaEventRecord(w->pe[0], s)) != cudaSuccess) return cuda_fail(e, "event");
+  for (size_t b = 0; b < w->active.size(); b += awgk::MAX_ACTIVE_PER_LAUNCH) {
+    awgk::PrepArgs pa;
+    prep_args(h, w->active, b, w->tile0, w->n_tiles, &pa);
+    pa.recs = h->d_recs;
+    pa.act_of_slot = h->d_act;
+    pa.start = w->first && b == 0 ? h->d_times : nullptr;
+    if (more) pa.more = 1;
+    if ((e = counted(h, awgk::launch_prep(pa, s))) != cudaSuccess) return cuda_fail(e, "prep launch");
+    ++w->launches;
+  }
+  if (w->pe[1] && (e = cudaEventRecord(w->pe[1], s)) != cudaSuccess) return cuda_fail(e, "event");
+  if (w->pe[2] && (e = cudaEventRecord(w->pe[2], s)) != cudaSuccess) return cuda_fail(e, "event");
+  return AWG_OK;
+}
+
+// The render launches; out_q, out_f, base, the tone list and q_stride come in ra.  pdl: the first
+// launch's form (a window of several launches always starts with PDL_SETUP_FIRST, so that the later
+// ones find the records).
+int window_render(awg_t* h, Window* w, awgk::RenderArgs ra, int32_t pdl, cudaStream_t s) {
+  cudaError_t e;
+  const int64_t c = w->c, n = w->n;
+  int16_t* out_q = ra.out_q;
+  float* out_f = ra.out_f;
+  const float* base = ra.base;
+  ra.tones = h->d_tones;
+  ra.exact_tab = h->d_tab;
+  ra.chirps = h->d_chirps;
+  ra.recs = h->d_recs;
+  ra.act_of_slot = h->d_act;
+  ra.K = h->K;
+  ra.split = w->split;
+  ra.sine_mode = h->sine_mode;
+  ra.scale = h->full_scale > 0 ? (float)(32767.0 / h->full_scale) : 0.f;
+  ra.status = h->d_status;
+  std::memcpy(ra.inv_odd, h->inv_odd, sizeof(ra.inv_odd));
+  ra.rec_stride = (int32_t)w->active.size();
+  ra.end = h->d_times + 1;
+  for (int32_t t0 = 0, i = 0; t0 < w->n_tiles; t0 += w->per_launch, ++i) {
+    awgk::RenderArgs rs = ra;
+    const int32_t nt = std::min(w->per_launch, w->n_tiles - t0);
+    const int64_t w0 = std::max(c, (w->tile0 + t0) * (int64_t)awgk::TILE);
+    const int64_t w1 = std::min(c + n, (w->tile0 + t0 + nt) * (int64_t)awgk::TILE);
+    rs.tile0 = w->tile0 + t0;
+    rs.n_tiles = nt;
+    rs.rec_tile0 = t0;
+    rs.parts = render_parts(nt, w->split, h->sine_mode);
+    rs.win_start = w0;
+    rs.win_end = w1;
+    rs.out_q = out_q ? out_q + (size_t)(w0 - c) * (size_t)(ra.q_stride ? ra.q_stride : 1) : nullptr;
+    rs.out_f = out_f ? out_f + (w0 - c) : nullptr;
+    rs.base = base ? base + (w0 - c) : nullptr;
+    rs.start = w->first && w->active.empty() && i == 0 ? h->d_times : nullptr;
+    rs.pdl = w->n_tiles > w->per_launch ? (i == 0 ? awgk::PDL_SETUP_FIRST : awgk::PDL_FREE) : pdl;
+    if (w->split > 1) {
+      rs.part = split_part(h, i & 1);
+      rs.tile_ctr = split_ctr(h, i & 1);
+    }
+    if ((e = counted(h, awgk::launch_render(rs, s))) != cudaSuccess) return cuda_fail(e, "render launch");
+    ++w->launches;
+  }
+  if (w->pe[3]) {
+    if ((e = cudaEventRecord(w->pe[3], s)) != cudaSuccess) return cuda_fail(e, "event");
+    ++h->prof_calls;
+    h->prof_launches += w->launches;
+  }
+  if ((e = cudaEventRecord(h->ev_done, s)) != cudaSuccess) return cuda_fail(e, "event");
+  h->timed = true;
+  h->have_done = true;
+  h->cursor = c + n;
+  return AWG_OK;
+}
 
 int render_impl(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream, int32_t q_stride = 1) {
   if (h && h->static_engine != AWG_STATIC_DIRECT && n > 0 && (out_f || out_q) &&
@@ -1078,127 +1215,33 @@ int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
     }
     const int64_t c = h->cursor, n2 = n - n1;
     cudaError_t e;
-    if ((e = cudaEventRecord(h->ev0, s)) != cudaSuccess) return cuda_fail(e, "event");
     if ((e = counted(h, awgk::launch_replay(h->d_periodic, h->periodic_log2, c, n2, out_q + (size_t)n1 * (size_t)q_stride,
-                                 q_stride, s))) != cudaSuccess)
+                                 q_stride, h->d_times, s))) != cudaSuccess)
       return cuda_fail(e, "replay launch");
-    if ((e = cudaEventRecord(h->ev1, s)) != cudaSuccess) return cuda_fail(e, "event");
     if ((e = cudaEventRecord(h->ev_done, s)) != cudaSuccess) return cuda_fail(e, "event");
     h->timed = true;
     h->have_done = true;
     h->cursor = c + n2;
     return AWG_OK;
   }
-  const int64_t c = h->cursor;
-  const int64_t tile0 = c / awgk::TILE;
-  const int64_t tile_last = (c + n - 1) / awgk::TILE;
-  const int64_t n_tiles64 = tile_last - tile0 + 1;
-  if (n_tiles64 > (int64_t)(INT32_MAX / awgk::MAX_SPLIT)) return fail(AWG_EINVAL, "render window too long");
-  int64_t tile0_;
-  int32_t n_tiles;
-  const std::vector<int32_t> active = active_slots(h, c, n, &tile0_, &n_tiles);
-  int st = ensure(&h->d_recs, &h->cap_recs, std::max<size_t>(1, active.size() * (size_t)n_tiles), h, "tile records");
+  Window w;
+  w.split = tone_list ? list_split : h->split;
+  w.first = base == nullptr;   // with a base, the engine's kernels came before
+  int st = window_plan(h, n, &w);
+  if (!st) st = window_setup(h, &w, false, s);
   if (st) return st;
-  // With a split, the window goes out in launches of at most SPLIT_LAUNCH_TILES tiles, chained by
-  // programmatic dependent launch, on alternating scratch buffers.
-  const int32_t split_used = tone_list ? list_split : h->split;
-  const bool scratch = split_used > 1;
-  const int32_t per_launch = scratch ? std::min(n_tiles, SPLIT_LAUNCH_TILES) : n_tiles;
-  if (scratch && (st = ensure_split_scratch(h, per_launch, split_used))) return st;
-
-  // The chirp tile set-up runs in stream order right before the render.  (Running it on a second
-  // stream, overlapped with the previous render, takes SM slots from the render and pushes its
-  // grid into a second wave; measured slower.)
-  cudaError_t e;
-  cudaEvent_t pe[4] = {nullptr, nullptr, nullptr, nullptr};
-  if (h->profiling) {
-    while (h->prof_ev.size() < 4 * (h->prof_calls + 1)) {
-      cudaEvent_t ev;
-      if ((e = cudaEventCreate(&ev)) != cudaSuccess) return cuda_fail(e, "profiling event");
-      h->prof_ev.push_back(ev);
-    }
-    for (int i = 0; i < 4; ++i) pe[i] = h->prof_ev[4 * h->prof_calls + (size_t)i];
-  }
-  int64_t launches = 0;
-  if ((e = order_after_uploads(h, s)) != cudaSuccess) return cuda_fail(e, "upload ordering");
-  if ((e = cudaEventRecord(h->ev0, s)) != cudaSuccess) return cuda_fail(e, "event");
-  if (pe[0] && (e = cudaEventRecord(pe[0], s)) != cudaSuccess) return cuda_fail(e, "event");
-  for (size_t b = 0; b < active.size(); b += awgk::MAX_ACTIVE_PER_LAUNCH) {
-    awgk::PrepArgs pa;
-    std::memset(&pa, 0, sizeof(pa));
-    pa.chirps = h->d_chirps;
-    pa.tones = h->d_tones;
-    pa.recs = h->d_recs;
-    pa.act_of_slot = h->d_act;
-    pa.tile0 = tile0;
-    pa.n_tiles = n_tiles;
-    pa.n_active = (int32_t)std::min<size_t>(awgk::MAX_ACTIVE_PER_LAUNCH, active.size() - b);
-    pa.act_base = (int32_t)b;
-    pa.rec_stride = (int32_t)active.size();
-    std::memcpy(pa.W, h->W, sizeof(pa.W));
-    std::memcpy(pa.inv_odd, h->inv_odd, sizeof(pa.inv_odd));
-    for (int i = 0; i < pa.n_active; ++i) pa.slots[i] = active[b + (size_t)i];
-    if ((e = counted(h, awgk::launch_prep(pa, s))) != cudaSuccess) return cuda_fail(e, "prep launch");
-    ++launches;
-  }
-  if (pe[1] && (e = cudaEventRecord(pe[1], s)) != cudaSuccess) return cuda_fail(e, "event");
-  if (pe[2] && (e = cudaEventRecord(pe[2], s)) != cudaSuccess) return cuda_fail(e, "event");
   awgk::RenderArgs ra;
   std::memset(&ra, 0, sizeof(ra));
-  ra.tones = h->d_tones;
-  ra.exact_tab = h->d_tab;
-  ra.chirps = h->d_chirps;
-  ra.recs = h->d_recs;
-  ra.act_of_slot = h->d_act;
-  ra.K = h->K;
-  ra.split = h->split;
-  ra.sine_mode = h->sine_mode;
+  ra.out_q = out_q;
+  ra.out_f = out_f;
   ra.q_stride = q_stride;
   ra.base = base;
   ra.skip_static = skip_static;
   ra.tone_list = tone_list;
   ra.n_list = n_list;
-  if (tone_list) {
-    ra.split = list_split;
+  if (tone_list)
     for (int r = 0; r <= list_split; ++r) ra.bounds[r] = list_bounds[r];
-  }
-  ra.scale = h->full_scale > 0 ? (float)(32767.0 / h->full_scale) : 0.f;
-  ra.status = h->d_status;
-  std::memcpy(ra.inv_odd, h->inv_odd, sizeof(ra.inv_odd));
-  for (int32_t t0 = 0, i = 0; t0 < n_tiles; t0 += per_launch, ++i) {
-    awgk::RenderArgs rs = ra;
-    const int32_t nt = std::min(per_launch, n_tiles - t0);
-    const int64_t w0 = std::max(c, (tile0 + t0) * (int64_t)awgk::TILE);
-    const int64_t w1 = std::min(c + n, (tile0 + t0 + nt) * (int64_t)awgk::TILE);
-    rs.tile0 = tile0 + t0;
-    rs.n_tiles = nt;
-    rs.rec_stride = (int32_t)active.size();
-    rs.rec_tile0 = t0;
-    rs.parts = render_parts(nt, split_used, h->sine_mode);
-    rs.win_start = w0;
-    rs.win_end = w1;
-    rs.out_q = out_q ? out_q + (size_t)(w0 - c) * (size_t)(q_stride ? q_stride : 1) : nullptr;
-    rs.out_f = out_f ? out_f + (w0 - c) : nullptr;
-    rs.base = base ? base + (w0 - c) : nullptr;
-    if (scratch) {
-      rs.part = split_part(h, i & 1);
-      rs.tile_ctr = split_ctr(h, i & 1);
-      rs.pdl = n_tiles > per_launch ? (i == 0 ? 1 : 2) : 0;
-    }
-    if ((e = counted(h, awgk::launch_render(rs, s))) != cudaSuccess) return cuda_fail(e, "render launch");
-    ++launches;
-  }
-  if (pe[3]) {
-    if ((e = cudaEventRecord(pe[3], s)) != cudaSuccess) return cuda_fail(e, "event");
-    ++h->prof_calls;
-    h->prof_launches += launches;
-  }
-  if ((e = cudaEventRecord(h->ev1, s)) != cudaSuccess) return cuda_fail(e, "event");
-  if ((e = cudaEventRecord(h->ev_done, s)) != cudaSuccess) return cuda_fail(e, "event");
-  h->timed = true;
-  h->have_done = true;
-  h->cursor = c + n;
-  return AWG_OK;
+  return window_render(h, &w, ra, w.active.empty() ? awgk::PDL_FREE : awgk::PDL_AFTER_SETUP, s);
 }
 
 }  // namespace
@@ -1280,6 +1323,7 @@ awgk::TableArgs2 engine_gemm_args(awg_t* h, int64_t c, int64_t m, bool two_segme
   t.scale = h->full_scale > 0 ? (float)(32767.0 / h->full_scale) : 0.f;
   t.a_scale = awgk::table_amp_scale(max_amplitude(h));
   t.status = h->d_status;
+  t.times = h->d_times;
   return t;
 }
 
@@ -1315,12 +1359,10 @@ int render_engine(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
     if (!all_static && (st = ensure(&h->d_base, &h->cap_base, (size_t)m, h, "static sum"))) return st;
     cudaError_t e;
     if ((e = order_after_uploads(h, s)) != cudaSuccess) return cuda_fail(e, "upload ordering");
-    if ((e = cudaEventRecord(h->ev0, s)) != cudaSuccess) return cuda_fail(e, "event");
     if ((st = engine_operand(h, two_segments, s))) return st;
     const awgk::TableArgs2 t = engine_gemm_args(h, c, m, two_segments, all_static ? oq : nullptr, all_static ? of : h->d_base);
     if ((e = counted(h, awgk::launch_table_gemm(t, s))) != cudaSuccess) return cuda_fail(e, "static GEMM launch");
     if (all_static) {
-      if ((e = cudaEventRecord(h->ev1, s)) != cudaSuccess) return cuda_fail(e, "event");
       if ((e = cudaEventRecord(h->ev_done, s)) != cudaSuccess) return cuda_fail(e, "event");
       h->timed = true;
       h->have_done = true;
@@ -1446,19 +1488,9 @@ int awgk::prepare_render(awg_t* h, int64_t n, int16_t* out_q, float* out_f, cuda
   }
   for (size_t b = 0; b < active.size(); b += awgk::MAX_ACTIVE_PER_LAUNCH) {
     awgk::PrepArgs pa;
-    std::memset(&pa, 0, sizeof(pa));
-    pa.chirps = h->d_chirps;
-    pa.tones = h->d_tones;
+    prep_args(h, active, b, tile0, n_tiles, &pa);
     pa.recs = recs;
     pa.act_of_slot = act;
-    pa.tile0 = tile0;
-    pa.n_tiles = n_tiles;
-    pa.n_active = (int32_t)std::min<size_t>(awgk::MAX_ACTIVE_PER_LAUNCH, active.size() - b);
-    pa.act_base = (int32_t)b;
-    pa.rec_stride = (int32_t)active.size();
-    std::memcpy(pa.W, h->W, sizeof(pa.W));
-    std::memcpy(pa.inv_odd, h->inv_odd, sizeof(pa.inv_odd));
-    for (int i = 0; i < pa.n_active; ++i) pa.slots[i] = active[b + (size_t)i];
     cudaError_t e = counted(h, awgk::launch_prep(pa, s));
     if (e != cudaSuccess) return cuda_fail(e, "prep launch");
   }
@@ -1567,7 +1599,6 @@ int render_chunks_impl(awg_t* h, int64_t chunk, int32_t n_chunks, int16_t* out, 
   }
   const int64_t launches0 = h->n_launches;
   if ((e = order_after_uploads(h, s)) != cudaSuccess) return cuda_fail(e, "upload ordering");
-  if ((e = cudaEventRecord(h->ev0, s)) != cudaSuccess) return cuda_fail(e, "event");
   if (pe[0] && (e = cudaEventRecord(pe[0], s)) != cudaSuccess) return cuda_fail(e, "event");
   for (const Group& grp : groups) {
     const int32_t g0 = grp.g0, g1 = grp.g1;
@@ -1576,20 +1607,10 @@ int render_chunks_impl(awg_t* h, int64_t chunk, int32_t n_chunks, int16_t* out, 
     const std::vector<int32_t>& active = grp.active;
     for (size_t b = 0; b < active.size(); b += awgk::MAX_ACTIVE_PER_LAUNCH) {
       awgk::PrepArgs pa;
-      std::memset(&pa, 0, sizeof(pa));
-      pa.chirps = h->d_chirps;
-      pa.tones = h->d_tones;
+      prep_args(h, active, b, tile0, n_tiles, &pa);
       pa.recs = h->d_seq_recs;
       pa.act_of_slot = h->d_seq_act;
-      pa.tile0 = tile0;
-      pa.n_tiles = n_tiles;
-      pa.n_active = (int32_t)std::min<size_t>(awgk::MAX_ACTIVE_PER_LAUNCH, active.size() - b);
-      pa.act_base = (int32_t)b;
-      pa.rec_stride = (int32_t)active.size();
-    pa.rec_stride = (int32_t)active.size();
-      std::memcpy(pa.W, h->W, sizeof(pa.W));
-      std::memcpy(pa.inv_odd, h->inv_odd, sizeof(pa.inv_odd));
-      for (int i = 0; i < pa.n_active; ++i) pa.slots[i] = active[b + (size_t)i];
+      pa.start = g0 == 0 && b == 0 ? h->d_times : nullptr;
       if ((e = counted(h, awgk::launch_prep(pa, s))) != cudaSuccess) return cuda_fail(e, "prep launch");
     }
     if (pe[1] && g0 == 0) {
@@ -1624,7 +1645,9 @@ int render_chunks_impl(awg_t* h, int64_t chunk, int32_t n_chunks, int16_t* out, 
       ra.status = h->d_status;
       std::memcpy(ra.inv_odd, h->inv_odd, sizeof(ra.inv_odd));
       ra.parts = parts;
-      ra.pdl = c == g0 ? 1 : 2;
+      ra.pdl = c == g0 ? awgk::PDL_SETUP_FIRST : awgk::PDL_SEQUENCE;
+      ra.start = c == 0 && active.empty() ? h->d_times : nullptr;
+      ra.end = h->d_times + 1;
       ra.exit_ctr = h->d_seq_exit;
       if (h->split > 1) {   // alternating scratch (see tile_epilogue_split)
         ra.part = split_part(h, c & 1);
@@ -1642,7 +1665,6 @@ int render_chunks_impl(awg_t* h, int64_t chunk, int32_t n_chunks, int16_t* out, 
     ++h->prof_calls;
     h->prof_launches += h->n_launches - launches0;
   }
-  if ((e = cudaEventRecord(h->ev1, s)) != cudaSuccess) return cuda_fail(e, "event");
   if ((e = cudaEventRecord(h->ev_done, s)) != cudaSuccess) return cuda_fail(e, "event");
   h->timed = true;
   h->have_done = true;
@@ -1730,8 +1752,8 @@ awg_t* awg_create(double sample_rate_hz) {
   if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_status, sizeof(int32_t));
   if (e == cudaSuccess) e = cudaMemset(h->d_status, 0, sizeof(int32_t));
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->priv, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaEventCreate(&h->ev0);
-  if (e == cudaSuccess) e = cudaEventCreate(&h->ev1);
+  if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_times, 2 * sizeof(unsigned long long));
+  if (e == cudaSuccess) e = cudaMemset(h->d_times, 0, 2 * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_done, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_upload, cudaEventDisableTiming);
   if (e != cudaSuccess) {
@@ -1768,8 +1790,7 @@ void awg_destroy(awg_t* h) {
   cudaFree(h->d_tab);
   cudaFree(h->d_gemm);
   for (cudaEvent_t ev : h->prof_ev) cudaEventDestroy(ev);
-  if (h->ev0) cudaEventDestroy(h->ev0);
-  if (h->ev1) cudaEventDestroy(h->ev1);
+  cudaFree(h->d_times);
   if (h->ev_done) cudaEventDestroy(h->ev_done);
   if (h->ev_upload) cudaEventDestroy(h->ev_upload);
   if (h->priv) cudaStreamDestroy(h->priv);
@@ -2105,6 +2126,39 @@ int awg_render_multiplexed(awg_t* const* handles, int32_t n_channels, int64_t n,
     if (h->cursor > INT64_MAX - n) return fail(AWG_EINVAL, "sample index overflow");
     cursors[c] = h->cursor;
   }
+  // Direct channels: every channel's set-up first, then the renders; the first render waits for the
+  // set-ups before the next may start, so the renders of all channels run side by side (each writes
+  // only after the one before has completed).
+  bool together = n_channels > 1;
+  for (int32_t c = 0; c < n_channels; ++c) {
+    const awg_t* h = handles[c];
+    together = together && h->static_engine == AWG_STATIC_DIRECT && !h->profiling &&
+               !(h->periodic_start >= 0 && h->cursor + n > h->periodic_start);
+  }
+  if (together) {
+    cudaStream_t s = (cudaStream_t)stream;
+    Window w[8];
+    int st = AWG_OK;
+    for (int32_t c = 0; c < n_channels && !st; ++c) {
+      w[c].split = handles[c]->split;
+      w[c].first = true;
+      st = window_plan(handles[c], n, &w[c]);
+    }
+    int32_t last_setup = 0;   // the last channel with a set-up kernel
+    for (int32_t c = 0; c < n_channels && !st; ++c)
+      if (!w[c].active.empty()) last_setup = c;
+    for (int32_t c = 0; c < n_channels && !st; ++c) st = window_setup(handles[c], &w[c], c < last_setup, s);
+    for (int32_t c = 0; c < n_channels && !st; ++c) {
+      awgk::RenderArgs ra;
+      std::memset(&ra, 0, sizeof(ra));
+      ra.out_q = out + c;
+      ra.q_stride = n_channels;
+      st = window_render(handles[c], &w[c], ra, c == 0 ? awgk::PDL_SETUP_FIRST : awgk::PDL_FREE, s);
+    }
+    if (st)
+      for (int32_t c = 0; c < n_channels; ++c) handles[c]->cursor = cursors[c];
+    return st;
+  }
   for (int32_t c = 0; c < n_channels; ++c) {
     const int st = render_impl(handles[c], n, nullptr, out + c, stream, n_channels);
     if (st) {
@@ -2244,9 +2298,15 @@ int32_t awg_tone_split(const awg_t* h) { return h ? h->split : 0; }
 
 float awg_last_render_ms(awg_t* h) {
   if (!h || !h->timed) return -1.f;
-  float ms = -1.f;
-  if (cudaEventElapsedTime(&ms, h->ev0, h->ev1) != cudaSuccess) return -1.f;
-  return ms;
+  if (cudaEventQuery(h->ev_done) != cudaSuccess) {
+    cudaGetLastError();
+    return -1.f;
+  }
+  unsigned long long t[2];
+  cudaError_t e = cudaMemcpyAsync(t, h->d_times, sizeof(t), cudaMemcpyDeviceToHost, h->priv);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->priv);
+  if (e != cudaSuccess || t[1] < t[0]) return -1.f;
+  return (float)((double)(t[1] - t[0]) * 1e-6);
 }
 
 int awg_table_gemm(awg_t* h, int32_t log2_len, int32_t precision, int16_t* out_q, float* out_f, void* stream) {
@@ -2283,6 +2343,7 @@ int awg_table_gemm(awg_t* h, int32_t log2_len, int32_t precision, int16_t* out_q
   t.scale = h->full_scale > 0 ? (float)(32767.0 / h->full_scale) : 0.f;
   t.a_scale = awgk::table_amp_scale(max_amplitude(h));
   t.status = h->d_status;
+  t.times = h->d_times;
   cudaStream_t s = (cudaStream_t)stream;
   cudaEvent_t pe[4] = {nullptr, nullptr, nullptr, nullptr};
   cudaError_t e = cudaSuccess;
@@ -2295,7 +2356,6 @@ int awg_table_gemm(awg_t* h, int32_t log2_len, int32_t precision, int16_t* out_q
     for (int i = 0; i < 4 && e == cudaSuccess; ++i) pe[i] = h->prof_ev[4 * h->prof_calls + (size_t)i];
   }
   if (e == cudaSuccess) e = order_after_uploads(h, s);
-  if (e == cudaSuccess) e = cudaEventRecord(h->ev0, s);
   if (e == cudaSuccess && pe[0]) e = cudaEventRecord(pe[0], s);
   if (e == cudaSuccess) e = counted(h, awgk::launch_table_prep(t, s));
   if (e == cudaSuccess && pe[1]) e = cudaEventRecord(pe[1], s);
@@ -2306,7 +2366,6 @@ int awg_table_gemm(awg_t* h, int32_t log2_len, int32_t precision, int16_t* out_q
     ++h->prof_calls;
     h->prof_launches += 3;
   }
-  if (e == cudaSuccess) e = cudaEventRecord(h->ev1, s);
   if (e == cudaSuccess) e = cudaEventRecord(h->ev_done, s);
   if (e != cudaSuccess) return cuda_fail(e, "table GEMM");
   h->timed = true;
@@ -2348,7 +2407,6 @@ int awg_render_noalloc(awg_t* h, int64_t n, int16_t* out, void* stream) {
                                 " chirp tile records; the fixed scratch holds " +
                                 std::to_string(awgk::NOALLOC_MAX_RECORDS) + " (AWG_NOALLOC_MAX_RECORDS)");
   if ((e = order_after_uploads(h, s)) != cudaSuccess) return cuda_fail(e, "upload ordering");
-  if ((e = cudaEventRecord(h->ev0, s)) != cudaSuccess) return cuda_fail(e, "event");
   awgk::PrepArgs pa;
   std::memset(&pa, 0, sizeof(pa));
   pa.chirps = h->d_chirps;
@@ -2366,6 +2424,7 @@ int awg_render_noalloc(awg_t* h, int64_t n, int16_t* out, void* stream) {
     pa.slots[pa.n_active++] = t.slot;
     if (pa.n_active == awgk::MAX_ACTIVE_PER_LAUNCH) {
       pa.act_base = batch_base;
+      pa.start = batch_base == 0 ? h->d_times : nullptr;
       if ((e = counted(h, awgk::launch_prep(pa, s))) != cudaSuccess) return cuda_fail(e, "prep launch");
       batch_base += pa.n_active;
       pa.n_active = 0;
@@ -2373,6 +2432,7 @@ int awg_render_noalloc(awg_t* h, int64_t n, int16_t* out, void* stream) {
   }
   if (pa.n_active > 0) {
     pa.act_base = batch_base;
+    pa.start = batch_base == 0 ? h->d_times : nullptr;
     if ((e = counted(h, awgk::launch_prep(pa, s))) != cudaSuccess) return cuda_fail(e, "prep launch");
   }
   awgk::RenderArgs ra;
@@ -2389,6 +2449,8 @@ int awg_render_noalloc(awg_t* h, int64_t n, int16_t* out, void* stream) {
   ra.n_tiles = (int32_t)n_tiles;
   ra.rec_stride = (int32_t)n_active;
   ra.cluster = 1;
+  ra.start = n_active == 0 ? h->d_times : nullptr;
+  ra.end = h->d_times + 1;
   ra.win_start = c;
   ra.win_end = c + n;
   ra.out_q = out;
@@ -2397,7 +2459,6 @@ int awg_render_noalloc(awg_t* h, int64_t n, int16_t* out, void* stream) {
   ra.status = h->d_status;
   std::memcpy(ra.inv_odd, h->inv_odd, sizeof(ra.inv_odd));
   if ((e = counted(h, awgk::launch_render(ra, s))) != cudaSuccess) return cuda_fail(e, "render launch");
-  if ((e = cudaEventRecord(h->ev1, s)) != cudaSuccess) return cuda_fail(e, "event");
   if ((e = cudaEventRecord(h->ev_done, s)) != cudaSuccess) return cuda_fail(e, "event");
   h->timed = true;
   h->have_done = true;

@@ -139,6 +139,8 @@ struct PrepArgsT {
   int32_t n_active;
   int32_t act_base;       // active index of slots[0]
   int32_t rec_stride;     // records per tile (active chirps of the window)
+  unsigned long long* start;   // device time of the call's start goes here (its first kernel; null: not first)
+  int32_t more;           // 1: the next kernel of the call is another set-up, which may start at once
   uint32_t W[7][7];       // W[q][i] = Delta^q_j C(j RUN, i) at j = 0 (all below 2^32)
   uint64_t inv_odd[3][3]; // inverses mod 2^192 of 3, 15, 45
   int32_t slots[CAP];
@@ -169,12 +171,18 @@ struct RenderArgs {
   // is recs[(rec_tile0 + t) * rec_stride + a]
   int32_t rec_stride;
   int32_t rec_tile0;
-  // pipelined chunk sequences (otherwise 0 / null): pdl 1 waits for the preceding kernel (the
-  // records' set-up) and then lets the next kernel launch early; pdl 2 lets it launch early and
-  // reads nothing the preceding kernel writes (with split scratch, it waits for that kernel before
-  // reusing the scratch); each CTA adds 1 to *exit_ctr once its samples are stored
+  // Programmatic dependent launch (0: plain launch): the kernel may start while the preceding one of
+  // the stream still runs.  PDL_AFTER_SETUP: the preceding kernel wrote the records, the kernels
+  // behind it may start at once; it waits for that kernel before it reads a record.  PDL_SETUP_FIRST:
+  // it waits for it before anything, and only then lets later kernels start, so that they need not
+  // wait for the records.  PDL_FREE: reads nothing that the preceding kernel writes.  These wait for
+  // the preceding kernel before their first write to global memory, so a kernel completes only after
+  // all before it in the stream.  PDL_SEQUENCE (chunk sequences, closed by a join kernel): as PDL_FREE,
+  // but it waits only before it reuses split scratch; each CTA adds 1 to *exit_ctr once its samples
+  // are stored.
   int32_t pdl;
   unsigned long long* exit_ctr;
+  unsigned long long *start, *end;   // device time of the call's start (first kernel) and end (every CTA)
   // tensor-core static engine (otherwise null / 0): tones static over the window are skipped here
   // (their sum comes from the table GEMM) and base[n - win_start] is added before quantising
   const float* base;
@@ -193,6 +201,8 @@ struct RenderArgs {
   float* part;
   unsigned long long* tile_ctr;
 };
+
+enum { PDL_NONE = 0, PDL_SETUP_FIRST = 1, PDL_SEQUENCE = 2, PDL_AFTER_SETUP = 3, PDL_FREE = 4 };
 
 struct PhaseArgs {
   const ToneRec* tones;
@@ -230,7 +240,7 @@ cudaError_t launch_prep(const PrepArgs& a, cudaStream_t s);
 cudaError_t launch_exact_table(const TableArgs& a, int64_t L, cudaStream_t s);
 cudaError_t launch_render(const RenderArgs& a, cudaStream_t s);
 cudaError_t launch_replay(const int16_t* tab, int32_t log2_len, int64_t c, int64_t n, int16_t* out, int32_t stride,
-                          cudaStream_t s);
+                          unsigned long long* times, cudaStream_t s);   // times: start, end
 // A bounded wait on the device (join of a pipelined sequence): at most limit_ns of wall time, then
 // the status word becomes AWG_ETIMEOUT and the kernel returns.
 constexpr uint64_t JOIN_LIMIT_NS = 2000000000ull;
@@ -281,6 +291,7 @@ struct TableArgs2 {
   // the epilogue
   float a_scale;
   int32_t* status;
+  unsigned long long* times;   // device time of the call's start and end (null: not taken)
 };
 // a_scale for amplitudes whose largest magnitude is amax (1 for amax 0)
 float table_amp_scale(double amax);

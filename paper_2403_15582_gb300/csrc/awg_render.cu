@@ -601,6 +601,18 @@ __device__ __forceinline__ void prep_exp(const ChirpRec& c, int64_t m, const Arg
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Device times of a handle's last render (awg_last_render_ms): the first kernel of a call writes the
+// start, every CTA raises the end once its samples are stored (time only grows, so the largest is
+// the last render's).  Events in the stream would serve too, but a timed event between two kernels
+// keeps the second from starting before the first has ended: 6.6 us between kernels with the
+// events, 2.3 without, none with the kernels overlapping.
+__device__ __forceinline__ void mark_start(unsigned long long* t) {
+  if (t && blockIdx.x == 0 && threadIdx.x == 0) *t = global_ns();
+}
+__device__ __forceinline__ void mark_end(unsigned long long* t) {
+  if (t && threadIdx.x == 0) atomicMax(t, (unsigned long long)global_ns());
+}
+
 // Bounded wait (limit_ns of wall time) until a device counter reaches target; false on timeout.
 __device__ bool wait_counter(const unsigned long long* ctr, unsigned long long target, uint64_t limit_ns) {
   const volatile unsigned long long* v = ctr;
@@ -633,6 +645,10 @@ __device__ __forceinline__ void store_record(TileRec* out, const TileRec& r) {
 
 template <class Args>
 __global__ void __launch_bounds__(128, 5) prep_kernel(const __grid_constant__ Args a) {
+  mark_start(a.start);
+  // A render behind this kernel starts when it is complete: one that started earlier would put its
+  // CTAs on the SMs that happen to have room, not evenly (1000-chirp 2^18 chunk: 109 against 96 us)
+  if (a.more) pdl_launch_dependents();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t total = (int64_t)a.n_active * a.n_tiles;
   if (idx >= total) return;
@@ -640,23 +656,28 @@ __global__ void __launch_bounds__(128, 5) prep_kernel(const __grid_constant__ Ar
   const int t = (int)(idx - (int64_t)ai * a.n_tiles);
   const int slot = a.slots[ai];
   const ChirpRec& c = a.chirps[slot];
-  if (t == 0) a.act_of_slot[slot] = a.act_base + ai;
   const int64_t T0 = (a.tile0 + t) * (int64_t)TILE;
   const int words = rec_words(c, a.tones[c.tone], T0);
   TileRec* out = a.recs + (int64_t)t * a.rec_stride + a.act_base + ai;
   TileRec r;
+  // the preceding kernel of the stream may be a render that reads the buffers written here: it has
+  // to be complete before the first write, not before the arithmetic
   if (words == REC_WORDS_LINEAR) {
     prep_one<2, REC_WORDS_LINEAR>(c, T0 - c.n_s, a, r);
+    pdl_wait();
     store_record<REC_WORDS_LINEAR>(out, r);
   } else if (words == REC_WORDS_LOW3) {
     if (c.flags & TONE_EXP) prep_exp<REC_WORDS_LOW3>(c, T0 - c.n_s, a, r);
     else prep_one<6, REC_WORDS_LOW3>(c, T0 - c.n_s, a, r);
+    pdl_wait();
     store_record<REC_WORDS_LOW3>(out, r);
   } else {
     if (c.flags & TONE_EXP) prep_exp<REC_WORDS>(c, T0 - c.n_s, a, r);
     else prep_one<6, REC_WORDS>(c, T0 - c.n_s, a, r);
+    pdl_wait();
     store_record<REC_WORDS>(out, r);
   }
+  if (t == 0) a.act_of_slot[slot] = a.act_base + ai;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1058,8 +1079,8 @@ __device__ __forceinline__ void store_group(const RenderArgs& a, int64_t n, cons
 // sums) and stores the part, thread t taking the 8-sample groups t, t + RT, ... (coalesced
 // 16-byte stores).  The loads of several ranks are in flight at a time: one rank at a time left
 // the last CTA of a tile waiting for the L2 `split` times in a row (12 us at split 11).
-// In a pipelined sequence (pdl 2) the scratch of this launch was used two launches back: waiting
-// for the preceding launch to complete (which waited for the one before) makes it free.
+// The preceding kernel of the stream is complete before the first write to global memory (in a
+// sequence: before the first write to the split scratch).
 template <int SPT>
 __device__ __forceinline__ void tile_epilogue_split(const RenderArgs& a, int unit, int crank, int split, int64_t P0,
                                                     int at, const Acc<SPT>& acc) {
@@ -1067,6 +1088,7 @@ __device__ __forceinline__ void tile_epilogue_split(const RenderArgs& a, int uni
   const int tid = threadIdx.x;
   __shared__ int s_last;
   const bool vec = q_vec_ok(a) && f_vec_ok(a);
+  if (a.pdl != PDL_NONE && (a.pdl != PDL_SEQUENCE || split > 1)) pdl_wait();
   if (split == 1) {
 #pragma unroll
     for (int g = 0; g < SPT / 8; ++g) {
@@ -1079,7 +1101,6 @@ __device__ __forceinline__ void tile_epilogue_split(const RenderArgs& a, int uni
       store_group(a, P0 + at + 8 * g, xv, vec);
     }
   } else {
-    if (a.pdl == 2) pdl_wait();
     float4* dst = reinterpret_cast<float4*>(a.part + ((int64_t)unit * split + crank) * PSAMP + at);
 #pragma unroll
     for (int j = 0; j < SPT / 4; ++j)
@@ -1137,6 +1158,7 @@ __device__ __forceinline__ void tile_epilogue_split(const RenderArgs& a, int uni
     __syncthreads();
     if (tid == 0) atomicAdd(a.exit_ctr, 1ull);
   }
+  mark_end(a.end);
 }
 
 // One CTA's share of one part of a tile: tones [K crank / split, K (crank+1) / split) of window tile
@@ -1195,10 +1217,10 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
 #pragma unroll
   for (int r = 0; r < SPT / 2; ++r) acc[r] = make_float2(0.f, 0.f);
 
-  if (a.pdl == 1) {   // pipelined sequence: the records' set-up (the preceding kernel) is complete
-    pdl_wait();         // before the next render may start (it relies on the same set-up)
+  if (a.pdl == PDL_SETUP_FIRST) {   // the records' set-up (the preceding kernel) is complete before
+    pdl_wait();                      // the next render may start (it relies on the same set-up)
     pdl_launch_dependents();
-  } else if (a.pdl == 2) {
+  } else if (a.pdl != PDL_NONE) {
     pdl_launch_dependents();
   }
   if (tid == 0) {
@@ -1299,6 +1321,7 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
     if (tid < 32) {
       issue_tones(0);
       if (n_stages > 1) issue_tones(1);
+      if (a.pdl == PDL_AFTER_SETUP) pdl_wait();   // the records' set-up is complete
       ok &= mbar_wait(&s_bar[0], 0);
       prepare_stage(0);
     }
@@ -1498,6 +1521,7 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
       const int sidx = s_first + u;
       if (u < per && sidx < hi) store_sample(a, T0 + sidx, xs[u]);
     }
+    mark_end(a.end);
   }
 }
 
@@ -1508,6 +1532,7 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
 #define AWG_RENDER_SPLIT_MIN_BLOCKS 6
 #define AWG_RENDER_PART_MIN_BLOCKS 8
 __global__ void __launch_bounds__(RT, AWG_RENDER_MIN_BLOCKS) render_kernel(const __grid_constant__ RenderArgs a) {
+  mark_start(a.start);
   cg::cluster_group cluster = cg::this_cluster();
   render_tile<RUN, true>(a, blockIdx.x / a.split, (int)cluster.block_rank(), a.split);
 }
@@ -1516,6 +1541,7 @@ __global__ void __launch_bounds__(RT, AWG_RENDER_MIN_BLOCKS) render_kernel(const
 template <int SPT>
 __global__ void __launch_bounds__(RT, SPT == RUN ? AWG_RENDER_SPLIT_MIN_BLOCKS : AWG_RENDER_PART_MIN_BLOCKS)
     render_split_kernel(const __grid_constant__ RenderArgs a) {
+  mark_start(a.start);
   render_tile<SPT, false>(a, blockIdx.x / a.split, blockIdx.x % a.split, a.split);
 }
 
@@ -1655,10 +1681,26 @@ cudaError_t launch_render_batch_split(const RenderArgs* reqs, const int2* items,
   return cudaGetLastError();
 }
 
+// A launch configuration with programmatic stream serialisation: the kernel may start before the
+// preceding one of the stream has completed (it then waits where it has to, pdl_wait).
+struct PdlLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  PdlLaunch(unsigned grid, unsigned block, cudaStream_t s) {
+    cfg.gridDim = dim3(grid, 1, 1);
+    cfg.blockDim = dim3(block, 1, 1);
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+  }
+};
+
 cudaError_t launch_prep(const PrepArgs& a, cudaStream_t s) {
   const int64_t total = (int64_t)a.n_active * a.n_tiles;
   if (total == 0) return cudaSuccess;
-  const int blocks = (int)((total + 127) / 128);
+  const PdlLaunch l((unsigned)((total + 127) / 128), 128, s);
   if (a.n_active <= SMALL_PREP) {   // the small parameter form: fewer bytes copied with the launch
     PrepArgsT<SMALL_PREP> b;
     b.chirps = a.chirps;
@@ -1670,23 +1712,25 @@ cudaError_t launch_prep(const PrepArgs& a, cudaStream_t s) {
     b.n_active = a.n_active;
     b.act_base = a.act_base;
     b.rec_stride = a.rec_stride;
+    b.start = a.start;
+    b.more = a.more;
     for (int q = 0; q < 7; ++q)
       for (int i = 0; i < 7; ++i) b.W[q][i] = a.W[q][i];
     for (int q = 0; q < 3; ++q)
       for (int i = 0; i < 3; ++i) b.inv_odd[q][i] = a.inv_odd[q][i];
     for (int i = 0; i < a.n_active; ++i) b.slots[i] = a.slots[i];
-    prep_kernel<PrepArgsT<SMALL_PREP>><<<blocks, 128, 0, s>>>(b);
-  } else {
-    prep_kernel<PrepArgs><<<blocks, 128, 0, s>>>(a);
+    return cudaLaunchKernelEx(&l.cfg, prep_kernel<PrepArgsT<SMALL_PREP>>, b);
   }
-  return cudaGetLastError();
+  return cudaLaunchKernelEx(&l.cfg, prep_kernel<PrepArgs>, a);
 }
 
 // Replay of a periodic record (period mask + 1 = 2^log2 samples): out[i * stride] =
 // table[(c + i) mod period].  16-byte vectors when the stride is 1 and both sides are aligned
 // to 8 samples (a vector never wraps: the period is a multiple of 8).
 __global__ void replay_kernel(const int16_t* __restrict__ tab, uint64_t mask, int64_t c, int64_t n,
-                              int16_t* __restrict__ out, int32_t stride, int vec) {
+                              int16_t* __restrict__ out, int32_t stride, int vec, unsigned long long* times) {
+  mark_start(times);
+  pdl_wait();
   const int64_t step = (int64_t)gridDim.x * blockDim.x;
   const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int64_t done = 0;
@@ -1709,17 +1753,18 @@ __global__ void replay_kernel(const int16_t* __restrict__ tab, uint64_t mask, in
     done = nv * 8;
   }
   for (int64_t i = done + t0; i < n; i += step) out[i * stride] = tab[((uint64_t)c + (uint64_t)i) & mask];
+  mark_end(times + 1);
 }
 
 cudaError_t launch_replay(const int16_t* tab, int32_t log2_len, int64_t c, int64_t n, int16_t* out, int32_t stride,
-                          cudaStream_t s) {
+                          unsigned long long* times, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const uint64_t mask = ((uint64_t)1 << log2_len) - 1;
   const int vec = stride == 1 && (c & 7) == 0 && ((uintptr_t)out & 15) == 0 && log2_len >= 3;
   const int64_t work = vec ? n / 8 + 1 : n;
   const int64_t blocks = std::min<int64_t>((work + 255) / 256, (int64_t)device_sm_count() * 16);
-  replay_kernel<<<(unsigned)std::max<int64_t>(blocks, 1), 256, 0, s>>>(tab, mask, c, n, out, stride, vec);
-  return cudaGetLastError();
+  const PdlLaunch l((unsigned)std::max<int64_t>(blocks, 1), 256, s);
+  return cudaLaunchKernelEx(&l.cfg, replay_kernel, tab, mask, c, n, out, stride, vec, times);
 }
 
 // End of a pipelined sequence: returns once every render CTA of the sequence has stored its

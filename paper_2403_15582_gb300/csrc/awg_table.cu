@@ -134,6 +134,7 @@ struct TableGemmArgs {
   int64_t win_start, win_end;
   int32_t window_mode;
   float a_scale, inv_a_scale;   // A operand scaling (a power of two) and its inverse
+  unsigned long long* end;      // device time of the call's end (null: not taken)
 };
 
 template <typename T>
@@ -444,6 +445,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     if (a.out_f) a.out_f[n - a.win_start] = x;
   }
   cluster.sync();   // remote reads done before any CTA of the cluster exits
+  if (a.end && threadIdx.x == 0) atomicMax(a.end, (unsigned long long)now_ns());
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -485,7 +487,9 @@ __device__ __forceinline__ void split_store(T* hi, T* lo, int64_t i, float v) {
 
 // Bt[n2][2k] = cos b_k(n2), Bt[n2][2k+1] = sin b_k(n2) (the B operand stored K-major).
 template <typename T>
-__global__ void prep_b_kernel(const ToneRec* tones, int K, int64_t Kp, T* hi, T* lo, int window_mode) {
+__global__ void prep_b_kernel(const ToneRec* tones, int K, int64_t Kp, T* hi, T* lo, int window_mode,
+                              unsigned long long* start) {
+  if (start && blockIdx.x == 0 && threadIdx.x == 0) *start = now_ns();
   const int64_t pairs = Kp / 2;
   const int64_t total = (int64_t)TN * pairs;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
@@ -536,9 +540,10 @@ cudaError_t launch_table_prep(const TableArgs2& t, cudaStream_t s) {
   const int blocks = device_sm_count() * 4;
   if (t.precision == 0)
     prep_b_kernel<__nv_bfloat16><<<blocks, threads, 0, s>>>(t.tones, t.K, Kp, (__nv_bfloat16*)t.b_hi,
-                                                           (__nv_bfloat16*)t.b_lo, t.window_mode);
+                                                           (__nv_bfloat16*)t.b_lo, t.window_mode, t.times);
   else
-    prep_b_kernel<__half><<<blocks, threads, 0, s>>>(t.tones, t.K, Kp, (__half*)t.b_hi, (__half*)t.b_lo, t.window_mode);
+    prep_b_kernel<__half><<<blocks, threads, 0, s>>>(t.tones, t.K, Kp, (__half*)t.b_hi, (__half*)t.b_lo, t.window_mode,
+                                                    t.times);
   return cudaGetLastError();
 }
 
@@ -575,6 +580,7 @@ cudaError_t launch_table_gemm(const TableArgs2& t, cudaStream_t s) {
   ga.window_mode = t.window_mode;
   ga.a_scale = t.a_scale > 0.f ? t.a_scale : 1.f;
   ga.inv_a_scale = 1.f / ga.a_scale;
+  ga.end = t.times ? t.times + 1 : nullptr;
   // instruction descriptor: FP32 accumulate, A/B BF16 (1) or FP16 (0), both K-major, N/8, M/16
   const uint32_t fmt = bf16 ? 1u : 0u;
   ga.idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
