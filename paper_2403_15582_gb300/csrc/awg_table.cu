@@ -161,86 +161,121 @@ __device__ __forceinline__ float2 unpack2<__half>(uint32_t u) {
   return __half22float2(v);
 }
 
-// The A tile of one stage for one generator warp: lane j takes tone kt0 + j (its phase word,
-// frequency word and amplitude, loaded once), warp g the rows g, g + 4, ..., g + 124; for each row
-// n1 it forms the hi and lo halves of (A_k sin a, A_k cos a), a = 2 pi (Phi0_k + n1 NB F_k) / 2^64,
-// stepping the exact phase word by 4 NB F_k from row to row.  The pair is one 32-bit word at byte
-// 4 (j mod 4) of 16-byte chunk j / 4 of the row, which the 128-byte swizzle moves to chunk
-// (j / 4) ^ (row mod 8).  The sine and cosine take the top 32 bits of the phase word as a signed
-// turn on the SFU (|error| < 5e-7).
-template <typename T, bool WINDOW>
-__device__ __forceinline__ void gen_a_tile(const TableGemmArgs& a, int kt0, uint32_t row0, int g, int lane,
-                                           uint32_t tile_hi, uint32_t tile_lo) {
-  // table mode: lane j = tone kt0 + j (one (sin, cos) pair per tone); static engine: lane j = tone
-  // kt0 / 2 + j / 2, segment j % 2 (two pairs per tone), zero in tiles where it is not static
-  const int k = WINDOW ? (kt0 >> 1) + (lane >> 1) : kt0 + lane;
-  const int seg = lane & 1;
-  uint64_t w = 0, step = 0;
-  float amp = 0.f;
-  // static engine: the tiles [T0, T0 + TILE) where this (tone, segment) is static are those with
-  // seg_lo <= T0 <= seg_hi outside (ramp_lo, ramp_hi); amplitude A before the ramp, A_end after
-  int64_t seg_lo = 0, seg_hi = -1, ramp_lo = INT64_MAX, ramp_hi = INT64_MIN;
-  float amp_end = 0.f;
-  if (k < a.K) {
-    uint64_t phi, F;
-    float A;
-    if (WINDOW) {
-      const ToneRec& t = a.tones[k];
-      phi = seg ? t.phi_post_ref : t.phi_ref;
-      F = seg ? t.F_end : t.F;
-      A = t.A;
-      amp_end = t.A;
-      if (seg == 0) {
-        seg_lo = INT64_MIN;
-        seg_hi = t.slot >= 0 ? t.n_s - TILE : INT64_MAX;      // T0 + TILE - 1 < n_s
-      } else if (t.slot >= 0) {
-        seg_lo = t.n_e + 1;                                   // T0 > n_e
-        seg_hi = INT64_MAX;
-      }
-      if (t.flags & TONE_AMP_RAMP) {                          // not static: T0 + TILE - 1 > a_ns and T0 < a_ns + a_L
-        ramp_lo = t.a_ns - TILE + 2;
-        ramp_hi = t.a_ns + t.a_L - 1;
-        amp_end = t.A_end;
-      }
-    } else {
-      const ToneRec* t = a.tones + k;
-      phi = __ldg(&t->phi_ref);
-      F = __ldg(&t->F);
-      A = __ldg(&t->A);
+// The static engine's A tile of one stage: 16 tones, four columns each (sine and cosine for the
+// segment before the tone's chirp, the same for the one after it), 128 rows.  A segment's columns are
+// zero in the 4096-sample tiles where the tone is not static in it (tile_segment_static), so every
+// (row, tone) holds at most one live segment: one sine and cosine per (row, tone), and one 8-byte
+// store per half, a row of 128 bytes per half warp.  Warp g takes the rows 16 g .. 16 g + 15, lane l
+// tone l mod 16 and every second row.  (Before, each segment had a lane of its own with 64-bit tile
+// compares per row, and the tone records were read after the wait for the stage: 270 us for 10,000
+// tones x 2^20; now 177, of which the MMAs take about 155 at the rate of the table.)
+//
+// The rows of a tone where a segment is live, as rows of this CTA's tile (clamped to 0 .. TM): segment
+// 0 in rows < pre, segment 1 in rows >= post, neither in the rows ramp_lo .. ramp_hi - 1 of an
+// amplitude ramp; the amplitude is amp before the ramp, amp_end from ramp_hi on.
+struct WindowTone {
+  uint64_t phi0, F0, phi1, F1;
+  int32_t pre, post, ramp_lo, ramp_hi;
+  float amp, amp_end;
+};
+// first row of the tile ceil or floor of which the caller has formed, relative to the CTA's rows
+__device__ __forceinline__ int32_t clamp_row(int64_t tile, int64_t R0) {
+  return (int32_t)max((int64_t)0, min((int64_t)TM, tile * (TILE / TN) - R0));
+}
+__device__ __forceinline__ WindowTone window_tone(const ToneRec* t, float a_scale, int64_t R0) {
+  WindowTone w;
+  w.phi0 = w.F0 = w.phi1 = w.F1 = 0;
+  w.pre = TM;
+  w.post = TM;
+  w.ramp_lo = w.ramp_hi = TM;
+  w.amp = w.amp_end = 0.f;
+  if (t) {
+    const int32_t flags = t->flags;
+    w.phi0 = t->phi_ref;
+    w.F0 = t->F;
+    w.amp = t->A * a_scale;
+    w.amp_end = w.amp;
+    if (t->slot >= 0) {
+      w.phi1 = t->phi_post_ref;
+      w.F1 = t->F_end;
+      w.pre = clamp_row(t->n_s / TILE, R0);           // T0 + TILE - 1 < n_s
+      w.post = clamp_row(t->n_e / TILE + 1, R0);      // T0 > n_e
     }
-    const uint64_t f8 = F << a.nb_log2;
-    w = phi + (uint64_t)(a.row_base + (int64_t)row0 + g) * f8;
-    step = f8 * (uint64_t)NGEN;
-    amp = A * a.a_scale;
-    amp_end *= a.a_scale;
+    if (flags & TONE_AMP_RAMP) {                      // T0 + TILE - 1 > a_ns and T0 < a_ns + a_L
+      w.ramp_lo = clamp_row((t->a_ns + 1) / TILE, R0);
+      w.ramp_hi = clamp_row((t->a_ns + t->a_L + TILE - 1) / TILE, R0);
+      w.amp_end = t->A_end * a_scale;
+    }
   }
-  const uint32_t col = (uint32_t)(lane & 3) * 4u;
-  const uint32_t chunk = (uint32_t)(lane >> 2);
-#pragma unroll 8
-  for (int i = 0; i < TM / NGEN; ++i) {
-    const uint32_t r = (uint32_t)(g + NGEN * i);
-    float sn, cs;
-    __sincosf((float)(int32_t)(w >> 32) * 1.46291807926715968e-9f, &sn, &cs);   // 2 pi / 2^32
-    float a_row = amp;
-    if (WINDOW) {   // the row's tile decides whether this segment is summed here
-      const int64_t T0 = ((a.row_base + (int64_t)row0 + (int64_t)r) << a.nb_log2) & ~(int64_t)(TILE - 1);
-      const bool in_seg = T0 >= seg_lo && T0 <= seg_hi;
-      const bool ramping = T0 >= ramp_lo && T0 <= ramp_hi;
-      a_row = (in_seg && !ramping) ? (T0 > ramp_hi ? amp_end : amp) : 0.f;
-    }
-    const float sv = a_row * sn, cv = a_row * cs;
-    const uint32_t hv = pack2<T>(sv, cv);
-    const float2 h = unpack2<T>(hv);
-    const uint32_t lv = pack2<T>(sv - h.x, cv - h.y);
+  return w;
+}
+
+// (a sin, a cos) of phase word w as packed hi and lo halves.  The sine and cosine take the top 32
+// bits of the phase word as a signed turn on the SFU (|error| < 5e-7).
+template <typename T>
+__device__ __forceinline__ void sincos_halves(uint64_t w, float a, uint32_t* hv, uint32_t* lv) {
+  float sn, cs;
+  __sincosf((float)(int32_t)(w >> 32) * 1.46291807926715968e-9f, &sn, &cs);   // 2 pi / 2^32
+  const float sv = a * sn, cv = a * cs;
+  *hv = pack2<T>(sv, cv);
+  const float2 h = unpack2<T>(*hv);
+  *lv = pack2<T>(sv - h.x, cv - h.y);
+}
+
+template <typename T>
+__device__ __forceinline__ void gen_a_window(const TableGemmArgs& a, const WindowTone& t, int64_t R0, int g, int lane,
+                                             uint32_t tile_hi, uint32_t tile_lo) {
+  constexpr int ROWS = TM / NGEN;   // rows of a warp
+  static_assert(ROWS == 16 && TK / 4 == 16, "a half warp holds the stage's tones");
+  const uint32_t r_first = (uint32_t)(ROWS * g + (lane >> 4));
+  const uint32_t chunk = (uint32_t)((lane & 15) >> 1), col = (uint32_t)(lane & 1) * 8u;
+  const uint64_t f0 = t.F0 << a.nb_log2;
+  uint64_t w0 = t.phi0 + (uint64_t)(R0 + r_first) * f0;
+  // one live segment and one amplitude in all rows of the tile (a tone whose chirp and ramp lie
+  // elsewhere), or none: segment and amplitude are chosen once
+  const bool ramp_out = t.ramp_lo >= TM || t.ramp_hi <= 0;
+  const bool plain = ramp_out && (t.pre >= TM || t.post <= 0 || (t.pre <= 0 && t.post >= TM));
+  auto store = [&](uint32_t r, uint32_t h0, uint32_t h1, uint32_t l0, uint32_t l1) {
     const uint32_t off = r * 128u + ((chunk ^ (r & 7u)) << 4) + col;
-    asm volatile("st.shared.b32 [%0], %1;" ::"r"(tile_hi + off), "r"(hv) : "memory");
-    asm volatile("st.shared.b32 [%0], %1;" ::"r"(tile_lo + off), "r"(lv) : "memory");
-    w += step;
+    asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(tile_hi + off), "r"(h0), "r"(h1) : "memory");
+    asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(tile_lo + off), "r"(l0), "r"(l1) : "memory");
+  };
+  if (__all_sync(0xffffffffu, plain)) {
+    const bool second = t.post <= 0, live = second || t.pre >= TM;
+    const uint64_t f = second ? t.F1 << a.nb_log2 : f0;
+    uint64_t w = second ? t.phi1 + (uint64_t)(R0 + r_first) * f : w0;
+    const uint64_t step = 2 * f;
+    const float amp = live ? (t.ramp_hi <= 0 ? t.amp_end : t.amp) : 0.f;
+#pragma unroll
+    for (int i = 0; i < ROWS / 2; ++i) {
+      uint32_t hv, lv;
+      sincos_halves<T>(w, amp, &hv, &lv);
+      store(r_first + 2 * i, second ? 0u : hv, second ? hv : 0u, second ? 0u : lv, second ? lv : 0u);
+      w += step;
+    }
+    return;
+  }
+  const uint64_t f1 = t.F1 << a.nb_log2;
+  uint64_t w1 = t.phi1 + (uint64_t)(R0 + r_first) * f1;
+#pragma unroll 2
+  for (int i = 0; i < ROWS / 2; ++i) {
+    const int r = (int)r_first + 2 * i;
+    const bool second = r >= t.post;
+    const bool live = (second || r < t.pre) && !(r >= t.ramp_lo && r < t.ramp_hi);
+    uint32_t hv, lv;
+    sincos_halves<T>(second ? w1 : w0, live ? (r >= t.ramp_hi ? t.amp_end : t.amp) : 0.f, &hv, &lv);
+    store((uint32_t)r, second ? 0u : hv, second ? hv : 0u, second ? 0u : lv, second ? lv : 0u);
+    w0 += 2 * f0;
+    w1 += 2 * f1;
   }
 }
 
-// Table mode with the lane's tone words already loaded (phi, F, A; zero amplitude past K): the
-// same rows as gen_a_tile<T, false>.
+// Table mode: the A tile of one stage for one generator warp.  Lane j holds tone kt0 + j (its phase
+// word, frequency word and scaled amplitude, loaded before; zero amplitude past K), warp g the rows g,
+// g + NGEN, ...; for each row n1 it forms the hi and lo halves of (A_k sin a, A_k cos a), a = 2 pi
+// (Phi0_k + n1 NB F_k) / 2^64, stepping the exact phase word by NGEN NB F_k from row to row.  The
+// pair is one 32-bit word at byte 4 (j mod 4) of 16-byte chunk j / 4 of the row, which the 128-byte
+// swizzle moves to chunk (j / 4) ^ (row mod 8).
 template <typename T>
 __device__ __forceinline__ void gen_a_rows(const TableGemmArgs& a, uint64_t phi, uint64_t F, float A, uint32_t row0,
                                            int g, int lane, uint32_t tile_hi, uint32_t tile_lo) {
@@ -252,12 +287,8 @@ __device__ __forceinline__ void gen_a_rows(const TableGemmArgs& a, uint64_t phi,
 #pragma unroll 8
   for (int i = 0; i < TM / NGEN; ++i) {
     const uint32_t r = (uint32_t)(g + NGEN * i);
-    float sn, cs;
-    __sincosf((float)(int32_t)(w >> 32) * 1.46291807926715968e-9f, &sn, &cs);   // 2 pi / 2^32
-    const float sv = A * sn, cv = A * cs;
-    const uint32_t hv = pack2<T>(sv, cv);
-    const float2 h = unpack2<T>(hv);
-    const uint32_t lv = pack2<T>(sv - h.x, cv - h.y);
+    uint32_t hv, lv;
+    sincos_halves<T>(w, A, &hv, &lv);
     const uint32_t off = r * 128u + ((chunk ^ (r & 7u)) << 4) + col;
     asm volatile("st.shared.b32 [%0], %1;" ::"r"(tile_hi + off), "r"(hv) : "memory");
     asm volatile("st.shared.b32 [%0], %1;" ::"r"(tile_lo + off), "r"(lv) : "memory");
@@ -354,14 +385,19 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
   } else if (warp >= 2) {
     // ---------------- A operand generation ----------------
     {
-      const int g = warp - 2;   // rows g, g + NGEN, ...
+      const int g = warp - 2;
+      const int64_t R0 = a.row_base + row0;   // absolute row of the CTA's first row
       for (int kb = 0; kb < n_kb; ++kb) {
         const int s = kb % NSTAGE;
-        // table mode: this k-block's tone words are loaded before the wait for the stage, so
-        // their latency hides under it
+        // this k-block's tone words are loaded before the wait for the stage, so their latency hides
+        // under it
         uint64_t phi = 0, F = 0;
         float A = 0.f;
-        if (!WINDOW) {
+        WindowTone wt;
+        if (WINDOW) {
+          const int k = (kb0 + kb) * (TK / 4) + (lane & 15);
+          wt = window_tone(k < a.K ? a.tones + k : nullptr, a.a_scale, R0);
+        } else {
           const int k = (kb0 + kb) * (TK / 2) + lane;
           if (k < a.K) {
             phi = __ldg(&a.tones[k].phi_ref);
@@ -375,7 +411,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         }
         if (s_fail) break;
         const uint32_t st = base + (uint32_t)s * STAGE_BYTES;
-        if (WINDOW) gen_a_tile<T, true>(a, (kb0 + kb) * (TK / 2), (uint32_t)row0, g, lane, st, st + A_TILE);
+        if (WINDOW) gen_a_window<T>(a, wt, R0, g, lane, st, st + A_TILE);
         else gen_a_rows<T>(a, phi, F, A, (uint32_t)row0, g, lane, st, st + A_TILE);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor cores
         __syncwarp();
@@ -465,44 +501,52 @@ __device__ __forceinline__ void sincos_word(uint64_t w, float* s, float* c) {
   *c = fmaf(-s1, d, c1);
 }
 
+// (c, s) as packed hi and lo halves
 template <typename T>
-__device__ __forceinline__ T to_half(float v);
-template <>
-__device__ __forceinline__ __nv_bfloat16 to_half<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
-template <>
-__device__ __forceinline__ __half to_half<__half>(float v) { return __float2half_rn(v); }
-template <typename T>
-__device__ __forceinline__ float from_half(T v);
-template <>
-__device__ __forceinline__ float from_half<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }
-template <>
-__device__ __forceinline__ float from_half<__half>(__half v) { return __half2float(v); }
-
-template <typename T>
-__device__ __forceinline__ void split_store(T* hi, T* lo, int64_t i, float v) {
-  const T h = to_half<T>(v);
-  hi[i] = h;
-  lo[i] = to_half<T>(v - from_half<T>(h));
+__device__ __forceinline__ void split_pair(float c, float s, uint32_t* hi, uint32_t* lo) {
+  *hi = pack2<T>(c, s);
+  const float2 h = unpack2<T>(*hi);
+  *lo = pack2<T>(c - h.x, s - h.y);
 }
 
-// Bt[n2][2k] = cos b_k(n2), Bt[n2][2k+1] = sin b_k(n2) (the B operand stored K-major).
-template <typename T>
-__global__ void prep_b_kernel(const ToneRec* tones, int K, int64_t Kp, T* hi, T* lo, int window_mode,
-                              unsigned long long* start) {
-  if (start && blockIdx.x == 0 && threadIdx.x == 0) *start = now_ns();
-  const int64_t pairs = Kp / 2;
-  const int64_t total = (int64_t)TN * pairs;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t n2 = i / pairs, k = i - n2 * pairs;
+// Bt[n2][2k] = cos b_k(n2), Bt[n2][2k+1] = sin b_k(n2) (the B operand stored K-major); static engine:
+// four columns per tone, its two segments' frequency words.  A thread holds one tone and PREP_ROWS
+// rows n2, stepping the phase word by the frequency word; a warp stores 32 neighbouring tones (128
+// or 256 bytes).  10,000 tones: 15.3 -> 8.7 us (two columns), 26.7 -> 13.5 us (four), from a 64-bit
+// division and four 2-byte stores per element.  A tone without a chirp has no second segment (its A columns are zero).
+constexpr int PREP_ROWS = 16;
+template <typename T, bool WINDOW>
+__global__ void __launch_bounds__(128) prep_b_kernel(const ToneRec* tones, int K, int64_t Kp, uint32_t* hi, uint32_t* lo,
+                                                     unsigned long long* start) {
+  if (start && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *start = now_ns();
+  constexpr int PAIRS = WINDOW ? 2 : 1;   // column pairs per tone
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= Kp / (2 * PAIRS)) return;
+  const bool in = k < K, second = WINDOW && in && tones[k].slot >= 0;
+  const uint64_t F0 = in ? tones[k].F : 0, F1 = second ? tones[k].F_end : 0;
+  const int n0 = (int)blockIdx.y * PREP_ROWS;
+  uint64_t w0 = (uint64_t)n0 * F0, w1 = (uint64_t)n0 * F1;
+  for (int n2 = n0; n2 < n0 + PREP_ROWS; ++n2) {
     float s = 0.f, c = 0.f;
-    // static engine: pair k = (tone k / 2, segment k % 2), the segment's frequency word
-    const int64_t tone = window_mode ? k >> 1 : k;
-    if (tone < K) {
-      const uint64_t F = (window_mode && (k & 1)) ? tones[tone].F_end : tones[tone].F;
-      sincos_word((uint64_t)n2 * F, &s, &c);
+    uint32_t h[2] = {0, 0}, l[2] = {0, 0};
+    if (in) {
+      sincos_word(w0, &s, &c);
+      split_pair<T>(c, s, &h[0], &l[0]);
     }
-    split_store<T>(hi, lo, n2 * Kp + 2 * k, c);
-    split_store<T>(hi, lo, n2 * Kp + 2 * k + 1, s);
+    if (second) {
+      sincos_word(w1, &s, &c);
+      split_pair<T>(c, s, &h[1], &l[1]);
+    }
+    const int64_t at = (int64_t)n2 * (Kp / 2) + PAIRS * k;
+    if (WINDOW) {
+      *reinterpret_cast<uint2*>(hi + at) = make_uint2(h[0], h[1]);
+      *reinterpret_cast<uint2*>(lo + at) = make_uint2(l[0], l[1]);
+    } else {
+      hi[at] = h[0];
+      lo[at] = l[0];
+    }
+    w0 += F0;
+    w1 += F1;
   }
 }
 
@@ -536,14 +580,11 @@ size_t table_kp_window(int K) { return (((size_t)4 * K + TK - 1) / TK) * TK; }
 
 cudaError_t launch_table_prep(const TableArgs2& t, cudaStream_t s) {
   const int64_t Kp = (int64_t)(t.window_mode ? table_kp_window(t.K) : table_kp(t.K));
-  const int threads = 256;
-  const int blocks = device_sm_count() * 4;
-  if (t.precision == 0)
-    prep_b_kernel<__nv_bfloat16><<<blocks, threads, 0, s>>>(t.tones, t.K, Kp, (__nv_bfloat16*)t.b_hi,
-                                                           (__nv_bfloat16*)t.b_lo, t.window_mode, t.times);
-  else
-    prep_b_kernel<__half><<<blocks, threads, 0, s>>>(t.tones, t.K, Kp, (__half*)t.b_hi, (__half*)t.b_lo, t.window_mode,
-                                                    t.times);
+  const int64_t per_row = Kp / (t.window_mode ? 4 : 2);
+  const dim3 grid((unsigned)((per_row + 127) / 128), TN / PREP_ROWS);
+  auto kern = t.window_mode ? (t.precision == 0 ? prep_b_kernel<__nv_bfloat16, true> : prep_b_kernel<__half, true>)
+                            : (t.precision == 0 ? prep_b_kernel<__nv_bfloat16, false> : prep_b_kernel<__half, false>);
+  kern<<<grid, 128, 0, s>>>(t.tones, t.K, Kp, (uint32_t*)t.b_hi, (uint32_t*)t.b_lo, t.times);
   return cudaGetLastError();
 }
 
