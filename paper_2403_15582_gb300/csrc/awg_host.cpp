@@ -575,16 +575,18 @@ struct awg {
   int split = 1;
   int32_t sine_mode = AWG_SINE_SFU;
   int32_t static_engine = AWG_STATIC_DIRECT;
-  float* d_base = nullptr;             // tensor-core engine: FP32 sum of the window's static tones
-  size_t cap_base = 0;
+  float* d_base = nullptr;             // tensor-core engine: FP32 sum of the window's static tones, then
+  size_t cap_base = 0;                 // that of its other tones, rendered on `side` beside the GEMM
+  cudaStream_t side = nullptr;         // created on first use, with its events
+  cudaEvent_t ev_fork = nullptr, ev_operand = nullptr, ev_join = nullptr;
   // split sums without clusters: two scratch buffers (alternating between consecutive launches)
   // of part_tiles x part_split partial tiles each, and a 64-bit counter per tile per buffer
   float* d_part = nullptr;
   unsigned long long* d_tctr = nullptr;
   int32_t part_tiles = 0, part_split = 0, ctr_split = 0;
   int64_t n_launches = 0;              // kernels this handle has launched
-  int32_t* d_list = nullptr;           // tensor-core engine: tones not static in some tile of the window
-  size_t cap_list = 0;
+  int32_t* d_list = nullptr;           // tensor-core engine: tones not static in some tile of the window,
+  size_t cap_list = 0;                 // then the same sifted per tile (RenderArgs::tile_first, the rows)
   std::vector<int32_t> list;
   // tones that hold a chirp or an amplitude ramp, ascending (the static engine's render part);
   // rebuilt on demand after tones, chirps or ramps change
@@ -1068,9 +1070,16 @@ int32_t render_parts(int64_t tiles, int32_t split, int32_t sine_mode) {
 }
 
 int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream, int32_t q_stride,
-                  const float* base, int32_t skip_static, const int32_t* tone_list = nullptr, int32_t n_list = 0,
-                  int32_t list_split = 0, const int32_t* list_bounds = nullptr);
+                  bool engine_part, const int32_t* tone_list = nullptr, int32_t n_list = 0, int32_t list_split = 0,
+                  const int32_t* list_bounds = nullptr);
 int render_engine(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream, int32_t q_stride);
+
+constexpr size_t SIFT_BUDGET = (size_t)1 << 24;   // entries of the sifted lists (64 MiB); longer ones go unsifted
+// Entries of the list buffer of a window of n_tiles tiles: the list, its sifted rows and their rank bounds.
+size_t list_entries(int32_t n_list, int64_t n_tiles, int32_t split) {
+  const size_t rows = (size_t)n_tiles * (size_t)n_list;
+  return std::max<size_t>(1, (size_t)n_list) + (rows <= SIFT_BUDGET ? rows + (size_t)n_tiles * (size_t)(split + 1) : 0);
+}
 
 // One direct render of the window [cursor, cursor + n): the plan (buffers made large enough), the
 // chirp tile set-up and the render launches.  Every launch may start while the kernel before it in
@@ -1133,15 +1142,14 @@ int window_setup(awg_t* h, Window* w, bool more, cudaStream_t s) {
   return AWG_OK;
 }
 
-// The render launches; out_q, out_f, base, the tone list and q_stride come in ra.  pdl: the first
-// launch's form (a window of several launches always starts with PDL_SETUP_FIRST, so that the later
-// ones find the records).
+// The render launches; out_q, out_f, the tone list and q_stride come in ra.  pdl: the first
+// launch's form (with programmatic launch, a window of several launches starts with PDL_SETUP_FIRST,
+// so that the later ones find the records).
 int window_render(awg_t* h, Window* w, awgk::RenderArgs ra, int32_t pdl, cudaStream_t s) {
   cudaError_t e;
   const int64_t c = w->c, n = w->n;
   int16_t* out_q = ra.out_q;
   float* out_f = ra.out_f;
-  const float* base = ra.base;
   ra.tones = h->d_tones;
   ra.exact_tab = h->d_tab;
   ra.chirps = h->d_chirps;
@@ -1168,9 +1176,8 @@ int window_render(awg_t* h, Window* w, awgk::RenderArgs ra, int32_t pdl, cudaStr
     rs.win_end = w1;
     rs.out_q = out_q ? out_q + (size_t)(w0 - c) * (size_t)(ra.q_stride ? ra.q_stride : 1) : nullptr;
     rs.out_f = out_f ? out_f + (w0 - c) : nullptr;
-    rs.base = base ? base + (w0 - c) : nullptr;
     rs.start = w->first && w->active.empty() && i == 0 ? h->d_times : nullptr;
-    rs.pdl = w->n_tiles > w->per_launch ? (i == 0 ? awgk::PDL_SETUP_FIRST : awgk::PDL_FREE) : pdl;
+    rs.pdl = pdl == awgk::PDL_NONE || w->n_tiles <= w->per_launch ? pdl : (i == 0 ? awgk::PDL_SETUP_FIRST : awgk::PDL_FREE);
     if (w->split > 1) {
       rs.part = split_part(h, i & 1);
       rs.tile_ctr = split_ctr(h, i & 1);
@@ -1194,12 +1201,12 @@ int render_impl(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream,
   if (h && h->static_engine != AWG_STATIC_DIRECT && n > 0 && (out_f || out_q) &&
       !(h->periodic_start >= 0 && !out_f && h->cursor + n > h->periodic_start))
     return render_engine(h, n, out_f, out_q, stream, q_stride);
-  return render_direct(h, n, out_f, out_q, stream, q_stride, nullptr, 0);
+  return render_direct(h, n, out_f, out_q, stream, q_stride, false);
 }
 
 int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream, int32_t q_stride,
-                  const float* base, int32_t skip_static, const int32_t* tone_list, int32_t n_list,
-                  int32_t list_split, const int32_t* list_bounds) {
+                  bool engine_part, const int32_t* tone_list, int32_t n_list, int32_t list_split,
+                  const int32_t* list_bounds) {
   if (!h) return fail(AWG_EINVAL, "null handle");
   if (n < 0) return fail(AWG_EINVAL, "sample count must be >= 0");
   if (n == 0) return AWG_OK;
@@ -1226,7 +1233,7 @@ int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
   }
   Window w;
   w.split = tone_list ? list_split : h->split;
-  w.first = base == nullptr;   // with a base, the engine's kernels came before
+  w.first = !engine_part;   // the engine's kernels came before
   int st = window_plan(h, n, &w);
   if (!st) st = window_setup(h, &w, false, s);
   if (st) return st;
@@ -1235,13 +1242,38 @@ int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
   ra.out_q = out_q;
   ra.out_f = out_f;
   ra.q_stride = q_stride;
-  ra.base = base;
-  ra.skip_static = skip_static;
+  ra.skip_static = engine_part;   // the tones that are static in a tile go through the GEMM
   ra.tone_list = tone_list;
   ra.n_list = n_list;
-  if (tone_list)
+  if (tone_list) {
     for (int r = 0; r <= list_split; ++r) ra.bounds[r] = list_bounds[r];
-  return window_render(h, &w, ra, w.active.empty() ? awgk::PDL_FREE : awgk::PDL_AFTER_SETUP, s);
+    // the list sifted per tile, where the rows take a reasonable buffer (behind the list itself)
+    const size_t rows = (size_t)w.n_tiles * (size_t)n_list;
+    if (n_list > 0 && rows <= SIFT_BUDGET) {
+      awgk::SiftArgs sa;
+      std::memset(&sa, 0, sizeof(sa));
+      sa.tones = h->d_tones;
+      sa.list = tone_list;
+      sa.n_list = n_list;
+      sa.split = list_split;
+      sa.n_tiles = w.n_tiles;
+      sa.tile0 = w.tile0;
+      std::memcpy(sa.bounds, ra.bounds, sizeof(sa.bounds));
+      sa.rows = h->d_list + n_list;
+      sa.first = sa.rows + rows;
+      const cudaError_t e = counted(h, awgk::launch_sift(sa, s));
+      if (e != cudaSuccess) return cuda_fail(e, "list launch");
+      ++w.launches;
+      ra.tone_list = sa.rows;
+      ra.tile_first = sa.first;
+    }
+  }
+  if (engine_part) {
+    const cudaError_t e = cudaStreamWaitEvent(s, h->ev_operand, 0);
+    if (e != cudaSuccess) return cuda_fail(e, "engine ordering");
+  }
+  // with a sifted list the render reads what the kernel right before it wrote
+  return window_render(h, &w, ra, ra.tile_first ? awgk::PDL_NONE : w.active.empty() ? awgk::PDL_FREE : awgk::PDL_AFTER_SETUP, s);
 }
 
 }  // namespace
@@ -1338,6 +1370,17 @@ int engine_operand(awg_t* h, bool two_segments, cudaStream_t s) {
   return AWG_OK;
 }
 
+int ensure_side_stream(awg_t* h) {
+  if (h->ev_join) return AWG_OK;
+  cudaError_t e = cudaSuccess;
+  if (!h->side) e = cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking);
+  if (e == cudaSuccess && !h->ev_fork) e = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming);
+  if (e == cudaSuccess && !h->ev_operand) e = cudaEventCreateWithFlags(&h->ev_operand, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming);
+  if (e != cudaSuccess) return cuda_fail(e, "engine stream");
+  return AWG_OK;
+}
+
 int render_engine(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream, int32_t q_stride) {
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t PIECE = (int64_t)1 << 26;
@@ -1353,13 +1396,25 @@ int render_engine(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
     float* of = out_f ? out_f + off : nullptr;
     int st;
     if (h->K == 0) {
-      if ((st = render_direct(h, m, of, oq, stream, q_stride, nullptr, 0))) return st;
+      if ((st = render_direct(h, m, of, oq, stream, q_stride, false))) return st;
       continue;
     }
-    if (!all_static && (st = ensure(&h->d_base, &h->cap_base, (size_t)m, h, "static sum"))) return st;
+    // (a list of all K tones is left out: one bulk copy per stage instead of one per tone)
+    const int32_t n_list = (int32_t)h->list.size();
+    const bool use_list = n_list < h->K;
+    const size_t live_at = ((size_t)m + 3) & ~(size_t)3;
+    if (!all_static) {
+      if ((st = ensure(&h->d_base, &h->cap_base, live_at + (size_t)m, h, "engine sums"))) return st;
+      const int64_t n_tiles = (c + m - 1) / awgk::TILE - c / awgk::TILE + 1;
+      if (use_list && (st = ensure(&h->d_list, &h->cap_list, list_entries(n_list, n_tiles, es.split), h, "tone list"))) return st;
+      if ((st = ensure_side_stream(h))) return st;
+    }
+    float* d_live = h->d_base + live_at;
     cudaError_t e;
     if ((e = order_after_uploads(h, s)) != cudaSuccess) return cuda_fail(e, "upload ordering");
+    if (!all_static && (e = cudaEventRecord(h->ev_fork, s)) != cudaSuccess) return cuda_fail(e, "event");
     if ((st = engine_operand(h, two_segments, s))) return st;
+    if (!all_static && (e = cudaEventRecord(h->ev_operand, s)) != cudaSuccess) return cuda_fail(e, "event");
     const awgk::TableArgs2 t = engine_gemm_args(h, c, m, two_segments, all_static ? oq : nullptr, all_static ? of : h->d_base);
     if ((e = counted(h, awgk::launch_table_gemm(t, s))) != cudaSuccess) return cuda_fail(e, "static GEMM launch");
     if (all_static) {
@@ -1369,19 +1424,25 @@ int render_engine(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
       h->cursor = c + m;
       continue;
     }
-    // (a list of all K tones is left out: one bulk copy per stage instead of one per tone)
-    const int32_t n_list = (int32_t)h->list.size();
-    const bool use_list = n_list < h->K;
-    if (use_list) {
-      if ((st = ensure(&h->d_list, &h->cap_list, std::max<size_t>(1, (size_t)n_list), h, "tone list"))) return st;
-      if (n_list > 0 &&
-          (e = cudaMemcpyAsync(h->d_list, h->list.data(), (size_t)n_list * sizeof(int32_t), cudaMemcpyHostToDevice,
-                               s)) != cudaSuccess)
-        return cuda_fail(e, "tone list upload");
-    }
-    if ((st = render_direct(h, m, of, oq, stream, q_stride, h->d_base, 1, use_list ? h->d_list : nullptr, n_list,
-                            es.split, es.bounds)))
-      return st;
+    // The tones that chirp or ramp, on the side stream beside the GEMM: a GEMM CTA leaves its SM room
+    // for a render CTA, and a window's GEMM often leaves SMs idle (128 CTAs for 2^20 samples on 152).
+    // The set-up runs beside the operand's; the render starts once the operand is made, so that the
+    // GEMM's CTAs (one per SM, nearly all of its shared memory) are placed first.  10,000 tones x
+    // 2^20, 400 of them chirping in turn: 300 us one after the other, 214 us side by side.
+    if ((e = cudaStreamWaitEvent(h->side, h->ev_fork, 0)) != cudaSuccess) return cuda_fail(e, "engine ordering");
+    if (use_list && n_list > 0 &&
+        (e = cudaMemcpyAsync(h->d_list, h->list.data(), (size_t)n_list * sizeof(int32_t), cudaMemcpyHostToDevice,
+                             h->side)) != cudaSuccess)
+      return cuda_fail(e, "tone list upload");
+    st = render_direct(h, m, d_live, nullptr, h->side, 1, true, use_list ? h->d_list : nullptr, n_list, es.split, es.bounds);
+    // whatever was queued on the side stream is joined, so that later calls come after it
+    e = cudaEventRecord(h->ev_join, h->side);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, h->ev_join, 0);
+    if (e == cudaSuccess && !st)
+      e = counted(h, awgk::launch_combine(d_live, h->d_base, m, t.scale, oq, q_stride, of, h->d_times + 1, s));
+    if (e == cudaSuccess) e = cudaEventRecord(h->ev_done, s);
+    if (e != cudaSuccess) return cuda_fail(e, "engine sum");
+    if (st) return st;
   }
   return AWG_OK;
 }
@@ -1772,6 +1833,7 @@ void awg_destroy(awg_t* h) {
   if (!h) return;
   if (h->have_done) cudaEventSynchronize(h->ev_done);
   if (h->priv) cudaStreamSynchronize(h->priv);
+  if (h->side) cudaStreamSynchronize(h->side);
   cudaFree(h->d_tones);
   cudaFree(h->d_chirps);
   cudaFree(h->d_act);
@@ -1793,6 +1855,10 @@ void awg_destroy(awg_t* h) {
   cudaFree(h->d_times);
   if (h->ev_done) cudaEventDestroy(h->ev_done);
   if (h->ev_upload) cudaEventDestroy(h->ev_upload);
+  if (h->ev_fork) cudaEventDestroy(h->ev_fork);
+  if (h->ev_operand) cudaEventDestroy(h->ev_operand);
+  if (h->ev_join) cudaEventDestroy(h->ev_join);
+  if (h->side) cudaStreamDestroy(h->side);
   if (h->priv) cudaStreamDestroy(h->priv);
   if (h->stage) cudaFreeHost(h->stage);
   delete h;

@@ -193,6 +193,10 @@ struct RenderArgs {
   const int32_t* tone_list;
   int32_t n_list;
   int32_t bounds[MAX_SPLIT + 1];
+  // sifted lists (null: none): row rec_tile0 + tile of tone_list (n_list entries) holds the listed
+  // tones that are not static in that tile, in order; rank r takes entries first[r] .. first[r + 1] of
+  // row rec_tile0 + tile of tile_first (split + 1 entries)
+  const int32_t* tile_first;
   int32_t cluster;        // 1: render_kernel, the split sums through a cluster's shared memory
   int32_t parts;          // CTAs that share a tile's samples: 1, 2 or 4 (render_split_kernel)
   // split sums without clusters: partial sums part[((tile parts + p) split + rank) (TILE / parts) +
@@ -238,9 +242,24 @@ struct TableArgs {      // exact per-sample 32-bit phases of one short chirp, m 
 
 cudaError_t launch_prep(const PrepArgs& a, cudaStream_t s);
 cudaError_t launch_exact_table(const TableArgs& a, int64_t L, cudaStream_t s);
+// Sifts the listed tones for tiles tile0 .. tile0 + n_tiles - 1 (RenderArgs::tile_first).
+struct SiftArgs {
+  const ToneRec* tones;
+  const int32_t* list;    // ascending, n_list entries
+  int32_t n_list, split, n_tiles;
+  int64_t tile0;
+  int32_t bounds[MAX_SPLIT + 1];
+  int32_t* rows;          // [n_tiles][n_list]
+  int32_t* first;         // [n_tiles][split + 1]
+};
+cudaError_t launch_sift(const SiftArgs& a, cudaStream_t s);
 cudaError_t launch_render(const RenderArgs& a, cudaStream_t s);
 cudaError_t launch_replay(const int16_t* tab, int32_t log2_len, int64_t c, int64_t n, int16_t* out, int32_t stride,
                           unsigned long long* times, cudaStream_t s);   // times: start, end
+// x[i] = part[i] + base[i], i < n (in the order the render adds its engine sum): FP32 to out_f,
+// scaled, rounded and clamped codes to out_q[i * q_stride] (either may be null).
+cudaError_t launch_combine(const float* part, const float* base, int64_t n, float scale, int16_t* out_q, int32_t q_stride,
+                           float* out_f, unsigned long long* end, cudaStream_t s);
 // A bounded wait on the device (join of a pipelined sequence): at most limit_ns of wall time, then
 // the status word becomes AWG_ETIMEOUT and the kernel returns.
 constexpr uint64_t JOIN_LIMIT_NS = 2000000000ull;

@@ -1197,13 +1197,19 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
   // positions [l_begin, l_end) of the visit: the CTA's range of tones, or of the tone list
   int l_begin = (int)((int64_t)a.K * crank / split);
   int l_end = (int)((int64_t)a.K * (crank + 1) / split);
-  if (a.tone_list) {
+  const int32_t* list = a.tone_list;
+  if (a.tile_first) {
+    const int32_t* first = a.tile_first + (int64_t)(a.rec_tile0 + tile) * (split + 1);
+    list += (int64_t)(a.rec_tile0 + tile) * a.n_list;
+    l_begin = first[crank];
+    l_end = first[crank + 1];
+  } else if (list) {
     const int k_begin = a.bounds[crank], k_end = a.bounds[crank + 1];
     auto lower = [&](int key) {
       int lo = 0, hi = a.n_list;
       while (lo < hi) {
         const int mid = (lo + hi) >> 1;
-        if (a.tone_list[mid] < key) lo = mid + 1;
+        if (list[mid] < key) lo = mid + 1;
         else hi = mid;
       }
       return lo;
@@ -1242,15 +1248,15 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
       issued += 1u << (8 * (st & 1));
     }
     __syncwarp();
-    if (!a.tone_list) {
+    if (!list) {
       if (tid == 0) bulk_g2s(&s_tone[st & 1][0], a.tones + lb, (uint32_t)cnt * (uint32_t)sizeof(ToneRec), &s_bar[st & 1]);
     } else if (tid < cnt) {
-      bulk_g2s(&s_tone[st & 1][tid], a.tones + a.tone_list[lb + tid], (uint32_t)sizeof(ToneRec), &s_bar[st & 1]);
+      bulk_g2s(&s_tone[st & 1][tid], a.tones + list[lb + tid], (uint32_t)sizeof(ToneRec), &s_bar[st & 1]);
     }
   };
   // warp 0, once the stage's tones have landed: descriptors, visit order, and the records of tones
   // that chirp inside this tile: the window's active chirps are numbered in tone order, so the
-  // stage's records lie one after another and come in one bulk copy
+  // records of a stage's consecutive tones lie one after another and come in one bulk copy
   auto prepare_stage = [&](int st) {
     const int b = st & 1;
     const int cnt = min(STAGE, l_end - (l_begin + st * STAGE));
@@ -1287,7 +1293,7 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
     // FP32 sums then depends on which tones share a stage; with a tone list (the window's listed
     // tones) that changes with the window, so listed renders keep plain tone order, and every window
     // cut gives the same bits.  Skipped tones are left out.
-    const int grp = kind == DESC_SKIP ? -1 : visit_group(kind, a.tone_list != nullptr, pairable);
+    const int grp = kind == DESC_SKIP ? -1 : visit_group(kind, list != nullptr, pairable);
     const unsigned below = (1u << tid) - 1u;
     int pos = 0, end = 0;
 #pragma unroll
@@ -1304,15 +1310,19 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
     const unsigned mask = __ballot_sync(0xffffffffu, need);
     const int first = __shfl_sync(0xffffffffu, act, mask ? __ffs(mask) - 1 : 0);
     const int last = __shfl_sync(0xffffffffu, act, mask ? 31 - __clz(mask) : 0);
-    if (need) s_desc[b][tid].rec = act - first;
+    // (the tones left out of a sifted list leave gaps: then one copy per record)
+    const bool dense = (unsigned)(last - first) < (unsigned)STAGE;
+    if (need) s_desc[b][tid].rec = dense ? act - first : tid;
+    const TileRec* recs = a.recs + (int64_t)(a.rec_tile0 + tile) * a.rec_stride;
     if (tid == 0) {
-      const uint32_t bytes = mask ? (uint32_t)(last - first + 1) * (uint32_t)sizeof(TileRec) : 0u;
+      const uint32_t n_rec = !mask ? 0u : dense ? (uint32_t)(last - first + 1) : (uint32_t)__popc(mask);
       fence_proxy_async();
-      mbar_arrive_expect_tx(&s_bar[2 + b], bytes);
+      mbar_arrive_expect_tx(&s_bar[2 + b], n_rec * (uint32_t)sizeof(TileRec));
       issued += 1u << (8 * (2 + b));
-      if (bytes)
-        bulk_g2s(&s_rec[b][0], a.recs + (int64_t)(a.rec_tile0 + tile) * a.rec_stride + first, bytes, &s_bar[2 + b]);
+      if (dense && n_rec) bulk_g2s(&s_rec[b][0], recs + first, n_rec * (uint32_t)sizeof(TileRec), &s_bar[2 + b]);
     }
+    __syncwarp();
+    if (!dense && need) bulk_g2s(&s_rec[b][tid], recs + act, (uint32_t)sizeof(TileRec), &s_bar[2 + b]);
     __syncwarp();
   };
 
@@ -1767,6 +1777,57 @@ cudaError_t launch_replay(const int16_t* tab, int32_t log2_len, int64_t c, int64
   return cudaLaunchKernelEx(&l.cfg, replay_kernel, tab, mask, c, n, out, stride, vec, times);
 }
 
+// The tensor-core engine's two sums of a window, formed side by side (awg_host.cpp, render_engine):
+// the render's (part) plus the GEMM's (base), quantised and stored as the render's own epilogue
+// would.  10 bytes per sample; 8 samples per thread, 16-byte accesses where the outputs allow.
+__global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ part, const float* __restrict__ base,
+                                                      int64_t n, float scale, int16_t* __restrict__ out_q, int32_t q_stride,
+                                                      float* __restrict__ out_f, int vec, unsigned long long* end) {
+  const int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 8;
+  if (vec && i0 + 8 <= n) {
+    float x[8];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float4 p = __ldg(reinterpret_cast<const float4*>(part + i0) + h), b = __ldg(reinterpret_cast<const float4*>(base + i0) + h);
+      x[4 * h] = p.x + b.x;
+      x[4 * h + 1] = p.y + b.y;
+      x[4 * h + 2] = p.z + b.z;
+      x[4 * h + 3] = p.w + b.w;
+    }
+    if (out_f) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        reinterpret_cast<float4*>(out_f + i0)[h] = make_float4(x[4 * h], x[4 * h + 1], x[4 * h + 2], x[4 * h + 3]);
+    }
+    if (out_q) {
+      uint32_t w[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float q0 = fminf(fmaxf(rintf(x[2 * u] * scale), -32767.f), 32767.f);
+        const float q1 = fminf(fmaxf(rintf(x[2 * u + 1] * scale), -32767.f), 32767.f);
+        w[u] = (uint32_t)(uint16_t)(int16_t)q0 | ((uint32_t)(uint16_t)(int16_t)q1 << 16);
+      }
+      *reinterpret_cast<uint4*>(out_q + i0) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+  } else {
+    for (int64_t i = i0; i < min(i0 + 8, n); ++i) {
+      const float x = part[i] + base[i];
+      if (out_f) out_f[i] = x;
+      if (out_q) out_q[i * q_stride] = (int16_t)fminf(fmaxf(rintf(x * scale), -32767.f), 32767.f);
+    }
+  }
+  mark_end(end);
+}
+
+cudaError_t launch_combine(const float* part, const float* base, int64_t n, float scale, int16_t* out_q, int32_t q_stride,
+                           float* out_f, unsigned long long* end, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  const int vec = (!out_q || (q_stride <= 1 && ((uintptr_t)out_q & 15) == 0)) && ((uintptr_t)out_f & 15) == 0;
+  combine_kernel<<<(unsigned)((n + 2047) / 2048), 256, 0, s>>>(part, base, n, scale, out_q, q_stride > 1 ? q_stride : 1, out_f,
+                                                              vec, end);
+  return cudaGetLastError();
+}
+
 // End of a pipelined sequence: returns once every render CTA of the sequence has stored its
 // samples (*exit_ctr >= target), so that later work in the stream sees all of them.  Gives up after
 // limit_ns, sets the status word to AWG_ETIMEOUT and returns.
@@ -1807,6 +1868,49 @@ cudaError_t launch_render(const RenderArgs& a, cudaStream_t s) {
   cfg.attrs = attr;
   cfg.numAttrs = a.pdl ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, render_kernel, a);
+}
+
+// A list covers its whole window, but groups of tones that chirp in turn are live in a few tiles each:
+// one CTA per tile keeps the listed tones that are not static there, in order, and notes where each
+// rank's share begins.  Without it every render CTA searched the list (4 us) and staged all its
+// listed tones to skip most of them.
+__global__ void __launch_bounds__(128) sift_kernel(const __grid_constant__ SiftArgs a) {
+  __shared__ int s_live[4];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t T0 = (a.tile0 + blockIdx.x) * (int64_t)TILE;
+  int32_t* row = a.rows + (int64_t)blockIdx.x * a.n_list;
+  int32_t* first = a.first + (int64_t)blockIdx.x * (a.split + 1);
+  int count = 0;     // live tones so far
+  for (int i0 = 0; i0 < a.n_list; i0 += 128) {
+    const int i = i0 + tid;
+    const int k = i < a.n_list ? a.list[i] : -1;
+    const bool live = k >= 0 && !tile_static(a.tones[k], T0);
+    const unsigned m = __ballot_sync(0xffffffffu, live);
+    if (lane == 0) s_live[warp] = __popc(m);
+    __syncthreads();
+    int at = count + __popc(m & ((1u << lane) - 1u));
+    for (int w = 0; w < 4; ++w) {
+      if (w < warp) at += s_live[w];
+      count += s_live[w];
+    }
+    if (live) row[at] = k;
+    __syncthreads();
+  }
+  // rank boundaries (the row is ascending, its entries visible after the last barrier)
+  const int key = tid <= a.split ? a.bounds[tid] : 0;
+  int lo = 0, hi = count;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (row[mid] < key) lo = mid + 1;
+    else hi = mid;
+  }
+  if (tid <= a.split) first[tid] = lo;
+}
+
+cudaError_t launch_sift(const SiftArgs& a, cudaStream_t s) {
+  if (a.n_tiles == 0) return cudaSuccess;
+  sift_kernel<<<(unsigned)a.n_tiles, 128, 0, s>>>(a);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_exact_table(const TableArgs& a, int64_t L, cudaStream_t s) {

@@ -632,6 +632,9 @@ cudaError_t launch_table_gemm(const TableArgs2& t, cudaStream_t s) {
   auto kern = t.window_mode ? (bf16 ? table_gemm_kernel<__nv_bfloat16, true> : table_gemm_kernel<__half, true>)
                             : (bf16 ? table_gemm_kernel<__nv_bfloat16, false> : table_gemm_kernel<__half, false>);
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // all of the SM's shared memory, not the smallest split that holds a CTA (196 KB): what is left
+  // over takes a render CTA beside it (render_engine)
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   if (e != cudaSuccess) return e;
   // K split over a cluster of 1, 2 or 4 CTAs per 128-row tile (periodic tables), whichever finishes first by a
   // simple model: waves of co-resident clusters (a cluster of 4 leaves SMs of some GPCs idle: 36

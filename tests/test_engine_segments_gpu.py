@@ -70,3 +70,46 @@ def test_segments_at_tile_edges(awg, oracle, K, start):
     dq = np.abs(q.cpu().numpy().astype(np.int32) - oracle.quantize(ref, full).astype(np.int32))
     assert dq.max() <= 1
     s.close()
+
+
+@pytest.mark.parametrize("K,groups,aligned", [(600, 10, True), (600, 10, False), (97, 3, True), (3000, 40, False)])
+def test_groups_that_chirp_in_turn(awg, oracle, K, groups, aligned):
+    """Groups of interleaved tones (tone k in group k mod groups) that chirp for about two tiles in turn:
+    the tile's live tones are spread over the list, their records over the window's; also into an
+    unaligned buffer and as two interleaved channels."""
+    rng = np.random.default_rng(K)
+    f = rng.uniform(1e6, 139e6, K)
+    a = rng.uniform(0.2, 1.0, K)
+    th = rng.uniform(0, 2 * np.pi, K)
+    L = 2 * TILE - 100
+    chirps = [dict(tone=k, f_start=float(f[k]), f_end=float(rng.uniform(1e6, 139e6)), duration=L / FS, profile=k % 2,
+                   start_sample=1000 + (k % groups) * L) for k in range(K) if k % 7]
+    n = 1000 + groups * L + 3 * TILE + 5
+    handles = []
+    for _ in range(2):
+        s = awg.Synth(FS)
+        s.set_tones(f, a, th)
+        s.set_chirp_list(chirps)
+        s.set_static_engine(awg.STATIC_GEMM_FP16)
+        handles.append(s)
+    s = handles[0]
+    off = 0 if aligned else 3
+    q = torch.zeros(n + 8, dtype=torch.int16, device="cuda")
+    x = torch.zeros(n + 8, dtype=torch.float32, device="cuda")
+    s.render_f32(n, x[off:], q[off:])
+    w = oracle.make_waveform(FS, f, a, th, chirps)
+    ref = oracle.render(w, 0, n, nthreads=NTHREADS)
+    err = float(np.max(np.abs(x[off:off + n].cpu().numpy().astype(np.float64) - ref))) / (s.full_scale / 32767.0)
+    assert err <= 0.23, err
+    dq = np.abs(q[off:off + n].cpu().numpy().astype(np.int32) - oracle.quantize(ref, s.full_scale).astype(np.int32))
+    assert dq.max() <= 1
+    both = torch.zeros(2 * n, dtype=torch.int16, device="cuda")
+    for h in handles:
+        h.seek(0)
+    awg.render_multiplexed(handles, n, both)
+    torch.cuda.synchronize()
+    for c in range(2):
+        assert torch.equal(both[c::2], q[off:off + n])
+    for h in handles:
+        assert h.device_status() == 0
+        h.close()
