@@ -1091,18 +1091,31 @@ struct Window {
   int32_t n_tiles, per_launch;
   int32_t split;              // CTAs per part of a tile (set by the caller)
   bool first;                 // its first kernel starts the call (device time)
+  bool once;                  // RenderArgs::once: no set-up kernel
+  int32_t beside = 1;         // windows of this size that run side by side
   std::vector<int32_t> active;
   cudaEvent_t pe[4] = {nullptr, nullptr, nullptr, nullptr};   // profiling
   int64_t launches = 0;
 };
 
-int window_plan(awg_t* h, int64_t n, Window* w) {
+// A window with chirps and at most 96 tones per CTA (1536 tones) goes without a set-up kernel: each CTA
+// takes all its tones at once and forms their chirp records itself.  A call then has one kernel, which
+// may run beside the end of the one before: 1000 chirps x 2^18 samples 96 -> 71 us among others (the
+// set-up alone 13 us, and the render waits for it).  Not in chunk sequences, where one set-up kernel
+// serves all chunks and the records cost less there than in the render's CTAs (35 ms record 2611
+// against 2722 us), not without chirps (100 static tones 25.2 against 26.2 us), and not with more
+// tones, whose records would be formed in the middle of the sums.
+int window_plan(awg_t* h, int64_t n, bool listed, Window* w) {
   w->c = h->cursor;
   w->n = n;
-  const int64_t n_tiles = (w->c + n - 1) / awgk::TILE - w->c / awgk::TILE + 1;
+  w->tile0 = w->c / awgk::TILE;
+  const int64_t n_tiles = (w->c + n - 1) / awgk::TILE - w->tile0 + 1;
   if (n_tiles > (int64_t)(INT32_MAX / awgk::MAX_SPLIT)) return fail(AWG_EINVAL, "render window too long");
+  w->n_tiles = (int32_t)n_tiles;
   w->active = active_slots(h, w->c, n, &w->tile0, &w->n_tiles);
-  int st = ensure(&h->d_recs, &h->cap_recs, std::max<size_t>(1, w->active.size() * (size_t)w->n_tiles), h, "tile records");
+  w->once = !listed && !w->active.empty() && (int64_t)h->K <= (int64_t)awgk::ONCE_TONES * w->split;
+  if (w->once) w->active.clear();
+  int st = ensure(&h->d_recs, &h->cap_recs, w->active.size() * (size_t)w->n_tiles, h, "tile records");
   if (st) return st;
   // With a split, the window goes out in launches of at most SPLIT_LAUNCH_TILES tiles, on
   // alternating scratch buffers.
@@ -1161,6 +1174,8 @@ int window_render(awg_t* h, Window* w, awgk::RenderArgs ra, int32_t pdl, cudaStr
   ra.scale = h->full_scale > 0 ? (float)(32767.0 / h->full_scale) : 0.f;
   ra.status = h->d_status;
   std::memcpy(ra.inv_odd, h->inv_odd, sizeof(ra.inv_odd));
+  std::memcpy(ra.W, h->W, sizeof(ra.W));
+  ra.once = w->once;
   ra.rec_stride = (int32_t)w->active.size();
   ra.end = h->d_times + 1;
   for (int32_t t0 = 0, i = 0; t0 < w->n_tiles; t0 += w->per_launch, ++i) {
@@ -1171,13 +1186,15 @@ int window_render(awg_t* h, Window* w, awgk::RenderArgs ra, int32_t pdl, cudaStr
     rs.tile0 = w->tile0 + t0;
     rs.n_tiles = nt;
     rs.rec_tile0 = t0;
-    rs.parts = render_parts(nt, w->split, h->sine_mode);
+    rs.parts = render_parts((int64_t)nt * w->beside, w->split, h->sine_mode);
     rs.win_start = w0;
     rs.win_end = w1;
     rs.out_q = out_q ? out_q + (size_t)(w0 - c) * (size_t)(ra.q_stride ? ra.q_stride : 1) : nullptr;
     rs.out_f = out_f ? out_f + (w0 - c) : nullptr;
     rs.start = w->first && w->active.empty() && i == 0 ? h->d_times : nullptr;
-    rs.pdl = pdl == awgk::PDL_NONE || w->n_tiles <= w->per_launch ? pdl : (i == 0 ? awgk::PDL_SETUP_FIRST : awgk::PDL_FREE);
+    rs.pdl = pdl == awgk::PDL_NONE || pdl == awgk::PDL_FREE || w->n_tiles <= w->per_launch
+                 ? pdl
+                 : (i == 0 ? awgk::PDL_SETUP_FIRST : awgk::PDL_FREE);
     if (w->split > 1) {
       rs.part = split_part(h, i & 1);
       rs.tile_ctr = split_ctr(h, i & 1);
@@ -1234,7 +1251,7 @@ int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
   Window w;
   w.split = tone_list ? list_split : h->split;
   w.first = !engine_part;   // the engine's kernels came before
-  int st = window_plan(h, n, &w);
+  int st = window_plan(h, n, tone_list != nullptr, &w);
   if (!st) st = window_setup(h, &w, false, s);
   if (st) return st;
   awgk::RenderArgs ra;
@@ -2208,18 +2225,20 @@ int awg_render_multiplexed(awg_t* const* handles, int32_t n_channels, int64_t n,
     for (int32_t c = 0; c < n_channels && !st; ++c) {
       w[c].split = handles[c]->split;
       w[c].first = true;
-      st = window_plan(handles[c], n, &w[c]);
+      st = window_plan(handles[c], n, false, &w[c]);
     }
-    int32_t last_setup = 0;   // the last channel with a set-up kernel
-    for (int32_t c = 0; c < n_channels && !st; ++c)
+    int32_t last_setup = -1;   // the last channel with a set-up kernel
+    for (int32_t c = 0; c < n_channels && !st; ++c) {
+      w[c].beside = n_channels;
       if (!w[c].active.empty()) last_setup = c;
+    }
     for (int32_t c = 0; c < n_channels && !st; ++c) st = window_setup(handles[c], &w[c], c < last_setup, s);
     for (int32_t c = 0; c < n_channels && !st; ++c) {
       awgk::RenderArgs ra;
       std::memset(&ra, 0, sizeof(ra));
       ra.out_q = out + c;
       ra.q_stride = n_channels;
-      st = window_render(handles[c], &w[c], ra, c == 0 ? awgk::PDL_SETUP_FIRST : awgk::PDL_FREE, s);
+      st = window_render(handles[c], &w[c], ra, c == 0 && last_setup >= 0 ? awgk::PDL_SETUP_FIRST : awgk::PDL_FREE, s);
     }
     if (st)
       for (int32_t c = 0; c < n_channels; ++c) handles[c]->cursor = cursors[c];

@@ -18,6 +18,7 @@ constexpr int RUNS = 128;
 constexpr int TILE = RUN * RUNS;   // 4096 samples
 constexpr int RT = RUNS;           // threads per render CTA
 constexpr int STAGE = 32;          // tones staged in shared memory at a time (double-buffered)
+constexpr int ONCE_TONES = 3 * STAGE;   // tones of a CTA that are staged at once (RenderArgs::once)
 constexpr int SINE_SFU = 0;        // static segments: SFU sine of every sample's phase
 constexpr int SINE_ROTATOR = 1;    // static segments: exact sin/cos at the run start, then rotations
 constexpr int MAX_PARTS = 4;       // CTAs that may share a tile's samples (render_parts)
@@ -165,6 +166,7 @@ struct RenderArgs {
   float scale;            // 32767 / FS
   int32_t* status;
   uint64_t inv_odd[3][3];
+  uint32_t W[7][7];       // as PrepArgsT::W (once)
   int32_t sine_mode;      // SINE_SFU or SINE_ROTATOR (static segments)
   int32_t q_stride;       // int16 output: sample i goes to out_q[i * q_stride] (0: 1; channel multiplexing)
   // records: active chirp a of the set-up's window (numbered in tone order) for this render's tile t
@@ -199,6 +201,8 @@ struct RenderArgs {
   const int32_t* tile_first;
   int32_t cluster;        // 1: render_kernel, the split sums through a cluster's shared memory
   int32_t parts;          // CTAs that share a tile's samples: 1, 2 or 4 (render_split_kernel)
+  int32_t once;           // 1: every CTA has at most ONCE_TONES tones: all staged at once, the chirp
+                          // records formed by the CTA itself (recs and act_of_slot are not read)
   // split sums without clusters: partial sums part[((tile parts + p) split + rank) (TILE / parts) +
   // sample] and one counter per part of a tile (a multiple of split between launches: every CTA
   // adds 1)

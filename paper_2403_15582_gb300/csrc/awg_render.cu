@@ -643,6 +643,29 @@ __device__ __forceinline__ void store_record(TileRec* out, const TileRec& r) {
     o[i] = make_uint4((uint32_t)r.w[2 * i], (uint32_t)(r.w[2 * i] >> 32), (uint32_t)r.w[2 * i + 1], (uint32_t)(r.w[2 * i + 1] >> 32));
 }
 
+// The record of chirp c (of tone t) at tile T0, handed to put(count, record, count as a constant).
+template <int N>
+struct Count {
+  static constexpr int value = N;
+};
+template <class Args, class Put>
+__device__ __forceinline__ void form_record(const ChirpRec& c, const ToneRec& t, int64_t T0, const Args& a, Put put) {
+  const int words = rec_words(c, t, T0);
+  TileRec r;
+  if (words == REC_WORDS_LINEAR) {
+    prep_one<2, REC_WORDS_LINEAR>(c, T0 - c.n_s, a, r);
+    put(words, r, Count<REC_WORDS_LINEAR>());
+  } else if (words == REC_WORDS_LOW3) {
+    if (c.flags & TONE_EXP) prep_exp<REC_WORDS_LOW3>(c, T0 - c.n_s, a, r);
+    else prep_one<6, REC_WORDS_LOW3>(c, T0 - c.n_s, a, r);
+    put(words, r, Count<REC_WORDS_LOW3>());
+  } else {
+    if (c.flags & TONE_EXP) prep_exp<REC_WORDS>(c, T0 - c.n_s, a, r);
+    else prep_one<6, REC_WORDS>(c, T0 - c.n_s, a, r);
+    put(words, r, Count<REC_WORDS>());
+  }
+}
+
 template <class Args>
 __global__ void __launch_bounds__(128, 5) prep_kernel(const __grid_constant__ Args a) {
   mark_start(a.start);
@@ -657,26 +680,13 @@ __global__ void __launch_bounds__(128, 5) prep_kernel(const __grid_constant__ Ar
   const int slot = a.slots[ai];
   const ChirpRec& c = a.chirps[slot];
   const int64_t T0 = (a.tile0 + t) * (int64_t)TILE;
-  const int words = rec_words(c, a.tones[c.tone], T0);
   TileRec* out = a.recs + (int64_t)t * a.rec_stride + a.act_base + ai;
-  TileRec r;
   // the preceding kernel of the stream may be a render that reads the buffers written here: it has
   // to be complete before the first write, not before the arithmetic
-  if (words == REC_WORDS_LINEAR) {
-    prep_one<2, REC_WORDS_LINEAR>(c, T0 - c.n_s, a, r);
+  form_record(c, a.tones[c.tone], T0, a, [&](int, const TileRec& r, auto words) {
     pdl_wait();
-    store_record<REC_WORDS_LINEAR>(out, r);
-  } else if (words == REC_WORDS_LOW3) {
-    if (c.flags & TONE_EXP) prep_exp<REC_WORDS_LOW3>(c, T0 - c.n_s, a, r);
-    else prep_one<6, REC_WORDS_LOW3>(c, T0 - c.n_s, a, r);
-    pdl_wait();
-    store_record<REC_WORDS_LOW3>(out, r);
-  } else {
-    if (c.flags & TONE_EXP) prep_exp<REC_WORDS>(c, T0 - c.n_s, a, r);
-    else prep_one<6, REC_WORDS>(c, T0 - c.n_s, a, r);
-    pdl_wait();
-    store_record<REC_WORDS>(out, r);
-  }
+    store_record<decltype(words)::value>(out, r);
+  });
   if (t == 0) a.act_of_slot[slot] = a.act_base + ai;
 }
 
@@ -728,35 +738,20 @@ __device__ __forceinline__ void static_loop(uint32_t p, uint32_t f, float A, Acc
   }
 }
 
-// Chirp cascade p += f, f += g (and g += h with WITH_H).  Without h the phases go in blocks of
-// four, p_{k+1} = p_k + f + k g with the multiples of g formed once: one three-input add per
-// sample (16 samples per thread, the loop alone: 4.09 -> 4.40e12 sines/s; 32 samples: 4.40 ->
-// 4.43e12).
+// Chirp cascade p += f, f += g (and g += h with WITH_H).
 template <int SPT, bool WITH_H>
 __device__ __forceinline__ void cascade(const RunPoly& q, float A, Acc<SPT>& acc) {
   uint32_t p = q.p, f = q.f, g = q.g;
-  if constexpr (WITH_H) {
-    const uint32_t h = q.h;
+  const uint32_t h = q.h;
 #pragma unroll
-    for (int r = 0; r < SPT; r += 2) {
-      const uint32_t p1 = p + f;
-      const uint32_t f1 = f + g;
-      g += h;
-      acc_pair(acc[r / 2], A, p, p1);
-      p = p1 + f1;
-      f = f1 + g;
-      g += h;
-    }
-  } else {
-    const uint32_t g2 = 2u * g, g3 = 3u * g, g4 = 4u * g;
-#pragma unroll
-    for (int r = 0; r < SPT; r += 4) {
-      const uint32_t p1 = p + f, p2 = p1 + f + g, p3 = p2 + f + g2;
-      acc_pair(acc[r / 2], A, p, p1);
-      acc_pair(acc[r / 2 + 1], A, p2, p3);
-      p = p3 + f + g3;
-      f += g4;
-    }
+  for (int r = 0; r < SPT; r += 2) {
+    const uint32_t p1 = p + f;
+    const uint32_t f1 = f + g;
+    if (WITH_H) g += h;
+    acc_pair(acc[r / 2], A, p, p1);
+    p = p1 + f1;
+    f = f1 + g;
+    if (WITH_H) g += h;
   }
 }
 
@@ -1170,17 +1165,22 @@ __device__ __forceinline__ void tile_epilogue_split(const RenderArgs& a, int uni
 //
 // The tones go through in stages of STAGE, in the stage's visit order: the groups of visit_group, each
 // in a loop of its own without a per-tone dispatch, then the rest.
-template <int SPT, bool CLUSTER>
+// MODE_ONCE: RenderArgs::once; MODE_LIST: a tone list, if a.tone_list is set; MODE_ALL: all tones.
+enum { MODE_ALL = 0, MODE_LIST = 1, MODE_ONCE = 2, N_MODES = 3 };
+template <int SPT, bool CLUSTER, int MODE>
 __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit, const int crank, const int split) {
   using G = Geo<SPT>;
   constexpr int PARTS = G::PARTS, RW = G::RW;
+  constexpr bool ONCE = MODE == MODE_ONCE;
   static_assert(!CLUSTER || SPT == RUN, "cluster sums take whole tiles");
-  __shared__ alignas(16) ToneRec s_tone[2][STAGE];
-  __shared__ alignas(16) TileRec s_rec[2][STAGE];
-  __shared__ alignas(16) Desc s_desc[2][STAGE];
-  __shared__ uint8_t s_order[2][STAGE];          // visit order
-  __shared__ uint8_t s_kind[2][STAGE];           // kinds, in visit order
-  __shared__ int s_ngrp[2][N_GRP];                // ends of the visit groups
+  constexpr int NBUF = ONCE ? ONCE_TONES / STAGE : 2;   // stage buffers
+  static_assert(!ONCE || NBUF <= RT / 32, "a warp prepares a stage");
+  __shared__ alignas(16) ToneRec s_tone[NBUF][STAGE];
+  __shared__ alignas(16) TileRec s_rec[NBUF][STAGE];
+  __shared__ alignas(16) Desc s_desc[NBUF][STAGE];
+  __shared__ uint8_t s_order[NBUF][STAGE];       // visit order
+  __shared__ uint8_t s_kind[NBUF][STAGE];        // kinds, in visit order
+  __shared__ int s_ngrp[NBUF][N_GRP];             // ends of the visit groups
   // cluster sums through distributed shared memory: [i][thread]
   __shared__ alignas(16) float s_red[CLUSTER ? TILE : 4];
   __shared__ alignas(8) uint64_t s_bar[4];        // tones[0], tones[1], records[0], records[1]
@@ -1197,8 +1197,9 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
   // positions [l_begin, l_end) of the visit: the CTA's range of tones, or of the tone list
   int l_begin = (int)((int64_t)a.K * crank / split);
   int l_end = (int)((int64_t)a.K * (crank + 1) / split);
-  const int32_t* list = a.tone_list;
-  if (a.tile_first) {
+  const int32_t* list = MODE == MODE_LIST ? a.tone_list : nullptr;
+  if (MODE != MODE_LIST) {
+  } else if (a.tile_first) {
     const int32_t* first = a.tile_first + (int64_t)(a.rec_tile0 + tile) * (split + 1);
     list += (int64_t)(a.rec_tile0 + tile) * a.n_list;
     l_begin = first[crank];
@@ -1254,26 +1255,27 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
       bulk_g2s(&s_tone[st & 1][tid], a.tones + list[lb + tid], (uint32_t)sizeof(ToneRec), &s_bar[st & 1]);
     }
   };
-  // warp 0, once the stage's tones have landed: descriptors, visit order, and the records of tones
-  // that chirp inside this tile: the window's active chirps are numbered in tone order, so the
-  // records of a stage's consecutive tones lie one after another and come in one bulk copy
+  // One warp (warp 0, or warp st with ONCE), once the stage's tones have landed: descriptors, visit
+  // order, and the records of tones that chirp inside this tile.  ONCE forms them here, a tone per
+  // lane; otherwise the set-up kernel did: the window's active chirps are numbered in tone order, so
+  // the records of a stage's consecutive tones lie one after another and come in one bulk copy.
   auto prepare_stage = [&](int st) {
-    const int b = st & 1;
+    const int b = ONCE ? st : st & 1;
     const int cnt = min(STAGE, l_end - (l_begin + st * STAGE));
     bool need = false, pairable = false;
     int kind = DESC_SKIP, act = 0;
-    if (tid < cnt) {
-      const ToneRec& tr = s_tone[b][tid];
+    if (lane < cnt) {
+      const ToneRec& tr = s_tone[b][lane];
       const int tcls = classify_tile(tr, T0);
       need = tcls == TILE_CHIRP && !(tr.flags & TONE_EXACT);
-      if (need) act = a.act_of_slot[tr.slot];
+      if (!ONCE && need) act = a.act_of_slot[tr.slot];
       Desc d;
       const bool ramp = (tr.flags & TONE_AMP_RAMP) != 0;
       d.A = (ramp && T0 >= tr.a_ns + tr.a_L) ? tr.A_end : tr.A;
       d.c = d.s = 0.f;
       d.F = 0;
       d.p0 = 0;
-      d.rec = 0;
+      d.rec = lane;
       if (tcls == TILE_PRE || tcls == TILE_POST) {
         const bool pre = tcls == TILE_PRE;
         d.F = pre ? tr.F : tr.F_end;
@@ -1285,7 +1287,7 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
       }
       kind = tile_kind(tr, T0, a.skip_static != 0);
       if (kind == DESC_STATIC && a.sine_mode == SINE_ROTATOR) kind = DESC_STATIC_ROT;
-      s_desc[b][tid] = d;
+      s_desc[b][lane] = d;
       pairable = (tr.flags & TONE_PAIR) && !a.skip_static;
     }
     // visit order: the chirps that cover the tile in linear form, those in LOW3 and LOW6 form, the
@@ -1294,25 +1296,35 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
     // tones) that changes with the window, so listed renders keep plain tone order, and every window
     // cut gives the same bits.  Skipped tones are left out.
     const int grp = kind == DESC_SKIP ? -1 : visit_group(kind, list != nullptr, pairable);
-    const unsigned below = (1u << tid) - 1u;
+    const unsigned below = (1u << lane) - 1u;
     int pos = 0, end = 0;
 #pragma unroll
     for (int g = 0; g < N_GRP; ++g) {
       const unsigned m = __ballot_sync(0xffffffffu, grp == g);
       if (grp == g) pos = end + __popc(m & below);
       end += __popc(m);
-      if (tid == 0) s_ngrp[b][g] = end;
+      if (lane == 0) s_ngrp[b][g] = end;
     }
     if (grp >= 0) {
-      s_order[b][pos] = (uint8_t)tid;
+      s_order[b][pos] = (uint8_t)lane;
       s_kind[b][pos] = (uint8_t)kind;
+    }
+    if constexpr (ONCE) {
+      if (need) {
+        const ToneRec& tr = s_tone[b][lane];
+        form_record(a.chirps[tr.slot], tr, T0, a, [&](int, const TileRec& r, auto words) {
+#pragma unroll
+          for (int i = 0; i < decltype(words)::value; ++i) s_rec[b][lane].w[i] = r.w[i];
+        });
+      }
+      return;
     }
     const unsigned mask = __ballot_sync(0xffffffffu, need);
     const int first = __shfl_sync(0xffffffffu, act, mask ? __ffs(mask) - 1 : 0);
     const int last = __shfl_sync(0xffffffffu, act, mask ? 31 - __clz(mask) : 0);
     // (the tones left out of a sifted list leave gaps: then one copy per record)
-    const bool dense = (unsigned)(last - first) < (unsigned)STAGE;
-    if (need) s_desc[b][tid].rec = dense ? act - first : tid;
+    const bool dense = MODE != MODE_LIST || (unsigned)(last - first) < (unsigned)STAGE;
+    if (need) s_desc[b][lane].rec = dense ? act - first : tid;
     const TileRec* recs = a.recs + (int64_t)(a.rec_tile0 + tile) * a.rec_stride;
     if (tid == 0) {
       const uint32_t n_rec = !mask ? 0u : dense ? (uint32_t)(last - first + 1) : (uint32_t)__popc(mask);
@@ -1327,7 +1339,20 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
   };
 
   bool ok = true;
-  if (n_stages > 0) {
+  if constexpr (ONCE) {
+    if (n_stages > 0) {
+      if (tid == 0) {
+        const uint32_t bytes = (uint32_t)(l_end - l_begin) * (uint32_t)sizeof(ToneRec);
+        mbar_arrive_expect_tx(&s_bar[0], bytes);
+        issued = 1u;
+        bulk_g2s(&s_tone[0][0], a.tones + l_begin, bytes, &s_bar[0]);
+      }
+      ok = mbar_wait(&s_bar[0], 0);
+      ok = __syncthreads_and(ok) != 0;
+      if (ok && warp < n_stages) prepare_stage(warp);
+      __syncthreads();
+    }
+  } else if (n_stages > 0) {
     if (tid < 32) {
       issue_tones(0);
       if (n_stages > 1) issue_tones(1);
@@ -1337,19 +1362,21 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
     }
     __syncthreads();   // stage-0 descriptors visible
   }
-  int fail_stage = -1;
+  int fail_stage = ONCE && !ok ? 0 : -1;
   const RunBin rb = run_binomials(run);
   for (int st = 0; st < n_stages; ++st) {
-    const int b = st & 1;
-    const uint32_t par = (uint32_t)((st >> 1) & 1);
-    if (tid < 32 && st + 1 < n_stages) {
-      ok &= mbar_wait(&s_bar[(st + 1) & 1], (uint32_t)(((st + 1) >> 1) & 1));
-      prepare_stage(st + 1);
+    const int b = ONCE ? st : st & 1;
+    if constexpr (!ONCE) {
+      const uint32_t par = (uint32_t)((st >> 1) & 1);
+      if (tid < 32 && st + 1 < n_stages) {
+        ok &= mbar_wait(&s_bar[(st + 1) & 1], (uint32_t)(((st + 1) >> 1) & 1));
+        prepare_stage(st + 1);
+      }
+      ok &= mbar_wait(&s_bar[b], par);
+      ok &= mbar_wait(&s_bar[2 + b], par);
+      // the same decision in every lane of the warp: the loops below exchange values between lanes
+      ok = __all_sync(0xffffffffu, ok);
     }
-    ok &= mbar_wait(&s_bar[b], par);
-    ok &= mbar_wait(&s_bar[2 + b], par);
-    // the same decision in every lane of the warp: the loops below exchange values between lanes
-    ok = __all_sync(0xffffffffu, ok);
     if (ok) {
       const int e_lp = s_ngrp[b][GRP_LIN_PAIR], e_lin = s_ngrp[b][GRP_LIN], e_l3p = s_ngrp[b][GRP_LOW3_PAIR],
                 e_l6p = s_ngrp[b][GRP_LOW6_PAIR], e_low6 = s_ngrp[b][GRP_LOW6], e_static = s_ngrp[b][GRP_STATIC],
@@ -1478,11 +1505,13 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
         }
       }
     }
-    if (!__syncthreads_and(ok)) {   // stage buffers free, next stage's descriptors visible
-      fail_stage = st;
-      break;
+    if constexpr (!ONCE) {
+      if (!__syncthreads_and(ok)) {   // stage buffers free, next stage's descriptors visible
+        fail_stage = st;
+        break;
+      }
+      if (tid < 32 && st + 2 < n_stages) issue_tones(st + 2);
     }
-    if (tid < 32 && st + 2 < n_stages) issue_tones(st + 2);
   }
   if (fail_stage >= 0) {
     // report, then let every copy still in flight land (bounded) before shared memory goes away
@@ -1535,24 +1564,26 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
   }
 }
 
-// Register budgets, by CTAs per SM.  Whole tiles: six (80 registers, 56 bytes of spill loads); the
+// Register budgets, by CTAs per SM.  Whole tiles: six (80 registers, 44 bytes of spill loads); the
 // 1000-chirp 35 ms record took 2636 us at six, 2703 at seven (72 registers), 2711 at five; the batched
-// and cluster renders keep five (no spills).  Parts need fewer accumulators: eight.
+// and cluster renders keep five (no spills).  Parts need fewer accumulators: eight, but six where the
+// CTA forms its records (at eight 1.2 KB of spills).  A kernel per mode: with the list's code in it the
+// plain render's registers change and the record takes 2640 instead of 2616 us.
 #define AWG_RENDER_MIN_BLOCKS 5
 #define AWG_RENDER_SPLIT_MIN_BLOCKS 6
 #define AWG_RENDER_PART_MIN_BLOCKS 8
 __global__ void __launch_bounds__(RT, AWG_RENDER_MIN_BLOCKS) render_kernel(const __grid_constant__ RenderArgs a) {
   mark_start(a.start);
   cg::cluster_group cluster = cg::this_cluster();
-  render_tile<RUN, true>(a, blockIdx.x / a.split, (int)cluster.block_rank(), a.split);
+  render_tile<RUN, true, MODE_ALL>(a, blockIdx.x / a.split, (int)cluster.block_rank(), a.split);
 }
 
 // The same without clusters (a.part set when split > 1): CTA blockIdx.x takes rank blockIdx.x % split.
-template <int SPT>
-__global__ void __launch_bounds__(RT, SPT == RUN ? AWG_RENDER_SPLIT_MIN_BLOCKS : AWG_RENDER_PART_MIN_BLOCKS)
+template <int SPT, int MODE>
+__global__ void __launch_bounds__(RT, SPT == RUN || MODE == MODE_ONCE ? AWG_RENDER_SPLIT_MIN_BLOCKS : AWG_RENDER_PART_MIN_BLOCKS)
     render_split_kernel(const __grid_constant__ RenderArgs a) {
   mark_start(a.start);
-  render_tile<SPT, false>(a, blockIdx.x / a.split, blockIdx.x % a.split, a.split);
+  render_tile<SPT, false, MODE>(a, blockIdx.x / a.split, blockIdx.x % a.split, a.split);
 }
 
 // Several renders in one grid (continuous batching): CTA group i (split CTAs) renders window tile
@@ -1563,7 +1594,7 @@ __global__ void __launch_bounds__(RT, AWG_RENDER_MIN_BLOCKS) render_batch_split_
                                                                                        const int2* __restrict__ items,
                                                                                        int split) {
   const int2 it = items[blockIdx.x / split];
-  render_tile<RUN, false>(reqs[it.x], it.y, (int)(blockIdx.x % split), split);
+  render_tile<RUN, false, MODE_LIST>(reqs[it.x], it.y, (int)(blockIdx.x % split), split);
 }
 
 // The 32-bit phase the render feeds to the sine for sample s of the tile [T0, T0 + TILE) (any
@@ -1675,12 +1706,24 @@ int device_sm_count() {
   return n;
 }
 
+// The render kernel that cuts a tile over `parts` CTAs.
+typedef void (*SplitKernel)(const RenderArgs);
+template <int MODE>
+static SplitKernel split_kernel_of(int parts) {
+  return parts == 4 ? render_split_kernel<8, MODE> : parts == 2 ? render_split_kernel<16, MODE> : render_split_kernel<32, MODE>;
+}
+static SplitKernel split_kernel(int parts, int mode) {
+  return mode == MODE_ONCE ? split_kernel_of<MODE_ONCE>(parts)
+         : mode == MODE_LIST ? split_kernel_of<MODE_LIST>(parts) : split_kernel_of<MODE_ALL>(parts);
+}
+
 cudaError_t render_setup_attributes() {
   cudaError_t e = cudaFuncSetAttribute(render_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   // shared memory before L1 for AWG_RENDER_SPLIT_MIN_BLOCKS CTAs
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(render_split_kernel<32>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(render_split_kernel<16>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(render_split_kernel<8>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  for (int parts = 1; parts <= MAX_PARTS; parts *= 2)
+    for (int mode = 0; mode < N_MODES; ++mode)
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(split_kernel(parts, mode), cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   return e;
 }
 
@@ -1909,9 +1952,7 @@ cudaError_t launch_render(const RenderArgs& a, cudaStream_t s) {
   if (!a.cluster) {   // the split sums through the scratch partials
     cfg.attrs = attr + 1;
     cfg.numAttrs = a.pdl ? 1 : 0;
-    if (parts == 4) return cudaLaunchKernelEx(&cfg, render_split_kernel<8>, a);
-    if (parts == 2) return cudaLaunchKernelEx(&cfg, render_split_kernel<16>, a);
-    return cudaLaunchKernelEx(&cfg, render_split_kernel<32>, a);
+    return cudaLaunchKernelEx(&cfg, split_kernel(parts, a.once ? MODE_ONCE : a.tone_list ? MODE_LIST : MODE_ALL), a);
   }
   cfg.attrs = attr;
   cfg.numAttrs = a.pdl ? 2 : 1;
