@@ -175,11 +175,27 @@ def chirp_rate_probe(out, blocks: int, runs: int, stream=None):
     _check(lib().awg_chirp_rate_probe(_ptr(out), int(blocks), int(runs), _stream_ptr(stream)))
 
 
+_current_stream = None
+
+
+def _find_current_stream():
+    """The handle of torch's current stream as a function, looked up once: through the raw-stream query
+    where torch has one (0.4 us a call), else through a Stream object (3.3 us)."""
+    global _current_stream
+    import torch
+    try:
+        device, raw = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
+        raw(device())
+        _current_stream = lambda: raw(device())   # noqa: E731
+    except Exception:
+        _current_stream = lambda: torch.cuda.current_stream().cuda_stream   # noqa: E731
+    return _current_stream
+
+
 def _stream_ptr(stream):
     if stream is None:
         try:
-            import torch
-            return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+            return ctypes.c_void_p((_current_stream or _find_current_stream())())
         except Exception:
             return ctypes.c_void_p(0)
     if hasattr(stream, "cuda_stream"):

@@ -88,3 +88,40 @@ def test_unsynchronised_calls_write_the_same(awglib, handles, seed):
     for h in handles:
         assert h.device_status() == 0
         assert 0 < h.last_render_ms() < 1000
+
+
+def test_new_tones_and_chirps_behind_renders(awglib):
+    """set_tones and set_chirps queue their uploads behind the renders issued so far: one handle that is
+    given new tones, scattered chirps (few and many, short ones with phase tables too) and fewer or more
+    tones again, without a synchronisation, against a fresh handle for every round."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    n = 60001
+    one = awglib.Synth(FS)
+    got, want = [], []
+    for rnd, K in enumerate([40, 700, 700, 30, 0, 650, 700, 1, 2000, 1900]):
+        r = np.random.default_rng(rnd)
+        f, a, th = r.uniform(1e6, 139e6, K), r.uniform(0.2, 1, K), r.uniform(0, 6, K)
+        nc = [K // 2, 3, K // 7, K, 0, 100, 5, 1, 40, 1900][rnd]
+        t = np.sort(r.choice(K, nc, replace=False)) if nc else np.zeros(0, dtype=int)
+        dur = np.where(np.arange(nc) % 4 == 0, 3e-7, 1.5e-4)
+        args = (t, f[t], r.uniform(1e6, 139e6, nc), dur, np.arange(nc) % 2, r.integers(0, 20000, nc))
+        fresh = awglib.Synth(FS)
+        for s, outs in ((one, got), (fresh, want)):
+            s.seek(0)
+            s.set_tones(f, a, th)
+            if nc:
+                s.set_chirps(*args)
+            out = torch.empty(n, dtype=torch.int16, device="cuda")
+            s.render(n, out)
+            outs.append(out)
+            out = torch.empty(n, dtype=torch.int16, device="cuda")
+            s.seek(0)
+            s.render_stream(n, 7000, out)
+            outs.append(out)
+        torch.cuda.synchronize() if rnd % 4 == 3 else None
+        fresh.device_status() if rnd % 5 == 4 else None
+    torch.cuda.synchronize()
+    for i, (x, y) in enumerate(zip(got, want)):
+        assert torch.equal(x, y), i
+    assert one.device_status() == 0
