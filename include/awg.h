@@ -259,7 +259,8 @@ int awg_render_chunks(awg_t* h, int64_t chunk, int32_t n_chunks, int16_t* out, v
 int awg_render_stream(awg_t* h, int64_t n, int64_t chunk, int16_t* out, void* stream);
 
 /* Number of kernels the handle has launched so far (every render, set-up, join, table and replay
- * kernel, including those of set-up calls and test hooks); -1 for a null handle.  Read it before
+ * kernel, including those of set-up calls and test hooks; a multiplexed launch of several channels
+ * counts on the first one); -1 for a null handle.  Read it before
  * and after a region to count that region's launches. */
 int64_t awg_launch_count(const awg_t* h);
 

@@ -1121,7 +1121,6 @@ struct Window {
   int32_t split;              // CTAs per part of a tile (set by the caller)
   bool first;                 // its first kernel starts the call (device time)
   bool once;                  // RenderArgs::once: no set-up kernel
-  int32_t beside = 1;         // windows of this size that run side by side
   std::vector<int32_t> active;
   cudaEvent_t pe[4] = {nullptr, nullptr, nullptr, nullptr};   // profiling
   int64_t launches = 0;
@@ -1134,7 +1133,9 @@ struct Window {
 // serves all chunks and the records cost less there than in the render's CTAs (35 ms record 2611
 // against 2722 us), not without chirps (100 static tones 25.2 against 26.2 us), and not with more
 // tones, whose records would be formed in the middle of the sums.
-int window_plan(awg_t* h, int64_t n, bool listed, Window* w) {
+bool once_fits(const awg_t* h, int32_t split) { return (int64_t)h->K <= (int64_t)awgk::ONCE_TONES * split; }
+
+int window_plan(awg_t* h, int64_t n, bool may_once, Window* w) {
   w->c = h->cursor;
   w->n = n;
   w->tile0 = w->c / awgk::TILE;
@@ -1142,7 +1143,7 @@ int window_plan(awg_t* h, int64_t n, bool listed, Window* w) {
   if (n_tiles > (int64_t)(INT32_MAX / awgk::MAX_SPLIT)) return fail(AWG_EINVAL, "render window too long");
   w->n_tiles = (int32_t)n_tiles;
   w->active = active_slots(h, w->c, n, &w->tile0, &w->n_tiles);
-  w->once = !listed && !w->active.empty() && (int64_t)h->K <= (int64_t)awgk::ONCE_TONES * w->split;
+  w->once = may_once && once_fits(h, w->split) && !w->active.empty();
   if (w->once) w->active.clear();
   int st = ensure(&h->d_recs, &h->cap_recs, w->active.size() * (size_t)w->n_tiles, h, "tile records");
   if (st) return st;
@@ -1184,50 +1185,60 @@ int window_setup(awg_t* h, Window* w, bool more, cudaStream_t s) {
   return AWG_OK;
 }
 
-// The render launches; out_q, out_f, the tone list and q_stride come in ra.  pdl: the first
-// launch's form (with programmatic launch, a window of several launches starts with PDL_SETUP_FIRST,
-// so that the later ones find the records).
-int window_render(awg_t* h, Window* w, awgk::RenderArgs ra, int32_t pdl, cudaStream_t s) {
+// Arguments of launch i of a window, of its tiles [t0, t0 + nt): out_q and out_f come in as the window's.
+void launch_args(awg_t* h, const Window& w, int32_t t0, int32_t nt, int i, awgk::RenderArgs* ra) {
+  ra->tones = h->d_tones;
+  ra->exact_tab = h->d_tab;
+  ra->chirps = h->d_chirps;
+  ra->recs = h->d_recs;
+  ra->act_of_slot = h->d_act;
+  ra->K = h->K;
+  ra->split = w.split;
+  ra->sine_mode = h->sine_mode;
+  ra->scale = h->full_scale > 0 ? (float)(32767.0 / h->full_scale) : 0.f;
+  ra->status = h->d_status;
+  std::memcpy(ra->inv_odd, h->inv_odd, sizeof(ra->inv_odd));
+  std::memcpy(ra->W, h->W, sizeof(ra->W));
+  ra->once = w.once;
+  ra->rec_stride = (int32_t)w.active.size();
+  ra->tile0 = w.tile0 + t0;
+  ra->n_tiles = nt;
+  ra->rec_tile0 = t0;
+  ra->win_start = std::max(w.c, ra->tile0 * (int64_t)awgk::TILE);
+  ra->win_end = std::min(w.c + w.n, (ra->tile0 + nt) * (int64_t)awgk::TILE);
+  const int64_t shift = ra->win_start - w.c;
+  if (ra->out_q) ra->out_q += (size_t)shift * (size_t)(ra->q_stride ? ra->q_stride : 1);
+  if (ra->out_f) ra->out_f += shift;
+  ra->start = w.first && w.active.empty() && i == 0 ? h->d_times : nullptr;
+  ra->end = h->d_times + 1;
+  if (w.split > 1) {
+    ra->part = split_part(h, i & 1);
+    ra->tile_ctr = split_ctr(h, i & 1);
+  }
+}
+
+// After the window's last launch on stream s.
+int window_done(awg_t* h, const Window& w, cudaStream_t s) {
+  const cudaError_t e = cudaEventRecord(h->ev_done, s);
+  if (e != cudaSuccess) return cuda_fail(e, "event");
+  h->timed = true;
+  h->have_done = true;
+  h->cursor = w.c + w.n;
+  return AWG_OK;
+}
+
+// The render launches.  With programmatic launch, a window of several launches starts with
+// PDL_SETUP_FIRST, so that the later ones find the records.
+int window_render(awg_t* h, Window* w, const awgk::RenderArgs& ra, int32_t pdl, cudaStream_t s) {
   cudaError_t e;
-  const int64_t c = w->c, n = w->n;
-  int16_t* out_q = ra.out_q;
-  float* out_f = ra.out_f;
-  ra.tones = h->d_tones;
-  ra.exact_tab = h->d_tab;
-  ra.chirps = h->d_chirps;
-  ra.recs = h->d_recs;
-  ra.act_of_slot = h->d_act;
-  ra.K = h->K;
-  ra.split = w->split;
-  ra.sine_mode = h->sine_mode;
-  ra.scale = h->full_scale > 0 ? (float)(32767.0 / h->full_scale) : 0.f;
-  ra.status = h->d_status;
-  std::memcpy(ra.inv_odd, h->inv_odd, sizeof(ra.inv_odd));
-  std::memcpy(ra.W, h->W, sizeof(ra.W));
-  ra.once = w->once;
-  ra.rec_stride = (int32_t)w->active.size();
-  ra.end = h->d_times + 1;
   for (int32_t t0 = 0, i = 0; t0 < w->n_tiles; t0 += w->per_launch, ++i) {
     awgk::RenderArgs rs = ra;
     const int32_t nt = std::min(w->per_launch, w->n_tiles - t0);
-    const int64_t w0 = std::max(c, (w->tile0 + t0) * (int64_t)awgk::TILE);
-    const int64_t w1 = std::min(c + n, (w->tile0 + t0 + nt) * (int64_t)awgk::TILE);
-    rs.tile0 = w->tile0 + t0;
-    rs.n_tiles = nt;
-    rs.rec_tile0 = t0;
-    rs.parts = render_parts((int64_t)nt * w->beside, w->split, h->sine_mode);
-    rs.win_start = w0;
-    rs.win_end = w1;
-    rs.out_q = out_q ? out_q + (size_t)(w0 - c) * (size_t)(ra.q_stride ? ra.q_stride : 1) : nullptr;
-    rs.out_f = out_f ? out_f + (w0 - c) : nullptr;
-    rs.start = w->first && w->active.empty() && i == 0 ? h->d_times : nullptr;
+    launch_args(h, *w, t0, nt, i, &rs);
+    rs.parts = render_parts(nt, w->split, h->sine_mode);
     rs.pdl = pdl == awgk::PDL_NONE || pdl == awgk::PDL_FREE || w->n_tiles <= w->per_launch
                  ? pdl
                  : (i == 0 ? awgk::PDL_SETUP_FIRST : awgk::PDL_FREE);
-    if (w->split > 1) {
-      rs.part = split_part(h, i & 1);
-      rs.tile_ctr = split_ctr(h, i & 1);
-    }
     if ((e = counted(h, awgk::launch_render(rs, s))) != cudaSuccess) return cuda_fail(e, "render launch");
     ++w->launches;
   }
@@ -1236,10 +1247,60 @@ int window_render(awg_t* h, Window* w, awgk::RenderArgs ra, int32_t pdl, cudaStr
     ++h->prof_calls;
     h->prof_launches += w->launches;
   }
-  if ((e = cudaEventRecord(h->ev_done, s)) != cudaSuccess) return cuda_fail(e, "event");
-  h->timed = true;
-  h->have_done = true;
-  h->cursor = c + n;
+  return window_done(h, *w, s);
+}
+
+// Several channels' direct renders, interleaved into out.  The launches take all channels (at most
+// SPLIT_LAUNCH_TILES tiles of each): launches of their own would each wait, before their sums and stores,
+// for the channel before to complete (eight channels of 100 chirps x 50,001 samples 89 -> 21 us, two of
+// 250 static tones x 2^18 47 -> 29, three of 900 tones x 10^6 640 -> 629, four of 250 chirps x 2^18 97 -> 97).
+// Each CTA forms its chirp records itself where it may on every channel; otherwise all channels' set-ups
+// come first.
+int render_channels(awg_t* const* handles, int32_t n_channels, int64_t n, int16_t* out, cudaStream_t s) {
+  Window w[awgk::MAX_CHANNELS];
+  bool may_once = true, once = false;
+  int32_t sine = AWG_SINE_SFU, max_tiles = 0, last_setup = -1;
+  for (int32_t c = 0; c < n_channels; ++c) {
+    may_once = may_once && once_fits(handles[c], handles[c]->split);
+    if (handles[c]->sine_mode == AWG_SINE_ROTATOR) sine = AWG_SINE_ROTATOR;   // whole tiles on all channels
+  }
+  int st = AWG_OK;
+  for (int32_t c = 0; c < n_channels; ++c) {
+    w[c].split = handles[c]->split;
+    w[c].first = true;
+    if ((st = window_plan(handles[c], n, may_once, &w[c]))) return st;
+    once = once || w[c].once;
+    if (!w[c].active.empty()) last_setup = c;
+    max_tiles = std::max(max_tiles, w[c].n_tiles);
+  }
+  for (int32_t c = 0; c < n_channels; ++c) {
+    w[c].once = once;   // one kernel for all: a static channel's CTAs stage their tones likewise
+    if ((st = window_setup(handles[c], &w[c], c < last_setup, s))) return st;
+  }
+  for (int32_t t0 = 0, i = 0; t0 < max_tiles; t0 += SPLIT_LAUNCH_TILES, ++i) {
+    awgk::MuxArgs m;
+    std::memset(&m, 0, sizeof(m));
+    m.n = n_channels;
+    int64_t ctas = 0;
+    for (int32_t c = 0; c < n_channels; ++c) {
+      const int32_t nt = std::max(0, std::min(SPLIT_LAUNCH_TILES, w[c].n_tiles - t0));
+      awgk::RenderArgs& ra = m.a[c];
+      ra.out_q = out + c;
+      ra.q_stride = n_channels;
+      if (nt > 0) launch_args(handles[c], w[c], t0, nt, i, &ra);
+      ra.pdl = i == 0 && last_setup >= 0 ? awgk::PDL_SETUP_FIRST : awgk::PDL_FREE;
+      ctas += (int64_t)nt * w[c].split;
+    }
+    const int32_t parts = render_parts(ctas, 1, sine);
+    for (int32_t c = 0; c < n_channels; ++c) {
+      m.a[c].parts = parts;
+      m.first[c + 1] = m.first[c] + m.a[c].n_tiles * parts * w[c].split;
+    }
+    const cudaError_t e = counted(handles[0], awgk::launch_render_mux(m, once, s));
+    if (e != cudaSuccess) return cuda_fail(e, "render launch");
+  }
+  for (int32_t c = 0; c < n_channels; ++c)
+    if ((st = window_done(handles[c], w[c], s))) return st;
   return AWG_OK;
 }
 
@@ -1280,7 +1341,7 @@ int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
   Window w;
   w.split = tone_list ? list_split : h->split;
   w.first = !engine_part;   // the engine's kernels came before
-  int st = window_plan(h, n, tone_list != nullptr, &w);
+  int st = window_plan(h, n, !tone_list, &w);
   if (!st) st = window_setup(h, &w, false, s);
   if (st) return st;
   awgk::RenderArgs ra;
@@ -2220,11 +2281,11 @@ int awg_render(awg_t* h, int64_t n, int16_t* out, void* stream) {
 }
 
 int awg_render_multiplexed(awg_t* const* handles, int32_t n_channels, int64_t n, int16_t* out, void* stream) {
-  if (!handles || n_channels < 1 || n_channels > 8) return fail(AWG_EINVAL, "need 1..8 channel handles");
+  if (!handles || n_channels < 1 || n_channels > awgk::MAX_CHANNELS) return fail(AWG_EINVAL, "need 1..8 channel handles");
   if (n < 0) return fail(AWG_EINVAL, "sample count must be >= 0");
   if (n == 0) return AWG_OK;
   if (!out) return fail(AWG_EINVAL, "null output");
-  int64_t cursors[8];
+  int64_t cursors[awgk::MAX_CHANNELS];
   for (int32_t c = 0; c < n_channels; ++c) {
     const awg_t* h = handles[c];
     if (!h) return fail(AWG_EINVAL, "null channel handle");
@@ -2235,9 +2296,6 @@ int awg_render_multiplexed(awg_t* const* handles, int32_t n_channels, int64_t n,
     if (h->cursor > INT64_MAX - n) return fail(AWG_EINVAL, "sample index overflow");
     cursors[c] = h->cursor;
   }
-  // Direct channels: every channel's set-up first, then the renders; the first render waits for the
-  // set-ups before the next may start, so the renders of all channels run side by side (each writes
-  // only after the one before has completed).
   bool together = n_channels > 1;
   for (int32_t c = 0; c < n_channels; ++c) {
     const awg_t* h = handles[c];
@@ -2245,27 +2303,7 @@ int awg_render_multiplexed(awg_t* const* handles, int32_t n_channels, int64_t n,
                !(h->periodic_start >= 0 && h->cursor + n > h->periodic_start);
   }
   if (together) {
-    cudaStream_t s = (cudaStream_t)stream;
-    Window w[8];
-    int st = AWG_OK;
-    for (int32_t c = 0; c < n_channels && !st; ++c) {
-      w[c].split = handles[c]->split;
-      w[c].first = true;
-      st = window_plan(handles[c], n, false, &w[c]);
-    }
-    int32_t last_setup = -1;   // the last channel with a set-up kernel
-    for (int32_t c = 0; c < n_channels && !st; ++c) {
-      w[c].beside = n_channels;
-      if (!w[c].active.empty()) last_setup = c;
-    }
-    for (int32_t c = 0; c < n_channels && !st; ++c) st = window_setup(handles[c], &w[c], c < last_setup, s);
-    for (int32_t c = 0; c < n_channels && !st; ++c) {
-      awgk::RenderArgs ra;
-      std::memset(&ra, 0, sizeof(ra));
-      ra.out_q = out + c;
-      ra.q_stride = n_channels;
-      st = window_render(handles[c], &w[c], ra, c == 0 && last_setup >= 0 ? awgk::PDL_SETUP_FIRST : awgk::PDL_FREE, s);
-    }
+    const int st = render_channels(handles, n_channels, n, out, (cudaStream_t)stream);
     if (st)
       for (int32_t c = 0; c < n_channels; ++c) handles[c]->cursor = cursors[c];
     return st;

@@ -212,6 +212,15 @@ struct RenderArgs {
 
 enum { PDL_NONE = 0, PDL_SETUP_FIRST = 1, PDL_SEQUENCE = 2, PDL_AFTER_SETUP = 3, PDL_FREE = 4 };
 
+// Several channels' renders in one launch (multiplexed channels): channel c takes CTAs first[c] ..
+// first[c + 1] - 1 of the grid.  The same parts, pdl and once on all channels.
+constexpr int MAX_CHANNELS = 8;
+struct MuxArgs {
+  RenderArgs a[MAX_CHANNELS];
+  int32_t first[MAX_CHANNELS + 1];
+  int32_t n;
+};
+
 struct PhaseArgs {
   const ToneRec* tones;
   const ChirpRec* chirps;
@@ -258,6 +267,7 @@ struct SiftArgs {
 };
 cudaError_t launch_sift(const SiftArgs& a, cudaStream_t s);
 cudaError_t launch_render(const RenderArgs& a, cudaStream_t s);
+cudaError_t launch_render_mux(const MuxArgs& m, bool once, cudaStream_t s);
 cudaError_t launch_replay(const int16_t* tab, int32_t log2_len, int64_t c, int64_t n, int16_t* out, int32_t stride,
                           unsigned long long* times, cudaStream_t s);   // times: start, end
 // x[i] = part[i] + base[i], i < n (in the order the render adds its engine sum): FP32 to out_f,

@@ -1586,6 +1586,19 @@ __global__ void __launch_bounds__(RT, SPT == RUN || MODE == MODE_ONCE ? AWG_REND
   render_tile<SPT, false, MODE>(a, blockIdx.x / a.split, blockIdx.x % a.split, a.split);
 }
 
+// All channels of a multiplexed render in one grid (the channels' arguments differ, so the kernel reads
+// them by channel; the loops are render_split_kernel's).
+template <int SPT, int MODE>
+__global__ void __launch_bounds__(RT, SPT == RUN || MODE == MODE_ONCE ? AWG_RENDER_SPLIT_MIN_BLOCKS : AWG_RENDER_PART_MIN_BLOCKS)
+    render_mux_kernel(const __grid_constant__ MuxArgs m) {
+  int c = 0;
+  while (c + 1 < m.n && (int)blockIdx.x >= m.first[c + 1]) ++c;
+  const RenderArgs& a = m.a[c];
+  const int i = (int)blockIdx.x - m.first[c];
+  if (a.start && i == 0 && threadIdx.x == 0) *a.start = global_ns();
+  render_tile<SPT, false, MODE>(a, i / a.split, i % a.split, a.split);
+}
+
 // Several renders in one grid (continuous batching): CTA group i (split CTAs) renders window tile
 // items[i].y of request items[i].x; every request of the launch has the same tone split.  The
 // split sums through each request's scratch (reqs[i].part and .tile_ctr, counters zero at
@@ -1717,6 +1730,13 @@ static SplitKernel split_kernel(int parts, int mode) {
          : mode == MODE_LIST ? split_kernel_of<MODE_LIST>(parts) : split_kernel_of<MODE_ALL>(parts);
 }
 
+typedef void (*MuxKernel)(const MuxArgs);
+static MuxKernel mux_kernel(int parts, bool once) {
+  if (once)
+    return parts == 4 ? render_mux_kernel<8, MODE_ONCE> : parts == 2 ? render_mux_kernel<16, MODE_ONCE> : render_mux_kernel<32, MODE_ONCE>;
+  return parts == 4 ? render_mux_kernel<8, MODE_ALL> : parts == 2 ? render_mux_kernel<16, MODE_ALL> : render_mux_kernel<32, MODE_ALL>;
+}
+
 cudaError_t render_setup_attributes() {
   cudaError_t e = cudaFuncSetAttribute(render_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   // shared memory before L1 for AWG_RENDER_SPLIT_MIN_BLOCKS CTAs
@@ -1724,6 +1744,10 @@ cudaError_t render_setup_attributes() {
     for (int mode = 0; mode < N_MODES; ++mode)
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute(split_kernel(parts, mode), cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  for (int parts = 1; parts <= MAX_PARTS; parts *= 2)
+    for (bool once : {false, true})
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(mux_kernel(parts, once), cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   return e;
 }
 
@@ -2000,6 +2024,11 @@ cudaError_t launch_sift(const SiftArgs& a, cudaStream_t s) {
   if (a.n_tiles == 0) return cudaSuccess;
   sift_kernel<<<(unsigned)a.n_tiles, 128, 0, s>>>(a);
   return cudaGetLastError();
+}
+
+cudaError_t launch_render_mux(const MuxArgs& m, bool once, cudaStream_t s) {
+  const PdlLaunch l((unsigned)m.first[m.n], RT, s);
+  return cudaLaunchKernelEx(&l.cfg, mux_kernel(m.a[0].parts, once), m);
 }
 
 cudaError_t launch_exact_table(const TableArgs& a, int64_t L, cudaStream_t s) {
