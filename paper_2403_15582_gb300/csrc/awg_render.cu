@@ -1038,33 +1038,30 @@ __device__ __forceinline__ bool f_vec_ok(const RenderArgs& a) {
   return !a.out_f || (((uintptr_t)a.out_f - 4u * (uint64_t)a.win_start) & 15u) == 0;
 }
 
-// Store the 8 samples n .. n + 7 (n a multiple of 8): one 16-byte vector of int16 codes (and two
-// of FP32 sums) when the group lies inside the window and the outputs are aligned, else sample
-// by sample.
-__device__ __forceinline__ void store_group(const RenderArgs& a, int64_t n, const float (&xv)[8], bool vec) {
-  if (vec && n >= a.win_start && n + 8 <= a.win_end) {
-    const int64_t o = n - a.win_start;
-    float x[8];
+// Store the 8 samples n .. n + 7 (n a multiple of 8) of a group inside the window, the outputs aligned:
+// one 16-byte vector of int16 codes and two of FP32 sums.
+__device__ __forceinline__ void store_group(const RenderArgs& a, int64_t n, const float (&xv)[8]) {
+  const int64_t o = n - a.win_start;
+  float x[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) x[u] = a.base ? xv[u] + a.base[o + u] : xv[u];
-    uint32_t w[4];
+  for (int u = 0; u < 8; ++u) x[u] = a.base ? xv[u] + a.base[o + u] : xv[u];
+  uint32_t w[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const float q0 = fminf(fmaxf(rintf(x[2 * u] * a.scale), -32767.f), 32767.f);
-      const float q1 = fminf(fmaxf(rintf(x[2 * u + 1] * a.scale), -32767.f), 32767.f);
-      w[u] = (uint32_t)(uint16_t)(int16_t)q0 | ((uint32_t)(uint16_t)(int16_t)q1 << 16);
-    }
-    if (a.out_q) *reinterpret_cast<uint4*>(a.out_q + o) = make_uint4(w[0], w[1], w[2], w[3]);
-    if (a.out_f) {
-      float4* f4 = reinterpret_cast<float4*>(a.out_f + o);
-      f4[0] = make_float4(x[0], x[1], x[2], x[3]);
-      f4[1] = make_float4(x[4], x[5], x[6], x[7]);
-    }
-    return;
+  for (int u = 0; u < 4; ++u) {
+    const float q0 = fminf(fmaxf(rintf(x[2 * u] * a.scale), -32767.f), 32767.f);
+    const float q1 = fminf(fmaxf(rintf(x[2 * u + 1] * a.scale), -32767.f), 32767.f);
+    w[u] = (uint32_t)(uint16_t)(int16_t)q0 | ((uint32_t)(uint16_t)(int16_t)q1 << 16);
   }
-#pragma unroll
-  for (int u = 0; u < 8; ++u) store_sample(a, n + u, xv[u]);
+  if (a.out_q) *reinterpret_cast<uint4*>(a.out_q + o) = make_uint4(w[0], w[1], w[2], w[3]);
+  if (a.out_f) {
+    float4* f4 = reinterpret_cast<float4*>(a.out_f + o);
+    f4[0] = make_float4(x[0], x[1], x[2], x[3]);
+    f4[1] = make_float4(x[4], x[5], x[6], x[7]);
+  }
 }
+
+// Samples of a part that go through shared memory at a time.
+constexpr int OUT_STAGE = 4096;
 
 // Sum over the split without clusters.  The thread holds samples at .. at + SPT - 1 of the part
 // in acc.  With split 1 it stores them; otherwise the CTA writes them to its partial part
@@ -1072,28 +1069,51 @@ __device__ __forceinline__ void store_group(const RenderArgs& a, int64_t n, cons
 // on a.tile_ctr[unit]; the CTA that brings the count to split - 1 (mod split) is the last of the
 // part: it sums the split's partials in rank order (as the cluster reduction does: the same FP32
 // sums) and stores the part, thread t taking the 8-sample groups t, t + RT, ... (coalesced
-// 16-byte stores).  The loads of several ranks are in flight at a time: one rank at a time left
-// the last CTA of a tile waiting for the L2 `split` times in a row (12 us at split 11).
+// 16-byte stores).  A part at the window's edge, an output off the vectors' alignment or with a stride
+// goes through s_out, OUT_STAGE samples at a time, so that a warp stores 32 consecutive samples; eight
+// by one thread, one after another, met a cache line per lane and store (80 tones x 1,000,001 samples
+// from sample 12345, FP32 and int16: 41.8 -> 18.6 us; eight multiplexed channels of 100 chirps x 50,001
+// 21.2 -> 18.7; two of 60 static tones x 2^20, at the stores' rate either way, 29.6 -> 30.4).
+// The loads of several ranks are in flight at a time: one rank at a time left the last CTA of a tile
+// waiting for the L2 `split` times in a row (12 us at split 11).
 // The preceding kernel of the stream is complete before the first write to global memory (in a
 // sequence: before the first write to the split scratch).
 template <int SPT>
 __device__ __forceinline__ void tile_epilogue_split(const RenderArgs& a, int unit, int crank, int split, int64_t P0,
-                                                    int at, const Acc<SPT>& acc) {
+                                                    int at, const Acc<SPT>& acc, float* s_out) {
   constexpr int PSAMP = Geo<SPT>::PSAMP;
   const int tid = threadIdx.x;
   __shared__ int s_last;
-  const bool vec = q_vec_ok(a) && f_vec_ok(a);
+  const bool vec = q_vec_ok(a) && f_vec_ok(a) && P0 >= a.win_start && P0 + PSAMP <= a.win_end;
+  auto store_out = [&](int64_t n0, int count) {   // s_out[0 .. count): samples n0 ..
+    __syncthreads();
+    for (int i = tid; i < count; i += RT) store_sample(a, n0 + i, s_out[i]);
+    __syncthreads();
+  };
   if (a.pdl != PDL_NONE && (a.pdl != PDL_SEQUENCE || split > 1)) pdl_wait();
   if (split == 1) {
+    if (vec) {
 #pragma unroll
-    for (int g = 0; g < SPT / 8; ++g) {
-      float xv[8];
+      for (int g = 0; g < SPT / 8; ++g) {
+        float xv[8];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        xv[2 * u] = 0.f + acc[4 * g + u].x;
-        xv[2 * u + 1] = 0.f + acc[4 * g + u].y;
+        for (int u = 0; u < 4; ++u) {
+          xv[2 * u] = 0.f + acc[4 * g + u].x;
+          xv[2 * u + 1] = 0.f + acc[4 * g + u].y;
+        }
+        store_group(a, P0 + at + 8 * g, xv);
       }
-      store_group(a, P0 + at + 8 * g, xv, vec);
+    } else {
+      __syncthreads();   // s_out is free
+      for (int b = 0; b < PSAMP; b += OUT_STAGE) {
+        if (at >= b && at < b + OUT_STAGE) {
+          float4* d = reinterpret_cast<float4*>(s_out + (at - b));
+#pragma unroll
+          for (int j = 0; j < SPT / 4; ++j)
+            d[j] = make_float4(0.f + acc[2 * j].x, 0.f + acc[2 * j].y, 0.f + acc[2 * j + 1].x, 0.f + acc[2 * j + 1].y);
+        }
+        store_out(P0 + b, PSAMP < OUT_STAGE ? PSAMP : OUT_STAGE);
+      }
     }
   } else {
     float4* dst = reinterpret_cast<float4*>(a.part + ((int64_t)unit * split + crank) * PSAMP + at);
@@ -1143,8 +1163,19 @@ __device__ __forceinline__ void tile_epilogue_split(const RenderArgs& a, int uni
               }
             }
         }
+        if (vec) {
 #pragma unroll
-        for (int v = 0; v < H; ++v) store_group(a, P0 + 8 * ((int64_t)tid + RT * (v0 + v)), xs[v], vec);
+          for (int v = 0; v < H; ++v) store_group(a, P0 + 8 * ((int64_t)tid + RT * (v0 + v)), xs[v]);
+        } else {
+          static_assert(8 * RT * H <= OUT_STAGE, "the groups summed at a time fit s_out");
+#pragma unroll
+          for (int v = 0; v < H; ++v) {
+            float4* d = reinterpret_cast<float4*>(s_out + 8 * (tid + RT * v));
+            d[0] = make_float4(xs[v][0], xs[v][1], xs[v][2], xs[v][3]);
+            d[1] = make_float4(xs[v][4], xs[v][5], xs[v][6], xs[v][7]);
+          }
+          store_out(P0 + 8 * RT * v0, 8 * RT * H);
+        }
       }
     }
   }
@@ -1175,12 +1206,25 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
   static_assert(!CLUSTER || SPT == RUN, "cluster sums take whole tiles");
   constexpr int NBUF = ONCE ? ONCE_TONES / STAGE : 2;   // stage buffers
   static_assert(!ONCE || NBUF <= RT / 32, "a warp prepares a stage");
-  __shared__ alignas(16) ToneRec s_tone[NBUF][STAGE];
-  __shared__ alignas(16) TileRec s_rec[NBUF][STAGE];
-  __shared__ alignas(16) Desc s_desc[NBUF][STAGE];
-  __shared__ uint8_t s_order[NBUF][STAGE];       // visit order
-  __shared__ uint8_t s_kind[NBUF][STAGE];        // kinds, in visit order
-  __shared__ int s_ngrp[NBUF][N_GRP];             // ends of the visit groups
+  // The stage buffers in one object: one base address and constant offsets.  As variables of their own
+  // (and with the output's stores not in a common loop) the 35 ms record took 2622 us, so 2524; one
+  // object per stage, with the descriptors in visit order, costs static tones more registers (1000
+  // tones x 2^19 118 against 113 us).  The epilogue stages the output in it.
+  struct StageBuf {
+    alignas(16) ToneRec tone[NBUF][STAGE];
+    alignas(16) TileRec rec[NBUF][STAGE];
+    alignas(16) Desc desc[NBUF][STAGE];
+    uint8_t order[NBUF][STAGE];
+    uint8_t kind[NBUF][STAGE];
+    int ngrp[NBUF][N_GRP];
+  };
+  __shared__ StageBuf s_buf;
+  auto& s_tone = s_buf.tone;
+  auto& s_rec = s_buf.rec;
+  auto& s_desc = s_buf.desc;
+  auto& s_order = s_buf.order;
+  auto& s_kind = s_buf.kind;
+  auto& s_ngrp = s_buf.ngrp;
   // cluster sums through distributed shared memory: [i][thread]
   __shared__ alignas(16) float s_red[CLUSTER ? TILE : 4];
   __shared__ alignas(8) uint64_t s_bar[4];        // tones[0], tones[1], records[0], records[1]
@@ -1526,7 +1570,9 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
   }
 
   if constexpr (!CLUSTER) {
-    tile_epilogue_split<SPT>(a, unit, crank, split, P0, (run - part * G::PRUNS) * RUN + (int)r0, acc);
+    static_assert(sizeof(StageBuf) >= OUT_STAGE * sizeof(float), "the stage buffers hold the staged samples");
+    tile_epilogue_split<SPT>(a, unit, crank, split, P0, (run - part * G::PRUNS) * RUN + (int)r0, acc,
+                             reinterpret_cast<float*>(&s_buf));
   } else {
     // partial sums -> shared memory ([i][thread], sample RUN thread + i), then the cluster-wide
     // sum in rank order
@@ -1564,8 +1610,8 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
   }
 }
 
-// Register budgets, by CTAs per SM.  Whole tiles: six (80 registers, 44 bytes of spill loads); the
-// 1000-chirp 35 ms record took 2636 us at six, 2703 at seven (72 registers), 2711 at five; the batched
+// Register budgets, by CTAs per SM.  Whole tiles: six (80 registers, 52 bytes of spill loads); the
+// 1000-chirp 35 ms record takes 2524 us at six, 2599 at seven (72 registers), 2587 at five; the batched
 // and cluster renders keep five (no spills).  Parts need fewer accumulators: eight, but six where the
 // CTA forms its records (at eight 1.2 KB of spills).  A kernel per mode: with the list's code in it the
 // plain render's registers change and the record takes 2640 instead of 2616 us.
