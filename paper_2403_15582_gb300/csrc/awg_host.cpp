@@ -584,6 +584,7 @@ struct awg {
   float* d_part = nullptr;
   unsigned long long* d_tctr = nullptr;
   int32_t part_tiles = 0, part_split = 0, ctr_split = 0;
+  int64_t ramp_end = 0;                // the end of the last amplitude ramp
   int64_t n_launches = 0;              // kernels this handle has launched
   int32_t* d_list = nullptr;           // tensor-core engine: tones not static in some tile of the window,
   size_t cap_list = 0;                 // then the same sifted per tile (RenderArgs::tile_first, the rows)
@@ -996,6 +997,7 @@ int set_tones_common(awg_t* h, const double* f, const double* amp, const double*
   h->K = n;
   h->flagged_ok = false;
   h->periodic_start = -1;
+  h->ramp_end = 0;
   h->chirps.clear();
   h->free_slots.clear();
   h->fs_explicit = false;
@@ -1081,22 +1083,28 @@ void prep_args(const awg_t* h, const std::vector<int32_t>& active, size_t b, int
   std::memcpy(pa->slots, active.data() + b, (size_t)pa->n_active * sizeof(int32_t));
 }
 
-// Parts a tile's samples are cut into (RenderArgs::parts) for work of `tiles` tiles.  A CTA is one
-// rank of one part; c of them land on the busiest SM.  Halves and quarters repeat the run set-ups (per
-// SM 0.56 and 0.36 of a whole tile's time instead of 0.5 and 0.25), so they pay only where whole
-// tiles leave SMs idle or unevenly loaded; the added constants are the SM's poorer rate with few
-// warps.  All from the chirp loop with set-ups, timed by CTAs per SM: 2.7, 3.6, 3.75 ... 4.03e12
-// sines/s at 1, 2, 3 ... 7 whole tiles per SM, 2.1, 3.0, 3.3 ... 3.6 for halves, 1.5, 2.2, 2.5 ... 2.8 for
-// quarters.  The rotator's runs cannot be entered in the middle: whole tiles.
-int32_t render_parts(int64_t tiles, int32_t split, int32_t sine_mode) {
+// Parts a tile's samples are cut into (RenderArgs::parts) for work of `tiles` tiles; every CTA of a tile
+// repeats its tones' run set-ups, so parts pay only where whole tiles leave the SMs without enough warps:
+// quarters up to 0.65 CTAs of whole tiles per SM, halves up to 1.5.  Where at most a quarter of the
+// tones chirp (few) halves go up to 2, and up to 4 where they even out a last row of whole tiles that is at
+// most half full (100 static tones x 256 tiles, 3.4 per SM: halves 24.3, whole tiles 25.2; 1000 x 38, 2.75
+// per SM: even; 6699 fast chirps x 28 tiles, 2.9 per SM: 465 against 346).  heavy: a part repeats more than that
+// (amplitude ramps; chirp records formed in the CTA): 0.25 and 0.62.  Back-to-back calls, us for whole
+// tiles / halves / quarters: 1000 static tones x 4 tiles (0.29 CTAs per SM) 12.7 / 9.6 / 7.3, x 8 (0.58)
+// 14.3 / 11.7 / 10.3, x 16 (1.2) 18.1 / 16.8 / 18.9, x 24 (1.7) 25.0 / 23.4 / 27.1, x 38 (2.75) 36.1 / 36.0 /
+// 42.3; 2000 chirps x 8 tiles (0.84) 53 / 46 / 44, x 12 (1.3) 67 / 55 / 58; heavy: 250 chirps x 8 tiles (0.16)
+// 9.5 / 7.1 / 6.3, x 16 (0.32) 10.2 / 8.0 / 9.6, x 24 (0.47) 10.7 / 10.3 / 12.9, x 38 (0.75) 13.3 / 14.6 / 19.9,
+// x 64 (1.3) 20.4 / 23.7 / 32.4; 500 ramps x 12 tiles (0.47) 19.5 / 17.0 / 20.3, x 24 (0.95) 25 / 28 / 37.
+// The rotator's runs cannot be entered in the middle: whole tiles.
+int32_t render_parts(int64_t tiles, int32_t split, int32_t sine_mode, bool heavy, bool few) {
   if (sine_mode == AWG_SINE_ROTATOR) return 1;
-  const int64_t sms = awgk::device_sm_count();
-  auto cost = [&](int32_t parts, double each, double more) {
-    return each * ((double)((tiles * split * parts + sms - 1) / sms) + more);
-  };
-  const double c1 = cost(1, 1.0, 0.5), c2 = cost(2, 0.56, 0.6), c4 = cost(4, 0.36, 0.9);
-  return c1 <= c2 && c1 <= c4 ? 1 : (c2 <= c4 ? 2 : 4);
+  const double per_sm = (double)(tiles * split) / (double)awgk::device_sm_count();
+  if (heavy) return per_sm <= 0.25 ? 4 : per_sm <= 0.62 ? 2 : 1;
+  const bool evens = per_sm <= 4.0 && std::ceil(2.0 * per_sm) < 2.0 * std::ceil(per_sm);
+  return per_sm <= 0.65 ? 4 : per_sm <= (few ? 2.0 : 1.5) || (few && evens) ? 2 : 1;
 }
+
+bool few_chirps(const awg_t* h, const std::vector<int32_t>& active) { return (int64_t)active.size() * 4 <= (int64_t)h->K; }
 
 int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream, int32_t q_stride,
                   bool engine_part, const int32_t* tone_list = nullptr, int32_t n_list = 0, int32_t list_split = 0,
@@ -1235,7 +1243,7 @@ int window_render(awg_t* h, Window* w, const awgk::RenderArgs& ra, int32_t pdl, 
     awgk::RenderArgs rs = ra;
     const int32_t nt = std::min(w->per_launch, w->n_tiles - t0);
     launch_args(h, *w, t0, nt, i, &rs);
-    rs.parts = render_parts(nt, w->split, h->sine_mode);
+    rs.parts = render_parts(nt, w->split, h->sine_mode, w->once || h->ramp_end > w->c, few_chirps(h, w->active));
     rs.pdl = pdl == awgk::PDL_NONE || pdl == awgk::PDL_FREE || w->n_tiles <= w->per_launch
                  ? pdl
                  : (i == 0 ? awgk::PDL_SETUP_FIRST : awgk::PDL_FREE);
@@ -1258,7 +1266,7 @@ int window_render(awg_t* h, Window* w, const awgk::RenderArgs& ra, int32_t pdl, 
 // come first.
 int render_channels(awg_t* const* handles, int32_t n_channels, int64_t n, int16_t* out, cudaStream_t s) {
   Window w[awgk::MAX_CHANNELS];
-  bool may_once = true, once = false;
+  bool may_once = true, once = false, ramps = false, few = true;
   int32_t sine = AWG_SINE_SFU, max_tiles = 0, last_setup = -1;
   for (int32_t c = 0; c < n_channels; ++c) {
     may_once = may_once && once_fits(handles[c], handles[c]->split);
@@ -1272,6 +1280,8 @@ int render_channels(awg_t* const* handles, int32_t n_channels, int64_t n, int16_
     once = once || w[c].once;
     if (!w[c].active.empty()) last_setup = c;
     max_tiles = std::max(max_tiles, w[c].n_tiles);
+    ramps = ramps || handles[c]->ramp_end > w[c].c;
+    few = few && few_chirps(handles[c], w[c].active);
   }
   for (int32_t c = 0; c < n_channels; ++c) {
     w[c].once = once;   // one kernel for all: a static channel's CTAs stage their tones likewise
@@ -1291,7 +1301,7 @@ int render_channels(awg_t* const* handles, int32_t n_channels, int64_t n, int16_
       ra.pdl = i == 0 && last_setup >= 0 ? awgk::PDL_SETUP_FIRST : awgk::PDL_FREE;
       ctas += (int64_t)nt * w[c].split;
     }
-    const int32_t parts = render_parts(ctas, 1, sine);
+    const int32_t parts = render_parts(ctas, 1, sine, once || ramps, few);
     for (int32_t c = 0; c < n_channels; ++c) {
       m.a[c].parts = parts;
       m.first[c + 1] = m.first[c] + m.a[c].n_tiles * parts * w[c].split;
@@ -1788,7 +1798,8 @@ int render_chunks_impl(awg_t* h, int64_t chunk, int32_t n_chunks, int16_t* out, 
     // a launch overlaps the next one (which waits for it before it reuses the scratch): two launches
     // fill the device together.  One form for the group: a change of kernel in mid-sequence costs
     // more than a better fit of the last launch gives (500 against 488 us for 1500 tones in 8 chunks)
-    const int32_t parts = render_parts(std::min<int64_t>(2 * ((chunk + awgk::TILE - 1) / awgk::TILE), n_tiles), h->split, h->sine_mode);
+    const int32_t parts = render_parts(std::min<int64_t>(2 * ((chunk + awgk::TILE - 1) / awgk::TILE), n_tiles), h->split, h->sine_mode,
+                                       h->ramp_end > c0 + (int64_t)g0 * chunk, few_chirps(h, active));
     for (int32_t c = g0; c < g1; ++c) {
       const int64_t wc = c0 + (int64_t)c * chunk, len = span(c, c + 1);
       const int64_t t_first = wc / awgk::TILE, t_last = (wc + len - 1) / awgk::TILE;
@@ -2149,6 +2160,7 @@ int awg_set_amp_ramps(awg_t* h, const int32_t* tone, const double* amp_end, cons
     h->flagged_ok = false;
     t.a_ns = start_sample[i];
     t.a_L = (int32_t)L[(size_t)i];
+    h->ramp_end = std::max(h->ramp_end, t.a_ns + t.a_L);
     t.A_end = (float)amp_end[i];
     t.flags = (t.flags & ~(awgk::TONE_AMP_RAMP | awgk::TONE_AMP_MINJERK)) | awgk::TONE_AMP_RAMP |
               (profile[i] == AWG_PROFILE_MINJERK ? awgk::TONE_AMP_MINJERK : 0);
