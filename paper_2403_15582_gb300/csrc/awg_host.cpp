@@ -777,6 +777,14 @@ class HostPool {
 // counters count every CTA of every launch, and a CTA is the last of its tile when its count is
 // split - 1 mod split; so they are zeroed when allocated and whenever the split changes.
 constexpr int32_t SPLIT_LAUNCH_TILES = 512;   // tiles per render launch when the split sums in scratch
+
+// Zero, and complete on return: the kernels that use the bytes run on streams that do not wait for the
+// default stream (the caller's, the engine's side stream).
+cudaError_t zero_now(awg_t* h, void* p, size_t bytes) {
+  const cudaError_t e = cudaMemsetAsync(p, 0, bytes, h->priv);
+  return e == cudaSuccess ? cudaStreamSynchronize(h->priv) : e;
+}
+
 int ensure_split_scratch(awg_t* h, int32_t tiles, int32_t split) {
   if (tiles <= h->part_tiles && split <= h->part_split && split == h->ctr_split) return AWG_OK;
   int st = wait_idle(h);
@@ -799,7 +807,7 @@ int ensure_split_scratch(awg_t* h, int32_t tiles, int32_t split) {
     h->part_tiles = nt;
     h->part_split = ns;
   }
-  if ((e = cudaMemset(h->d_tctr, 0, (size_t)2 * h->part_tiles * awgk::MAX_PARTS * sizeof(unsigned long long))) != cudaSuccess)
+  if ((e = zero_now(h, h->d_tctr, (size_t)2 * h->part_tiles * awgk::MAX_PARTS * sizeof(unsigned long long))) != cudaSuccess)
     return cuda_fail(e, "split counters");
   h->ctr_split = split;
   return AWG_OK;
@@ -1715,7 +1723,7 @@ int ensure_seq_counter(awg_t* h) {
   if (h->d_seq_exit) return AWG_OK;
   if (cudaMalloc((void**)&h->d_seq_exit, sizeof(unsigned long long)) != cudaSuccess)
     return fail(AWG_ENOMEM, "cudaMalloc sequence counter");
-  cudaError_t e = cudaMemset(h->d_seq_exit, 0, sizeof(unsigned long long));
+  cudaError_t e = zero_now(h, h->d_seq_exit, sizeof(unsigned long long));
   if (e != cudaSuccess) return cuda_fail(e, "sequence counter");
   return AWG_OK;
 }
@@ -1932,7 +1940,7 @@ awg_t* awg_create(double sample_rate_hz) {
   if (e == cudaSuccess) e = cudaMemset(h->d_status, 0, sizeof(int32_t));
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->priv, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_times, 2 * sizeof(unsigned long long));
-  if (e == cudaSuccess) e = cudaMemset(h->d_times, 0, 2 * sizeof(unsigned long long));
+  if (e == cudaSuccess) e = zero_now(h, h->d_times, 2 * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_done, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_upload, cudaEventDisableTiming);
   if (e != cudaSuccess) {

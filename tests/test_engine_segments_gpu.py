@@ -113,3 +113,33 @@ def test_groups_that_chirp_in_turn(awg, oracle, K, groups, aligned):
     for h in handles:
         assert h.device_status() == 0
         h.close()
+
+
+def test_first_call_of_a_handle_on_used_memory(awg):
+    """The split sums' counters are zero before the engine's side stream counts on them, also when the
+    memory held another split's counts and the caller's stream is busy."""
+    K, n = 700, 12000
+    rng = np.random.default_rng(5)
+    f, th = rng.uniform(80e6, 180e6, K), rng.uniform(0, 6.28, K)
+    busy = torch.empty(1 << 28, dtype=torch.float32, device="cuda")
+    for split_tones in (480, 200, 900):
+        old = awg.Synth(280e6)
+        old.set_tones(f[:split_tones] if split_tones < K else np.resize(f, split_tones), np.full(split_tones, 1e-3), np.zeros(split_tones))
+        x = torch.empty(n, dtype=torch.float32, device="cuda")
+        old.render_f32(n, x)
+        torch.cuda.synchronize()
+        old.close()
+        s = awg.Synth(280e6)
+        s.set_tones(f, np.full(K, 1.0 / K), th)
+        s.set_amp_ramps(np.arange(K), np.zeros(K), np.full(K, 1e-5), np.arange(K) % 2, rng.integers(0, n, K))
+        s.set_static_engine(awg.STATIC_GEMM_FP16)
+        first, again = torch.empty_like(x), torch.empty_like(x)
+        for _ in range(8):
+            busy.zero_()
+        s.render_f32(n, first)
+        torch.cuda.synchronize()
+        s.seek(0)
+        s.render_f32(n, again)
+        torch.cuda.synchronize()
+        assert torch.equal(first, again)
+        s.close()
