@@ -1144,7 +1144,7 @@ struct Window {
 
 // A window with chirps and at most 96 tones per CTA (1536 tones) goes without a set-up kernel: each CTA
 // takes all its tones at once and forms their chirp records itself.  A call then has one kernel, which
-// may run beside the end of the one before: 1000 chirps x 2^18 samples 96 -> 71 us among others (the
+// may run beside the end of the one before: 1000 chirps x 2^18 samples 96 -> 67 us among others (the
 // set-up alone 13 us, and the render waits for it).  Not in chunk sequences, where one set-up kernel
 // serves all chunks and the records cost less there than in the render's CTAs (35 ms record 2611
 // against 2722 us), not without chirps (100 static tones 25.2 against 26.2 us), and not with more
@@ -1268,8 +1268,9 @@ int window_render(awg_t* h, Window* w, const awgk::RenderArgs& ra, int32_t pdl, 
 
 // Several channels' direct renders, interleaved into out.  The launches take all channels (at most
 // SPLIT_LAUNCH_TILES tiles of each): launches of their own would each wait, before their sums and stores,
-// for the channel before to complete (eight channels of 100 chirps x 50,001 samples 89 -> 21 us, two of
-// 250 static tones x 2^18 47 -> 29, three of 900 tones x 10^6 640 -> 629, four of 250 chirps x 2^18 97 -> 97).
+// for the channel before to complete (eight channels of 100 chirps x 50,001 samples 89 -> 17 us, two of
+// 250 static tones x 2^18 47 -> 30, three of 900 tones x 10^6 640 -> 629, four of 250 chirps x 2^18 97 -> 72,
+// the last with parts counted over all channels).
 // Each CTA forms its chirp records itself where it may on every channel; otherwise all channels' set-ups
 // come first.
 int render_channels(awg_t* const* handles, int32_t n_channels, int64_t n, int16_t* out, cudaStream_t s) {
@@ -1553,7 +1554,7 @@ int render_engine(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
     // for a render CTA, and a window's GEMM often leaves SMs idle (128 CTAs for 2^20 samples on 152).
     // The set-up runs beside the operand's; the render starts once the operand is made, so that the
     // GEMM's CTAs (one per SM, nearly all of its shared memory) are placed first.  10,000 tones x
-    // 2^20, 400 of them chirping in turn: 300 us one after the other, 214 us side by side.
+    // 2^20, 400 of them chirping in turn: 300 us one after the other, 208 us side by side.
     if ((e = cudaStreamWaitEvent(h->side, h->ev_fork, 0)) != cudaSuccess) return cuda_fail(e, "engine ordering");
     if (use_list && n_list > 0 &&
         (e = cudaMemcpyAsync(h->d_list, h->list.data(), (size_t)n_list * sizeof(int32_t), cudaMemcpyHostToDevice,
