@@ -593,6 +593,7 @@ struct awg {
   // rebuilt on demand after tones, chirps or ramps change
   std::vector<int32_t> flagged;
   double amax = 0;                     // largest |amplitude| (ramp targets included), with `flagged`
+  int64_t full0 = 0, full1 = -1;       // RenderArgs::full0, full1, with `flagged`
   bool flagged_ok = false;
   // periodic hand-off: from sample periodic_start on, x[n] = periodic table[n mod 2^periodic_log2]
   int16_t* d_periodic = nullptr;
@@ -1369,6 +1370,8 @@ int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
   ra.out_f = out_f;
   ra.q_stride = q_stride;
   ra.skip_static = engine_part;   // the tones that are static in a tile go through the GEMM
+  ra.full0 = h->full0;            // (current since engine_split)
+  ra.full1 = h->full1;
   ra.tone_list = tone_list;
   ra.n_list = n_list;
   if (tone_list) {
@@ -1426,6 +1429,12 @@ const std::vector<int32_t>& flagged_tones(awg_t* h) {
     h->flagged.clear();
     for (size_t k = 0; k < h->tones.size(); ++k)
       if (h->tones[k].slot >= 0 || (h->tones[k].flags & awgk::TONE_AMP_RAMP)) h->flagged.push_back((int32_t)k);
+    h->full0 = 0;
+    h->full1 = h->tones.empty() ? -1 : INT64_MAX;
+    for (const ToneRec& t : h->tones) {   // (a chirp's tiles: those its samples n_s .. n_e meet)
+      h->full0 = std::max(h->full0, t.slot >= 0 ? t.n_s / awgk::TILE * awgk::TILE : 0);
+      h->full1 = std::min(h->full1, t.slot >= 0 ? t.n_e / awgk::TILE * awgk::TILE : -1);
+    }
     h->flagged_ok = true;
   }
   return h->flagged;
@@ -1644,6 +1653,8 @@ int awgk::prepare_render_engine(awg_t* h, int64_t n, int16_t* out_q, cudaStream_
   }
   ra->base = base;
   ra->skip_static = 1;
+  ra->full0 = h->full0;
+  ra->full1 = h->full1;
   ra->tone_list = use_list ? d_list : nullptr;
   ra->n_list = n_list;
   ra->split = es.split;

@@ -189,6 +189,8 @@ struct RenderArgs {
   // (their sum comes from the table GEMM) and base[n - win_start] is added before quantising
   const float* base;
   int32_t skip_static;
+  int64_t full0, full1;   // with skip_static: first samples of the first and the last tile in which every
+                          // tone chirps (full1 < full0: none); such a tile is never rendered by a list
   // tones to visit (sorted, n_list of them; null: all K): CTA crank of a tile takes the listed
   // tones of [bounds[crank], bounds[crank + 1]) in ascending order (bounds[0] = 0,
   // bounds[split] = K); without a list it takes all of [K crank / split, K (crank + 1) / split)
