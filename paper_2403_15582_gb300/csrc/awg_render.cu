@@ -607,7 +607,7 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // keeps the second from starting before the first has ended: 6.6 us between kernels with the
 // events, 2.3 without, none with the kernels overlapping.
 __device__ __forceinline__ void mark_start(unsigned long long* t) {
-  if (t && blockIdx.x == 0 && threadIdx.x == 0) *t = global_ns();
+  if (t && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *t = global_ns();   // (the replay's grid has rows)
 }
 __device__ __forceinline__ void mark_end(unsigned long long* t) {
   if (t && threadIdx.x == 0) atomicMax(t, (unsigned long long)global_ns());
