@@ -1115,10 +1115,11 @@ int32_t render_parts(int64_t tiles, int32_t split, int32_t sine_mode, bool heavy
 
 bool few_chirps(const awg_t* h, const std::vector<int32_t>& active) { return (int64_t)active.size() * 4 <= (int64_t)h->K; }
 
-int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream, int32_t q_stride,
+// first: the call's first kernels are these (they write the device time of its start)
+int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream, int32_t q_stride, bool first,
                   bool engine_part, const int32_t* tone_list = nullptr, int32_t n_list = 0, int32_t list_split = 0,
                   const int32_t* list_bounds = nullptr);
-int render_engine(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream, int32_t q_stride);
+int render_engine(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream, int32_t q_stride, bool first);
 
 constexpr size_t SIFT_BUDGET = (size_t)1 << 24;   // entries of the sifted lists (64 MiB); longer ones go unsifted
 // Entries of the list buffer of a window of n_tiles tiles: the list, its sifted rows and their rank bounds.
@@ -1324,14 +1325,14 @@ int render_channels(awg_t* const* handles, int32_t n_channels, int64_t n, int16_
   return AWG_OK;
 }
 
-int render_impl(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream, int32_t q_stride = 1) {
+int render_impl(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream, int32_t q_stride = 1, bool first = true) {
   if (h && h->static_engine != AWG_STATIC_DIRECT && n > 0 && (out_f || out_q) &&
       !(h->periodic_start >= 0 && !out_f && h->cursor + n > h->periodic_start))
-    return render_engine(h, n, out_f, out_q, stream, q_stride);
-  return render_direct(h, n, out_f, out_q, stream, q_stride, false);
+    return render_engine(h, n, out_f, out_q, stream, q_stride, first);
+  return render_direct(h, n, out_f, out_q, stream, q_stride, first, false);
 }
 
-int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream, int32_t q_stride,
+int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream, int32_t q_stride, bool first,
                   bool engine_part, const int32_t* tone_list, int32_t n_list, int32_t list_split,
                   const int32_t* list_bounds) {
   if (!h) return fail(AWG_EINVAL, "null handle");
@@ -1344,13 +1345,13 @@ int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
     // periodic hand-off: render up to the start of the periodic part, replay the table after it
     const int64_t n1 = std::max<int64_t>(0, h->periodic_start - h->cursor);
     if (n1 > 0) {
-      const int st = render_impl(h, n1, nullptr, out_q, stream, q_stride);
+      const int st = render_impl(h, n1, nullptr, out_q, stream, q_stride, first);
       if (st) return st;
     }
     const int64_t c = h->cursor, n2 = n - n1;
     cudaError_t e;
     if ((e = counted(h, awgk::launch_replay(h->d_periodic, h->periodic_log2, c, n2, out_q + (size_t)n1 * (size_t)q_stride,
-                                 q_stride, h->d_times, s))) != cudaSuccess)
+                                 q_stride, first && n1 == 0 ? h->d_times : nullptr, h->d_times + 1, s))) != cudaSuccess)
       return cuda_fail(e, "replay launch");
     if ((e = cudaEventRecord(h->ev_done, s)) != cudaSuccess) return cuda_fail(e, "event");
     h->timed = true;
@@ -1360,7 +1361,7 @@ int render_direct(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
   }
   Window w;
   w.split = tone_list ? list_split : h->split;
-  w.first = !engine_part;   // the engine's kernels came before
+  w.first = first && !engine_part;   // the engine's kernels came before
   int st = window_plan(h, n, !tone_list, &w);
   if (!st) st = window_setup(h, &w, false, s);
   if (st) return st;
@@ -1490,16 +1491,17 @@ awgk::TableArgs2 engine_gemm_args(awg_t* h, int64_t c, int64_t m, bool two_segme
   t.scale = h->full_scale > 0 ? (float)(32767.0 / h->full_scale) : 0.f;
   t.a_scale = awgk::table_amp_scale(max_amplitude(h));
   t.status = h->d_status;
-  t.times = h->d_times;
+  t.end = h->d_times + 1;
   return t;
 }
 
 // B operand of the handle's GEMM (cos, sin of 2 pi n2 F / 2^64 per tone and segment, hi + lo).
-int engine_operand(awg_t* h, bool two_segments, cudaStream_t s) {
+int engine_operand(awg_t* h, bool two_segments, bool first, cudaStream_t s) {
   const size_t Kp = two_segments ? awgk::table_kp_window(std::max(h->K, 1)) : awgk::table_kp(std::max(h->K, 1));
   int st = ensure(&h->d_gemm, &h->cap_gemm, 2 * (size_t)256 * Kp, h, "table GEMM operands");
   if (st) return st;
-  const awgk::TableArgs2 t = engine_gemm_args(h, h->cursor, awgk::TILE, two_segments, nullptr, nullptr);
+  awgk::TableArgs2 t = engine_gemm_args(h, h->cursor, awgk::TILE, two_segments, nullptr, nullptr);
+  t.start = first ? h->d_times : nullptr;
   cudaError_t e;
   if ((e = counted(h, awgk::launch_table_prep(t, s))) != cudaSuccess) return cuda_fail(e, "static operand launch");
   return AWG_OK;
@@ -1516,7 +1518,7 @@ int ensure_side_stream(awg_t* h) {
   return AWG_OK;
 }
 
-int render_engine(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream, int32_t q_stride) {
+int render_engine(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream, int32_t q_stride, bool first) {
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t PIECE = (int64_t)1 << 26;
   const EngineSplit es = engine_split(h);
@@ -1531,7 +1533,7 @@ int render_engine(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
     float* of = out_f ? out_f + off : nullptr;
     int st;
     if (h->K == 0) {
-      if ((st = render_direct(h, m, of, oq, stream, q_stride, false))) return st;
+      if ((st = render_direct(h, m, of, oq, stream, q_stride, first && off == 0, false))) return st;
       continue;
     }
     // (a list of all K tones is left out: one bulk copy per stage instead of one per tone)
@@ -1548,7 +1550,7 @@ int render_engine(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
     cudaError_t e;
     if ((e = order_after_uploads(h, s)) != cudaSuccess) return cuda_fail(e, "upload ordering");
     if (!all_static && (e = cudaEventRecord(h->ev_fork, s)) != cudaSuccess) return cuda_fail(e, "event");
-    if ((st = engine_operand(h, two_segments, s))) return st;
+    if ((st = engine_operand(h, two_segments, first && off == 0, s))) return st;
     if (!all_static && (e = cudaEventRecord(h->ev_operand, s)) != cudaSuccess) return cuda_fail(e, "event");
     const awgk::TableArgs2 t = engine_gemm_args(h, c, m, two_segments, all_static ? oq : nullptr, all_static ? of : h->d_base);
     if ((e = counted(h, awgk::launch_table_gemm(t, s))) != cudaSuccess) return cuda_fail(e, "static GEMM launch");
@@ -1569,7 +1571,7 @@ int render_engine(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
         (e = cudaMemcpyAsync(h->d_list, h->list.data(), (size_t)n_list * sizeof(int32_t), cudaMemcpyHostToDevice,
                              h->side)) != cudaSuccess)
       return cuda_fail(e, "tone list upload");
-    st = render_direct(h, m, d_live, nullptr, h->side, 1, true, use_list ? h->d_list : nullptr, n_list, es.split, es.bounds);
+    st = render_direct(h, m, d_live, nullptr, h->side, 1, false, true, use_list ? h->d_list : nullptr, n_list, es.split, es.bounds);
     // whatever was queued on the side stream is joined, so that later calls come after it
     e = cudaEventRecord(h->ev_join, h->side);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, h->ev_join, 0);
@@ -1604,7 +1606,7 @@ int awgk::engine_setup(awg_t* h, int32_t engine, cudaStream_t s, int32_t* render
   const EngineSplit es = engine_split(h);
   cudaError_t e = order_after_uploads(h, s);
   if (e != cudaSuccess) return cuda_fail(e, "upload ordering");
-  const int st = engine_operand(h, es.n_flagged > 0, s);
+  const int st = engine_operand(h, es.n_flagged > 0, false, s);
   if (st) return st;
   if (render_split) *render_split = es.split;
   return AWG_OK;
@@ -2367,7 +2369,7 @@ int awg_render_chunks(awg_t* h, int64_t chunk, int32_t n_chunks, int16_t* out, v
     // a periodic tail is replayed per chunk; chunks above SPLIT_LAUNCH_TILES tiles go out in
     // several launches each (a pipelined sequence records its profiling events itself)
     for (int32_t c = 0; c < n_chunks; ++c) {
-      const int st = render_impl(h, chunk, nullptr, out + (size_t)c * (size_t)chunk, stream);
+      const int st = render_impl(h, chunk, nullptr, out + (size_t)c * (size_t)chunk, stream, 1, c == 0);
       if (st) return st;
     }
     return AWG_OK;
@@ -2390,7 +2392,7 @@ int awg_render_stream(awg_t* h, int64_t n, int64_t chunk, int16_t* out, void* st
   if (full + (tail > 0 ? 1 : 0) <= 1 || h->periodic_start >= 0 || h->static_engine != AWG_STATIC_DIRECT ||
       (h->split > 1 && chunk / awgk::TILE + 2 > SPLIT_LAUNCH_TILES)) {
     for (int64_t c = 0; c < n; c += chunk) {
-      const int st = render_impl(h, std::min(chunk, n - c), nullptr, out + c, stream);
+      const int st = render_impl(h, std::min(chunk, n - c), nullptr, out + c, stream, 1, c == 0);
       if (st) return st;
     }
     return AWG_OK;
@@ -2524,7 +2526,8 @@ int awg_table_gemm(awg_t* h, int32_t log2_len, int32_t precision, int16_t* out_q
   t.scale = h->full_scale > 0 ? (float)(32767.0 / h->full_scale) : 0.f;
   t.a_scale = awgk::table_amp_scale(max_amplitude(h));
   t.status = h->d_status;
-  t.times = h->d_times;
+  t.start = h->d_times;
+  t.end = h->d_times + 1;
   cudaStream_t s = (cudaStream_t)stream;
   cudaEvent_t pe[4] = {nullptr, nullptr, nullptr, nullptr};
   cudaError_t e = cudaSuccess;

@@ -271,7 +271,7 @@ cudaError_t launch_sift(const SiftArgs& a, cudaStream_t s);
 cudaError_t launch_render(const RenderArgs& a, cudaStream_t s);
 cudaError_t launch_render_mux(const MuxArgs& m, bool once, cudaStream_t s);
 cudaError_t launch_replay(const int16_t* tab, int32_t log2_len, int64_t c, int64_t n, int16_t* out, int32_t stride,
-                          unsigned long long* times, cudaStream_t s);   // times: start, end
+                          unsigned long long* start, unsigned long long* end, cudaStream_t s);   // device times
 // x[i] = part[i] + base[i], i < n (in the order the render adds its engine sum): FP32 to out_f,
 // scaled, rounded and clamped codes to out_q[i * q_stride] (either may be null).
 cudaError_t launch_combine(const float* part, const float* base, int64_t n, float scale, int16_t* out_q, int32_t q_stride,
@@ -326,7 +326,7 @@ struct TableArgs2 {
   // the epilogue
   float a_scale;
   int32_t* status;
-  unsigned long long* times;   // device time of the call's start and end (null: not taken)
+  unsigned long long *start, *end;   // device time of the call's start and end (null: not taken)
 };
 // a_scale for amplitudes whose largest magnitude is amax (1 for amax 0)
 float table_amp_scale(double amax);

@@ -1861,13 +1861,14 @@ cudaError_t launch_prep(const PrepArgs& a, cudaStream_t s) {
 // Replay of a periodic record of 2^log2 samples, written at a stride (multiplexed channels):
 // out[i * stride] = table[(c + i) mod period].
 __global__ void replay_strided_kernel(const int16_t* __restrict__ tab, uint64_t mask, int64_t c, int64_t n,
-                                      int16_t* __restrict__ out, int32_t stride, unsigned long long* times) {
-  mark_start(times);
+                                      int16_t* __restrict__ out, int32_t stride, unsigned long long* start,
+                                      unsigned long long* end) {
+  mark_start(start);
   pdl_wait();
   const int64_t step = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += step)
     out[i * stride] = tab[((uint64_t)c + (uint64_t)i) & mask];
-  mark_end(times + 1);
+  mark_end(end);
 }
 
 // The same for a plain output, bound by the samples written (2 bytes each).  `out` is the first 16-byte
@@ -1879,8 +1880,9 @@ __global__ void replay_strided_kernel(const int16_t* __restrict__ tab, uint64_t 
 // table in the L2.  Samples before `out` and after its last whole vector are copied one by one.
 constexpr int REPLAY_VEC = 2, REPLAY_REPS = 8;
 __global__ void __launch_bounds__(256) replay_kernel(const int16_t* __restrict__ tab, uint64_t mask, int64_t c, int64_t n,
-                                                     int16_t* __restrict__ out, int head, unsigned long long* times) {
-  mark_start(times);
+                                                     int16_t* __restrict__ out, int head, unsigned long long* start,
+                                                     unsigned long long* end) {
+  mark_start(start);
   const uint64_t P = (mask + 1) >> 3;
   const int64_t nv = (n - head) >> 3;
   const uint64_t c1 = (uint64_t)c + (uint64_t)head, v0 = c1 >> 3;
@@ -1930,23 +1932,23 @@ __global__ void __launch_bounds__(256) replay_kernel(const int16_t* __restrict__
     if (t < head) out[t - head] = tab[((uint64_t)c + (uint64_t)t) & mask];
     else if (t >= 8 && t - 8 < tail) out[8 * nv + t - 8] = tab[(c1 + 8 * (uint64_t)nv + (uint64_t)(t - 8)) & mask];
   }
-  mark_end(times + 1);
+  mark_end(end);
 }
 
 cudaError_t launch_replay(const int16_t* tab, int32_t log2_len, int64_t c, int64_t n, int16_t* out, int32_t stride,
-                          unsigned long long* times, cudaStream_t s) {
+                          unsigned long long* start, unsigned long long* end, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const uint64_t mask = ((uint64_t)1 << log2_len) - 1;
   if (stride != 1) {
     const int64_t blocks = std::min<int64_t>((n + 255) / 256, (int64_t)device_sm_count() * 16);
     const PdlLaunch l((unsigned)blocks, 256, s);
-    return cudaLaunchKernelEx(&l.cfg, replay_strided_kernel, tab, mask, c, n, out, stride, times);
+    return cudaLaunchKernelEx(&l.cfg, replay_strided_kernel, tab, mask, c, n, out, stride, start, end);
   }
   const int head = (int)std::min<int64_t>(n, (int64_t)((16 - ((uintptr_t)out & 15)) & 15) / 2);
   const int64_t P = (int64_t)(mask + 1) / 8, nv = (n - head) / 8, span = std::max<int64_t>(1, std::min(P, nv));
   PdlLaunch l((unsigned)((span + 256 * REPLAY_VEC - 1) / (256 * REPLAY_VEC)), 256, s);
   l.cfg.gridDim.y = (unsigned)std::max<int64_t>(1, std::min<int64_t>(65535, (nv + P * REPLAY_REPS - 1) / (P * REPLAY_REPS)));
-  return cudaLaunchKernelEx(&l.cfg, replay_kernel, tab, mask, c, n, out + head, head, times);
+  return cudaLaunchKernelEx(&l.cfg, replay_kernel, tab, mask, c, n, out + head, head, start, end);
 }
 
 // The tensor-core engine's two sums of a window, formed side by side (awg_host.cpp, render_engine):

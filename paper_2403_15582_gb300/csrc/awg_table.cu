@@ -584,7 +584,7 @@ cudaError_t launch_table_prep(const TableArgs2& t, cudaStream_t s) {
   const dim3 grid((unsigned)((per_row + 127) / 128), TN / PREP_ROWS);
   auto kern = t.window_mode ? (t.precision == 0 ? prep_b_kernel<__nv_bfloat16, true> : prep_b_kernel<__half, true>)
                             : (t.precision == 0 ? prep_b_kernel<__nv_bfloat16, false> : prep_b_kernel<__half, false>);
-  kern<<<grid, 128, 0, s>>>(t.tones, t.K, Kp, (uint32_t*)t.b_hi, (uint32_t*)t.b_lo, t.times);
+  kern<<<grid, 128, 0, s>>>(t.tones, t.K, Kp, (uint32_t*)t.b_hi, (uint32_t*)t.b_lo, t.start);
   return cudaGetLastError();
 }
 
@@ -621,7 +621,7 @@ cudaError_t launch_table_gemm(const TableArgs2& t, cudaStream_t s) {
   ga.window_mode = t.window_mode;
   ga.a_scale = t.a_scale > 0.f ? t.a_scale : 1.f;
   ga.inv_a_scale = 1.f / ga.a_scale;
-  ga.end = t.times ? t.times + 1 : nullptr;
+  ga.end = t.end;
   // instruction descriptor: FP32 accumulate, A/B BF16 (1) or FP16 (0), both K-major, N/8, M/16
   const uint32_t fmt = bf16 ? 1u : 0u;
   ga.idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);

@@ -36,3 +36,36 @@ def test_replay_of_many_periods(awglib):
     ms, ev = _times(s, lambda: s.render(n, out))
     assert 0.7 * ev < ms < 1.1 * ev, (ms, ev)
     s.close()
+
+
+def test_hand_off(awglib):
+    """The rendered part before the periodic one counts."""
+    s = _grid_synth(awglib, 1000, 16)
+    f = FS / 65536 * (20000 + np.arange(1000))
+    s.set_tones(f, np.full(1000, 1e-3), np.zeros(1000), grid_log2=16)
+    s.set_chirps(np.arange(1000), f, f[::-1].copy(), np.full(1000, 5e-3), np.arange(1000) % 2, np.zeros(1000, dtype=np.int64))
+    s.set_periodic(16, awglib.PERIODIC_DIRECT)
+    n = s.periodic_start + 5000
+    out = torch.empty(n, dtype=torch.int16, device="cuda")
+    for call in (lambda: s.render(n, out), lambda: s.render_stream(n, 1 << 18, out), lambda: s.render_chunks(n // 5, 5, out)):
+        ms, ev = _times(s, call)
+        assert 0.7 * ev < ms < 1.1 * ev, (ms, ev)
+    s.close()
+
+
+@pytest.mark.parametrize("chirps", [0, 20])
+def test_engine_pieces(awglib, chirps):
+    """A window of more samples than the engine takes at a time."""
+    K = 64
+    f = np.linspace(80e6, 180e6, K)
+    s = awglib.Synth(FS)
+    s.set_tones(f, np.full(K, 1.0 / K), np.zeros(K))
+    if chirps:
+        s.set_chirps(np.arange(chirps), f[:chirps], f[:chirps] + 1e6, np.full(chirps, 1e-3), np.zeros(chirps, dtype=np.int64),
+                     np.zeros(chirps, dtype=np.int64))
+    s.set_static_engine(awglib.STATIC_GEMM_FP16)
+    n = (1 << 26) + 5000
+    out = torch.empty(n, dtype=torch.int16, device="cuda")
+    ms, ev = _times(s, lambda: s.render(n, out))
+    assert 0.7 * ev < ms < 1.1 * ev, (ms, ev)
+    s.close()
