@@ -1847,8 +1847,7 @@ int render_chunks_impl(awg_t* h, int64_t chunk, int32_t n_chunks, int16_t* out, 
       std::memcpy(ra.inv_odd, h->inv_odd, sizeof(ra.inv_odd));
       ra.parts = parts;
       ra.pdl = c == g0 ? awgk::PDL_SETUP_FIRST : awgk::PDL_SEQUENCE;
-      ra.start = c == 0 && active.empty() ? h->d_times : nullptr;
-      ra.end = h->d_times + 1;
+      ra.start = c == 0 && active.empty() ? h->d_times : nullptr;   // (the end is the join's)
       ra.exit_ctr = h->d_seq_exit;
       if (h->split > 1) {   // alternating scratch (see tile_epilogue_split)
         ra.part = split_part(h, c & 1);
@@ -1857,8 +1856,8 @@ int render_chunks_impl(awg_t* h, int64_t chunk, int32_t n_chunks, int16_t* out, 
       if ((e = counted(h, awgk::launch_render(ra, s))) != cudaSuccess) return cuda_fail(e, "render launch");
       h->seq_exit_target += (unsigned long long)ra.n_tiles * (unsigned long long)(ra.parts * h->split);
     }
-    if ((e = counted(h, awgk::launch_join(h->d_seq_exit, h->seq_exit_target, h->d_status, awgk::JOIN_LIMIT_NS, s))) !=
-        cudaSuccess)
+    if ((e = counted(h, awgk::launch_join(h->d_seq_exit, h->seq_exit_target, h->d_status, awgk::JOIN_LIMIT_NS,
+                                          h->d_times + 1, s))) != cudaSuccess)
       return cuda_fail(e, "join launch");
   }
   if (pe[3]) {
@@ -2685,7 +2684,7 @@ int awg_test_wait_timeout(awg_t* h, int64_t limit_us, void* stream) {
   // one above the running total of every sequence issued so far: no render CTA brings the counter
   // there, so the wait runs out
   cudaError_t e = counted(h, awgk::launch_join(h->d_seq_exit, h->seq_exit_target + 1, h->d_status,
-                                               (uint64_t)limit_us * 1000ull, (cudaStream_t)stream));
+                                               (uint64_t)limit_us * 1000ull, nullptr, (cudaStream_t)stream));
   if (e != cudaSuccess) return cuda_fail(e, "join launch");
   return AWG_OK;
 }

@@ -184,7 +184,8 @@ struct RenderArgs {
   // are stored.
   int32_t pdl;
   unsigned long long* exit_ctr;
-  unsigned long long *start, *end;   // device time of the call's start (first kernel) and end (every CTA)
+  unsigned long long *start, *end;   // device time of the call's start (first kernel) and end (every CTA;
+                                     // null in sequences, whose join writes it)
   // tensor-core static engine (otherwise null / 0): tones static over the window are skipped here
   // (their sum comes from the table GEMM) and base[n - win_start] is added before quantising
   const float* base;
@@ -280,7 +281,7 @@ cudaError_t launch_combine(const float* part, const float* base, int64_t n, floa
 // the status word becomes AWG_ETIMEOUT and the kernel returns.
 constexpr uint64_t JOIN_LIMIT_NS = 2000000000ull;
 cudaError_t launch_join(const unsigned long long* exit_ctr, unsigned long long target, int32_t* status,
-                        uint64_t limit_ns, cudaStream_t s);
+                        uint64_t limit_ns, unsigned long long* end, cudaStream_t s);   // end: RenderArgs::end, of the sequence
 // items[i] = (request index into reqs, window tile); every request has split == `split`.
 // Several renders in one launch (tiles items[i] = (request, tile) of the requests reqs[]; all of
 // tone split `split`); every request carries split scratch (part, tile_ctr with n_tiles zeroed

@@ -2004,16 +2004,18 @@ cudaError_t launch_combine(const float* part, const float* base, int64_t n, floa
 
 // End of a pipelined sequence: returns once every render CTA of the sequence has stored its
 // samples (*exit_ctr >= target), so that later work in the stream sees all of them.  Gives up after
-// limit_ns, sets the status word to AWG_ETIMEOUT and returns.
+// limit_ns, sets the status word to AWG_ETIMEOUT and returns.  The end of the call's device time is the
+// join's: a CTA that has counted itself in may still be on its way to a stamp of its own.
 __global__ void join_kernel(const unsigned long long* exit_ctr, unsigned long long target, int32_t* status,
-                            uint64_t limit_ns) {
+                            uint64_t limit_ns, unsigned long long* end) {
   if (!wait_counter(exit_ctr, target, limit_ns)) atomicExch(status, STATUS_TIMEOUT);
   __threadfence();
+  mark_end(end);
 }
 
 cudaError_t launch_join(const unsigned long long* exit_ctr, unsigned long long target, int32_t* status,
-                        uint64_t limit_ns, cudaStream_t s) {
-  join_kernel<<<1, 1, 0, s>>>(exit_ctr, target, status, limit_ns);
+                        uint64_t limit_ns, unsigned long long* end, cudaStream_t s) {
+  join_kernel<<<1, 1, 0, s>>>(exit_ctr, target, status, limit_ns, end);
   return cudaGetLastError();
 }
 

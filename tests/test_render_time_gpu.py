@@ -53,6 +53,21 @@ def test_hand_off(awglib):
     s.close()
 
 
+@pytest.mark.parametrize("K,chirps,chunk", [(1000, 1000, 1 << 18), (60, 0, 1 << 16), (2000, 100, 1 << 17)])
+def test_sequence(awglib, K, chirps, chunk):
+    s = awglib.Synth(FS)
+    f = np.linspace(80e6, 180e6, K)
+    s.set_tones(f, np.full(K, 1.0 / K), np.zeros(K))
+    if chirps:
+        s.set_chirps(np.arange(chirps), f[:chirps], f[:chirps] + 1e6, np.full(chirps, 5e-3), np.zeros(chirps, dtype=np.int64),
+                     np.zeros(chirps, dtype=np.int64))
+    n = 12 * chunk + 777
+    out = torch.empty(n, dtype=torch.int16, device="cuda")
+    ms, ev = _times(s, lambda: s.render_stream(n, chunk, out))
+    assert 0.6 * ev < ms < 1.1 * ev, (ms, ev)
+    s.close()
+
+
 @pytest.mark.parametrize("chirps", [0, 20])
 def test_engine_pieces(awglib, chirps):
     """A window of more samples than the engine takes at a time."""
