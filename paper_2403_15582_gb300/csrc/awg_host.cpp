@@ -886,14 +886,6 @@ int upload_runs(T* dev, const std::vector<T>& host, const std::vector<int32_t>& 
 }
 
 // Largest |amplitude| any tone takes (its ramp target included), in FP32 as the kernels hold it.
-double max_amplitude_scan(const awg_t* h) {
-  double m = 0;
-  for (const ToneRec& t : h->tones) {
-    m = std::max(m, (double)std::fabs(t.A));
-    if (t.flags & awgk::TONE_AMP_RAMP) m = std::max(m, (double)std::fabs(t.A_end));
-  }
-  return m;
-}
 const std::vector<int32_t>& flagged_tones(awg_t* h);
 double max_amplitude(awg_t* h) {
   (void)flagged_tones(h);   // refreshes the cached maximum with the flagged tones
@@ -1426,16 +1418,25 @@ struct EngineSplit {
 };
 const std::vector<int32_t>& flagged_tones(awg_t* h) {
   if (!h->flagged_ok) {
-    h->amax = max_amplitude_scan(h);
+    float amax = 0.f;
+    int64_t full0 = 0, full1 = h->tones.empty() ? -1 : INT64_MAX;
     h->flagged.clear();
-    for (size_t k = 0; k < h->tones.size(); ++k)
-      if (h->tones[k].slot >= 0 || (h->tones[k].flags & awgk::TONE_AMP_RAMP)) h->flagged.push_back((int32_t)k);
-    h->full0 = 0;
-    h->full1 = h->tones.empty() ? -1 : INT64_MAX;
-    for (const ToneRec& t : h->tones) {   // (a chirp's tiles: those its samples n_s .. n_e meet)
-      h->full0 = std::max(h->full0, t.slot >= 0 ? t.n_s / awgk::TILE * awgk::TILE : 0);
-      h->full1 = std::min(h->full1, t.slot >= 0 ? t.n_e / awgk::TILE * awgk::TILE : -1);
+    for (size_t k = 0; k < h->tones.size(); ++k) {
+      const ToneRec& t = h->tones[k];
+      const bool ramp = (t.flags & awgk::TONE_AMP_RAMP) != 0;
+      amax = std::max(amax, std::fabs(t.A));
+      if (ramp) amax = std::max(amax, std::fabs(t.A_end));
+      if (t.slot >= 0 || ramp) h->flagged.push_back((int32_t)k);
+      if (t.slot >= 0) {   // a chirp's tiles: those its samples n_s .. n_e meet
+        full0 = std::max(full0, t.n_s / awgk::TILE * awgk::TILE);
+        full1 = std::min(full1, t.n_e / awgk::TILE * awgk::TILE);
+      } else {
+        full1 = -1;
+      }
     }
+    h->amax = amax;
+    h->full0 = full0;
+    h->full1 = full1;
     h->flagged_ok = true;
   }
   return h->flagged;
