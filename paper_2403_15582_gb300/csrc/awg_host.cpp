@@ -577,7 +577,8 @@ struct awg {
   int32_t static_engine = AWG_STATIC_DIRECT;
   float* d_base = nullptr;             // tensor-core engine: FP32 sum of the window's static tones, then
   size_t cap_base = 0;                 // that of its other tones, rendered on `side` beside the GEMM
-  cudaStream_t side = nullptr;         // created on first use, with its events
+  cudaStream_t side = nullptr;         // created on first use, with its events, at the caller's priority
+  int side_priority = 0;
   cudaEvent_t ev_fork = nullptr, ev_operand = nullptr, ev_join = nullptr;
   // split sums without clusters: two scratch buffers (alternating between consecutive launches)
   // of part_tiles x part_split partial tiles each, and a 64-bit counter per tile per buffer
@@ -1508,13 +1509,24 @@ int engine_operand(awg_t* h, bool two_segments, bool first, cudaStream_t s) {
   return AWG_OK;
 }
 
-int ensure_side_stream(awg_t* h) {
-  if (h->ev_join) return AWG_OK;
-  cudaError_t e = cudaSuccess;
-  if (!h->side) e = cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking);
+// The side stream of a call on stream s, at its priority (what a call on a high-priority stream queued at
+// the default priority would wait for other work of that priority: 71 ms behind one kernel of 74 ms that
+// fills the device, now 0.65).  Another priority than the last call's takes another stream; the last one's
+// work is joined.
+int ensure_side_stream(awg_t* h, cudaStream_t s) {
+  int priority = 0;
+  cudaError_t e = cudaStreamGetPriority(s, &priority);
+  if (e == cudaSuccess && h->side && priority != h->side_priority) {
+    e = cudaStreamDestroy(h->side);
+    h->side = nullptr;
+  }
+  if (e == cudaSuccess && !h->side) {
+    e = cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, priority);
+    h->side_priority = priority;
+  }
   if (e == cudaSuccess && !h->ev_fork) e = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming);
   if (e == cudaSuccess && !h->ev_operand) e = cudaEventCreateWithFlags(&h->ev_operand, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming);
+  if (e == cudaSuccess && !h->ev_join) e = cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming);
   if (e != cudaSuccess) return cuda_fail(e, "engine stream");
   return AWG_OK;
 }
@@ -1545,7 +1557,7 @@ int render_engine(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
       if ((st = ensure(&h->d_base, &h->cap_base, live_at + (size_t)m, h, "engine sums"))) return st;
       const int64_t n_tiles = (c + m - 1) / awgk::TILE - c / awgk::TILE + 1;
       if (use_list && (st = ensure(&h->d_list, &h->cap_list, list_entries(n_list, n_tiles, es.split), h, "tone list"))) return st;
-      if ((st = ensure_side_stream(h))) return st;
+      if ((st = ensure_side_stream(h, s))) return st;
     }
     float* d_live = h->d_base + live_at;
     cudaError_t e;
