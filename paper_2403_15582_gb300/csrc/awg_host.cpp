@@ -780,10 +780,15 @@ class HostPool {
 // split - 1 mod split; so they are zeroed when allocated and whenever the split changes.
 constexpr int32_t SPLIT_LAUNCH_TILES = 512;   // tiles per render launch when the split sums in scratch
 
-// Zero, and complete on return: the kernels that use the bytes run on streams that do not wait for the
-// default stream (the caller's, the engine's side stream).
+// Zeroed or copied, and complete on return: the kernels that use the bytes run on streams that do not wait
+// for the default stream (the caller's, the private and the side stream), and neither cudaMemset nor
+// cudaMemcpy from pageable memory says that the device is done when it returns.
 cudaError_t zero_now(awg_t* h, void* p, size_t bytes) {
   const cudaError_t e = cudaMemsetAsync(p, 0, bytes, h->priv);
+  return e == cudaSuccess ? cudaStreamSynchronize(h->priv) : e;
+}
+cudaError_t copy_now(awg_t* h, void* dev, const void* host, size_t bytes) {
+  const cudaError_t e = cudaMemcpyAsync(dev, host, bytes, cudaMemcpyHostToDevice, h->priv);
   return e == cudaSuccess ? cudaStreamSynchronize(h->priv) : e;
 }
 
@@ -827,7 +832,7 @@ int upload_tones(awg_t* h) {
   int st = ensure(&h->d_tones, &h->cap_tones, std::max<size_t>(1, h->tones.size()), h, "tones");
   if (st) return st;
   if (!h->tones.empty()) {
-    cudaError_t e = cudaMemcpy(h->d_tones, h->tones.data(), h->tones.size() * sizeof(ToneRec), cudaMemcpyHostToDevice);
+    cudaError_t e = copy_now(h, h->d_tones, h->tones.data(), h->tones.size() * sizeof(ToneRec));
     if (e != cudaSuccess) return cuda_fail(e, "upload tones");
   }
   return AWG_OK;
@@ -853,7 +858,7 @@ int upload_chirps(awg_t* h) {
     h->cap_chirps = ncap;
   }
   if (!h->chirps.empty()) {
-    cudaError_t e = cudaMemcpy(h->d_chirps, h->chirps.data(), h->chirps.size() * sizeof(ChirpRec), cudaMemcpyHostToDevice);
+    cudaError_t e = copy_now(h, h->d_chirps, h->chirps.data(), h->chirps.size() * sizeof(ChirpRec));
     if (e != cudaSuccess) return cuda_fail(e, "upload chirps");
   }
   return AWG_OK;
@@ -876,14 +881,15 @@ std::vector<Span> copy_spans(const std::vector<int32_t>& idx, size_t record_byte
   return spans;
 }
 
-// Upload the records at the given (sorted, unique) indices.
+// Upload the records at the given (sorted, unique) indices; complete on return (copy_now).
 template <class T>
-int upload_runs(T* dev, const std::vector<T>& host, const std::vector<int32_t>& idx, const char* what) {
-  for (const Span& sp : copy_spans(idx, sizeof(T))) {
-    cudaError_t e = cudaMemcpy(dev + sp.first, host.data() + sp.first, sp.count * sizeof(T), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return cuda_fail(e, what);
-  }
-  return AWG_OK;
+int upload_runs(awg_t* h, T* dev, const std::vector<T>& host, const std::vector<int32_t>& idx, const char* what) {
+  cudaError_t e = cudaSuccess;
+  for (const Span& sp : copy_spans(idx, sizeof(T)))
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(dev + sp.first, host.data() + sp.first, sp.count * sizeof(T), cudaMemcpyHostToDevice, h->priv);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->priv);
+  return e == cudaSuccess ? AWG_OK : cuda_fail(e, what);
 }
 
 // Largest |amplitude| any tone takes (its ramp target included), in FP32 as the kernels hold it.
@@ -1962,9 +1968,9 @@ awg_t* awg_create(double sample_rate_hz) {
     int32_t* act = nullptr;
     e = awgk::noalloc_scratch(h->device, &recs, &act);
   }
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_status, sizeof(int32_t));
-  if (e == cudaSuccess) e = cudaMemset(h->d_status, 0, sizeof(int32_t));
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->priv, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_status, sizeof(int32_t));
+  if (e == cudaSuccess) e = zero_now(h, h->d_status, sizeof(int32_t));
   if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_times, 2 * sizeof(unsigned long long));
   if (e == cudaSuccess) e = zero_now(h, h->d_times, 2 * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_done, cudaEventDisableTiming);
@@ -2145,7 +2151,7 @@ int awg_set_chirps(awg_t* h, const int32_t* tone, const double* f_start_hz, cons
     if ((st = upload_chirps(h))) return st;
     if ((st = build_exact_tables(h))) return st;
     if (any_exact) return upload_tones(h);   // table offsets may have moved for any exact tone
-    return upload_runs(h->d_tones, h->tones, changed_tones, "upload tones");
+    return upload_runs(h, h->d_tones, h->tones, changed_tones, "upload tones");
   }
   // steady state: the copies (and the exact tables' kernels) run on the private stream after the
   // renders issued so far, and later renders wait for them, so this call does not wait for the
@@ -2201,7 +2207,7 @@ int awg_set_amp_ramps(awg_t* h, const int32_t* tone, const double* amp_end, cons
     changed.push_back(tone[i]);
   }
   std::sort(changed.begin(), changed.end());
-  return upload_runs(h->d_tones, h->tones, changed, "upload tones");
+  return upload_runs(h, h->d_tones, h->tones, changed, "upload tones");
 }
 
 int awg_set_full_scale(awg_t* h, double v) {
@@ -2725,7 +2731,7 @@ int awg_device_status(awg_t* h) {
   int32_t v = 0;
   cudaError_t e = cudaDeviceSynchronize();
   if (e == cudaSuccess) e = cudaMemcpy(&v, h->d_status, sizeof(v), cudaMemcpyDeviceToHost);
-  if (e == cudaSuccess) e = cudaMemset(h->d_status, 0, sizeof(int32_t));
+  if (e == cudaSuccess) e = zero_now(h, h->d_status, sizeof(int32_t));
   if (e != cudaSuccess) return cuda_fail(e, "device status");
   return v;
 }
