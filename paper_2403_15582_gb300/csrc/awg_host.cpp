@@ -907,9 +907,11 @@ double default_full_scale(const awg_t* h) {
 
 // Stream-ordered upload through the pinned staging buffer: stage_begin makes room for `bytes` behind the
 // uploads that are still pending (their copies have yet to read the buffer; it waits for them only
-// when there is no room) and orders the private stream after the last render issued; stage_spans
+// when there is no room; a buffer holds three such uploads, up to STAGE_ROOM) and orders the private
+// stream after the last render issued; stage_spans
 // queues the copies of the records of the given spans; stage_end marks the upload's completion
 // (ev_upload) for later launches to wait on.
+constexpr size_t STAGE_ROOM = (size_t)16 << 20;
 int stage_begin(awg_t* h, size_t bytes) {
   cudaError_t e;
   if (h->upload_pending && cudaEventQuery(h->ev_upload) == cudaSuccess) h->upload_pending = false;
@@ -921,8 +923,8 @@ int stage_begin(awg_t* h, size_t bytes) {
       h->upload_pending = false;
     }
     h->stage_used = 0;
-    if (3 * bytes > h->cap_stage) {   // room for a call's tones and chirps and the next call's
-      const size_t ncap = std::max(3 * bytes, 2 * h->cap_stage);
+    if (std::max(bytes, std::min(3 * bytes, STAGE_ROOM)) > h->cap_stage) {   // a call's tones and chirps and the next call's
+      const size_t ncap = std::max(bytes, std::min(std::max(3 * bytes, 2 * h->cap_stage), STAGE_ROOM));
       unsigned char* p = nullptr;
       if (cudaHostAlloc((void**)&p, ncap, cudaHostAllocDefault) != cudaSuccess) {
         cudaGetLastError();
@@ -995,11 +997,16 @@ int set_tones_common(awg_t* h, const double* f, const double* amp, const double*
   }
   // Into larger device arrays: synchronous (reallocation waits for the device anyway), and before the
   // host's state changes.  Otherwise the copy is queued behind the last render and later renders wait
-  // for it, so this call does not wait for the device.
-  const bool grow = (size_t)n > h->cap_tones || h->cap_tones == 0;
+  // for it, so this call does not wait for the device; unless the pinned memory for it is large
+  // (STAGE_ROOM: 174,000 tones) or not to be had.
+  const size_t bytes = (size_t)n * sizeof(ToneRec);
+  bool now = (size_t)n > h->cap_tones || h->cap_tones == 0 || bytes > STAGE_ROOM;
   int st;
-  if (grow && (st = wait_idle(h))) return st;
-  if (!grow && n > 0 && (st = stage_begin(h, (size_t)n * sizeof(ToneRec)))) return st;
+  if (!now && n > 0 && (st = stage_begin(h, bytes))) {
+    if (st != AWG_ENOMEM) return st;
+    now = true;
+  }
+  if (now && (st = wait_idle(h))) return st;
   h->tones.swap(tones);
   h->amp.swap(a);
   h->K = n;
@@ -1011,7 +1018,7 @@ int set_tones_common(awg_t* h, const double* f, const double* amp, const double*
   h->fs_explicit = false;
   h->full_scale = default_full_scale(h);
   h->split = awgk::tone_split_for(n);
-  if (grow) {
+  if (now) {
     if ((st = upload_tones(h))) return st;
     return upload_chirps(h);
   }
