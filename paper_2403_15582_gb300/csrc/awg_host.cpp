@@ -1144,6 +1144,7 @@ struct Window {
   int32_t n_tiles, per_launch;
   int32_t split;              // CTAs per part of a tile (set by the caller)
   bool first;                 // its first kernel starts the call (device time)
+  bool together = false;      // one of several channels in one launch
   bool once;                  // RenderArgs::once: no set-up kernel
   std::vector<int32_t> active;
   cudaEvent_t pe[4] = {nullptr, nullptr, nullptr, nullptr};   // profiling
@@ -1152,12 +1153,24 @@ struct Window {
 
 // A window with chirps and at most 96 tones per CTA (1536 tones) goes without a set-up kernel: each CTA
 // takes all its tones at once and forms their chirp records itself.  A call then has one kernel, which
-// may run beside the end of the one before: 1000 chirps x 2^18 samples 96 -> 67 us among others (the
+// may run beside the end of the one before: 1000 chirps x 2^18 samples 93 -> 67 us among others (the
 // set-up alone 13 us, and the render waits for it).  Not in chunk sequences, where one set-up kernel
-// serves all chunks and the records cost less there than in the render's CTAs (35 ms record 2611
-// against 2722 us), not without chirps (100 static tones 25.2 against 26.2 us), and not with more
-// tones, whose records would be formed in the middle of the sums.
+// serves all chunks and the records cost less there than in the render's CTAs, not without chirps (100
+// static tones 25.2 against 26.2 us), and not with more tones, whose records would be formed in the middle
+// of the sums.
 bool once_fits(const awg_t* h, int32_t split) { return (int64_t)h->K <= (int64_t)awgk::ONCE_TONES * split; }
+
+// Whether a single window of several launches gains by it.  A CTA waits for its records before it sums, the
+// longer in proportion the fewer tones it sums, while the set-up kernel is paid once (20 to 30 us with
+// its launch): the line is n_tiles x (112 - tones per CTA) = 56,000.  Set-up kernel / records in the CTA, us:
+// 100 chirps 768 tiles 103 / 102, 896 115 / 119, 1024 139 / 150, 2048 256 / 298; 128 chirps 768 tiles 125 / 114,
+// 1024 157 / 158, 2048 297 / 318; 160 chirps 1536 tiles 281 / 277, 2048 368 / 369; 220 chirps 1024 tiles
+// 260 / 260, 2048 493 / 522; 250 chirps 1536 tiles 420 / 416, 2048 550 / 555; 1000 chirps 1536 tiles 1583 /
+// 1573, 2048 2116 / 2118.  Where few tones chirp the CTAs have little to form (20 of 100 tones, 2048 tiles:
+// 227 / 216), and a window with one CTA per tile is one launch (96 chirps, 2048 tiles: 220 / 197).
+bool once_pays(const awg_t* h, const Window& w) {
+  return w.split == 1 || few_chirps(h, w.active) || (int64_t)w.n_tiles * (112 * w.split - h->K) <= (int64_t)56000 * w.split;
+}
 
 int window_plan(awg_t* h, int64_t n, bool may_once, Window* w) {
   w->c = h->cursor;
@@ -1167,7 +1180,7 @@ int window_plan(awg_t* h, int64_t n, bool may_once, Window* w) {
   if (n_tiles > (int64_t)(INT32_MAX / awgk::MAX_SPLIT)) return fail(AWG_EINVAL, "render window too long");
   w->n_tiles = (int32_t)n_tiles;
   w->active = active_slots(h, w->c, n, &w->tile0, &w->n_tiles);
-  w->once = may_once && once_fits(h, w->split) && !w->active.empty();
+  w->once = may_once && once_fits(h, w->split) && !w->active.empty() && (w->together || once_pays(h, *w));
   if (w->once) w->active.clear();
   int st = ensure(&h->d_recs, &h->cap_recs, w->active.size() * (size_t)w->n_tiles, h, "tile records");
   if (st) return st;
@@ -1293,6 +1306,7 @@ int render_channels(awg_t* const* handles, int32_t n_channels, int64_t n, int16_
   for (int32_t c = 0; c < n_channels; ++c) {
     w[c].split = handles[c]->split;
     w[c].first = true;
+    w[c].together = true;
     if ((st = window_plan(handles[c], n, may_once, &w[c]))) return st;
     once = once || w[c].once;
     if (!w[c].active.empty()) last_setup = c;
