@@ -1057,14 +1057,18 @@ int build_exact_tables(awg_t* h, bool sync = true) {
   return AWG_OK;
 }
 
-// Chirp slots active in the window [c, c + n) (tile-aligned span), excluding exact-table chirps, in
-// tone order: the render copies the records of a stage's tones in one piece.
+// The tiles of the window [c, c + n).
+void window_tiles(int64_t c, int64_t n, int64_t* tile0, int64_t* n_tiles) {
+  *tile0 = c / awgk::TILE;
+  *n_tiles = (c + n - 1) / awgk::TILE - *tile0 + 1;
+}
+// Chirp slots active in the tiles [tile0, tile0 + n_tiles), excluding exact-table chirps, in tone order:
+// the render copies the records of a stage's tones in one piece.
 bool slot_active(const ChirpRec& cr, int64_t span0, int64_t span1) {
   return cr.tone >= 0 && !(cr.flags & awgk::TONE_EXACT) && cr.n_s <= span1 && cr.n_s + cr.L >= span0;
 }
-std::vector<int32_t> active_slots(const awg_t* h, int64_t c, int64_t n, int64_t* tile0, int32_t* n_tiles) {
-  const int64_t t0 = c / awgk::TILE, t1 = (c + n - 1) / awgk::TILE;
-  const int64_t span0 = t0 * awgk::TILE, span1 = (t1 + 1) * awgk::TILE - 1;
+std::vector<int32_t> active_slots(const awg_t* h, int64_t tile0, int64_t n_tiles) {
+  const int64_t span0 = tile0 * awgk::TILE, span1 = (tile0 + n_tiles) * awgk::TILE - 1;
   std::vector<int32_t> active;
   if (h->chirps.size() < h->tones.size() / 8) {   // few chirps: their slots, sorted
     for (size_t sl = 0; sl < h->chirps.size(); ++sl)
@@ -1075,8 +1079,6 @@ std::vector<int32_t> active_slots(const awg_t* h, int64_t c, int64_t n, int64_t*
     for (const ToneRec& t : h->tones)
       if (t.slot >= 0 && !(t.flags & awgk::TONE_EXACT) && t.n_s <= span1 && t.n_e >= span0) active.push_back(t.slot);
   }
-  *tile0 = t0;
-  *n_tiles = (int32_t)(t1 - t0 + 1);
   return active;
 }
 
@@ -1175,11 +1177,11 @@ bool once_pays(const awg_t* h, const Window& w) {
 int window_plan(awg_t* h, int64_t n, bool may_once, Window* w) {
   w->c = h->cursor;
   w->n = n;
-  w->tile0 = w->c / awgk::TILE;
-  const int64_t n_tiles = (w->c + n - 1) / awgk::TILE - w->tile0 + 1;
+  int64_t n_tiles;
+  window_tiles(w->c, n, &w->tile0, &n_tiles);
   if (n_tiles > (int64_t)(INT32_MAX / awgk::MAX_SPLIT)) return fail(AWG_EINVAL, "render window too long");
   w->n_tiles = (int32_t)n_tiles;
-  w->active = active_slots(h, w->c, n, &w->tile0, &w->n_tiles);
+  w->active = active_slots(h, w->tile0, n_tiles);
   w->once = may_once && once_fits(h, w->split) && !w->active.empty() && (w->together || once_pays(h, *w));
   if (w->once) w->active.clear();
   int st = ensure(&h->d_recs, &h->cap_recs, w->active.size() * (size_t)w->n_tiles, h, "tile records");
@@ -1709,9 +1711,10 @@ int awgk::prepare_render(awg_t* h, int64_t n, int16_t* out_q, float* out_f, cuda
                          awgk::TileRec* recs, size_t recs_cap, int32_t* act, size_t* recs_need) {
   if (!h || n <= 0 || (!out_q && !out_f) || !ra) return fail(AWG_EINVAL, "prepare_render: bad arguments");
   const int64_t c = h->cursor;
-  int64_t tile0;
-  int32_t n_tiles;
-  const std::vector<int32_t> active = active_slots(h, c, n, &tile0, &n_tiles);
+  int64_t tile0, tiles;
+  window_tiles(c, n, &tile0, &tiles);
+  const int32_t n_tiles = (int32_t)tiles;
+  const std::vector<int32_t> active = active_slots(h, tile0, tiles);
   const size_t need = active.size() * (size_t)n_tiles;
   if (recs_need) *recs_need = need;
   if (recs || act) {
@@ -1806,15 +1809,16 @@ int render_chunks_impl(awg_t* h, int64_t chunk, int32_t n_chunks, int16_t* out, 
     Group g;
     g.g0 = g0;
     g.g1 = g0 + 1;
-    g.active = active_slots(h, c0 + (int64_t)g0 * chunk, span(g0, g0 + 1), &g.tile0, &g.n_tiles);
+    int64_t nt;
+    window_tiles(c0 + (int64_t)g0 * chunk, span(g0, g0 + 1), &g.tile0, &nt);
+    g.n_tiles = (int32_t)nt;
+    g.active = active_slots(h, g.tile0, nt);
     while (g.g1 < n_chunks) {
-      int64_t t0;
-      int32_t nt;
-      std::vector<int32_t> a2 = active_slots(h, c0 + (int64_t)g0 * chunk, span(g0, g.g1 + 1), &t0, &nt);
+      window_tiles(c0 + (int64_t)g0 * chunk, span(g0, g.g1 + 1), &g.tile0, &nt);
+      std::vector<int32_t> a2 = active_slots(h, g.tile0, nt);
       if (a2.size() * (size_t)nt > SEQ_RECORD_BUDGET || nt > INT32_MAX / awgk::MAX_SPLIT) break;
       g.active.swap(a2);
-      g.tile0 = t0;
-      g.n_tiles = nt;
+      g.n_tiles = (int32_t)nt;
       ++g.g1;
     }
     max_recs = std::max(max_recs, g.active.size() * (size_t)g.n_tiles);

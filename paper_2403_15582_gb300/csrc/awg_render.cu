@@ -10,9 +10,10 @@
 //
 // Work decomposition (see awg_internal.h): a CTA renders one tile of TILE = 4096 absolute-aligned
 // samples (or a half or a quarter of it, see Geo); thread j owns the run of RUN = 32 samples starting
-// at T0 + 32 j (or a half or a quarter of a run) and keeps its partial sums in registers; the tones are split over `split` CTAs, whose partial tiles are added in rank
-// order (through L2 scratch by the last CTA of the tile to finish, or through distributed shared
-// memory in a thread-block cluster), then scaled, rounded and stored by the same kernel.
+// at T0 + 32 j (or a half or a quarter of a run) and keeps its partial sums in registers; the tones are
+// split over `split` CTAs, whose partial tiles are added in rank order (through L2 scratch by the last
+// CTA of the tile to finish, or through distributed shared memory in a thread-block cluster), then
+// scaled, rounded and stored by the same kernel.
 //
 // Per (tone, run) the phase is set up once and then stepped per sample in 32-bit fixed point
 // (units of 2^-32 turn):
@@ -156,7 +157,7 @@ constexpr uint64_t HALF32 = 1ull << 31;
 constexpr uint64_t B0_OFFSET = P_OFFSET + (1ull << 63);
 
 // A run's 32-bit cascade state: p is the run-start phase plus half a turn (the centred form that
-// sin_centred takes), f, g, h its first three differences.
+// sin_pair takes), f, g, h its first three differences.
 struct RunPoly {
   uint32_t p, f, g, h;
 };
@@ -335,16 +336,10 @@ __device__ __forceinline__ int classify_tile(const ToneRec& t, int64_t T0) {
   return TILE_CHIRP;
 }
 
-// sin(2 pi p / 2^32) for a phase already offset by half a turn (pc = p + 2^31): the top 23 bits
-// of pc become the mantissa of a float v in [1, 2); 2 pi (v - 3/2) lies in [-pi, pi) and is
-// congruent to the phase.  The half-turn offset is added once per run, not per sample.
+// The sine takes a phase already offset by half a turn (pc = p + 2^31, added once per run, not per
+// sample; sin_pair): the float v = 1.m with the 23-bit fraction m = pc >> 9 (exponent field of [1, 2)).
 constexpr uint32_t HALF_TURN = 1u << 31;
-// The float 1.m with the 23-bit fraction m = pc >> 9 (exponent field of [1, 2)).
 __device__ __forceinline__ float mantissa_float(uint32_t pc) { return __uint_as_float((pc >> 9) + 0x3F800000u); }
-__device__ __forceinline__ float sin_centred(uint32_t pc) {
-  const float v = mantissa_float(pc);
-  return __sinf(fmaf(v, 6.28318530717958647692f, -9.42477796076937971538f));
-}
 
 // ------------------------------------------------------------------------------------------
 // TMA bulk copies and mbarriers (inline PTX)
@@ -643,7 +638,7 @@ __device__ __forceinline__ void store_record(TileRec* out, const TileRec& r) {
     o[i] = make_uint4((uint32_t)r.w[2 * i], (uint32_t)(r.w[2 * i] >> 32), (uint32_t)r.w[2 * i + 1], (uint32_t)(r.w[2 * i + 1] >> 32));
 }
 
-// The record of chirp c (of tone t) at tile T0, handed to put(count, record, count as a constant).
+// The record of chirp c (of tone t) at tile T0, handed to put(record, its word count as a constant).
 template <int N>
 struct Count {
   static constexpr int value = N;
@@ -654,15 +649,15 @@ __device__ __forceinline__ void form_record(const ChirpRec& c, const ToneRec& t,
   TileRec r;
   if (words == REC_WORDS_LINEAR) {
     prep_one<2, REC_WORDS_LINEAR>(c, T0 - c.n_s, a, r);
-    put(words, r, Count<REC_WORDS_LINEAR>());
+    put(r, Count<REC_WORDS_LINEAR>());
   } else if (words == REC_WORDS_LOW3) {
     if (c.flags & TONE_EXP) prep_exp<REC_WORDS_LOW3>(c, T0 - c.n_s, a, r);
     else prep_one<6, REC_WORDS_LOW3>(c, T0 - c.n_s, a, r);
-    put(words, r, Count<REC_WORDS_LOW3>());
+    put(r, Count<REC_WORDS_LOW3>());
   } else {
     if (c.flags & TONE_EXP) prep_exp<REC_WORDS>(c, T0 - c.n_s, a, r);
     else prep_one<6, REC_WORDS>(c, T0 - c.n_s, a, r);
-    put(words, r, Count<REC_WORDS>());
+    put(r, Count<REC_WORDS>());
   }
 }
 
@@ -683,7 +678,7 @@ __global__ void __launch_bounds__(128, 5) prep_kernel(const __grid_constant__ Ar
   TileRec* out = a.recs + (int64_t)t * a.rec_stride + a.act_base + ai;
   // the preceding kernel of the stream may be a render that reads the buffers written here: it has
   // to be complete before the first write, not before the arithmetic
-  form_record(c, a.tones[c.tone], T0, a, [&](int, const TileRec& r, auto words) {
+  form_record(c, a.tones[c.tone], T0, a, [&](const TileRec& r, auto words) {
     pdl_wait();
     store_record<decltype(words)::value>(out, r);
   });
@@ -716,7 +711,8 @@ using Acc = float2[SPT / 2];
 constexpr float TWO_PI_F = 6.28318530717958647692f;
 constexpr float THREE_PI_F = 9.42477796076937971538f;
 
-// the sines of two phases already offset by half a turn (see sin_centred)
+// sin(2 pi p / 2^32) of two phases already offset by half a turn: 2 pi (v - 3/2) of their mantissa floats
+// v lies in [-pi, pi) and is congruent to the phase
 __device__ __forceinline__ float2 sin_pair(uint32_t p0, uint32_t p1) {
   const float2 v = make_float2(mantissa_float(p0), mantissa_float(p1));
   const float2 x = __ffma2_rn(v, make_float2(TWO_PI_F, TWO_PI_F), make_float2(-THREE_PI_F, -THREE_PI_F));
@@ -1046,8 +1042,8 @@ __device__ __forceinline__ bool f_vec_ok(const RenderArgs& a) {
   return !a.out_f || (((uintptr_t)a.out_f - 4u * (uint64_t)a.win_start) & 15u) == 0;
 }
 
-// Store the 8 samples n .. n + 7 (n a multiple of 8) of a group inside the window, the outputs aligned:
-// one 16-byte vector of int16 codes and two of FP32 sums.
+// Store the 8 samples n .. n + 7 (n a multiple of 8) of a group inside the window, the outputs aligned
+// (q_vec_ok, f_vec_ok): one 16-byte vector of int16 codes and, where asked for, two of FP32 sums.
 __device__ __forceinline__ void store_group(const RenderArgs& a, int64_t n, const float (&xv)[8]) {
   const int64_t o = n - a.win_start;
   float x[8];
@@ -1332,13 +1328,13 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
         const bool pre = tcls == TILE_PRE;
         d.F = pre ? tr.F : tr.F_end;
         d.p0 = (pre ? tr.phi_ref : tr.phi_post_ref) + (uint64_t)T0 * d.F;
-        if (a.sine_mode == SINE_ROTATOR) {
+        if (PARTS == 1 && a.sine_mode == SINE_ROTATOR) {   // (parts never take the rotator: render_parts)
           d.c = pre ? tr.rot_c : tr.rot_c_end;
           d.s = pre ? tr.rot_s : tr.rot_s_end;
         }
       }
       kind = tile_kind(tr, T0, a.skip_static != 0);
-      if (kind == DESC_STATIC && a.sine_mode == SINE_ROTATOR) kind = DESC_STATIC_ROT;
+      if (PARTS == 1 && kind == DESC_STATIC && a.sine_mode == SINE_ROTATOR) kind = DESC_STATIC_ROT;
       s_desc[b][lane] = d;
       pairable = (tr.flags & TONE_PAIR) && !a.skip_static;
     }
@@ -1367,7 +1363,7 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
     if constexpr (ONCE) {
       if (need) {
         const ToneRec& tr = s_tone[b][lane];
-        form_record(a.chirps[tr.slot], tr, T0, a, [&](int, const TileRec& r, auto words) {
+        form_record(a.chirps[tr.slot], tr, T0, a, [&](const TileRec& r, auto words) {
 #pragma unroll
           for (int i = 0; i < decltype(words)::value; ++i) s_rec[b][lane].w[i] = r.w[i];
         });
@@ -1473,8 +1469,6 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
         float re, im;
         phasor(d, re, im);
         const float c = d.c, s = d.s;
-        if (PARTS > 1)
-          for (uint32_t r = 0; r < r0; ++r) rotate(re, im, c, s);
 #pragma unroll
         for (int r = 0; r < SPT; ++r) {
           if (r & 1) acc[r / 2].y += im;
@@ -1506,8 +1500,9 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
         pair(poly_state_low6(record(odd ? k : i), rb), i, k);
       }
       for (int o = e_l3p + ((e_l6p - e_l3p) & ~1); o < e_low6; ++o) low6(s_order[b][o]);
-      if (a.sine_mode == SINE_ROTATOR) {
-        for (int o = e_low6; o < e_static; ++o) static_rot(s_order[b][o]);
+      if (a.sine_mode == SINE_ROTATOR) {   // never with parts; without the test the loop below is 0.5 % slower
+        if constexpr (PARTS == 1)
+          for (int o = e_low6; o < e_static; ++o) static_rot(s_order[b][o]);
       } else {
         // the next tone's set-up before this tone's loop
         RunPoly nx = {0, 0, 0, 0};
