@@ -2117,9 +2117,10 @@ int awg_set_chirps(awg_t* h, const int32_t* tone, const double* f_start_hz, cons
       rotation_of(p.F1, &co[i].rot_c, &co[i].rot_s);
     }
   };
-  // ranges of at least 8 chirps, about 32 of them (more of them cost more in claims than they even out:
-  // 1000 chirps 213 us in 32 ranges, 287 in 126), from 1024 chirps on 32 to a range
-  HostPool::get().parallel_for(pend.size(), std::min(pend.size() / 8 + 1, std::max<size_t>(32, pend.size() / 32 + 1)), work);
+  // ranges of about 32 chirps; fewer chirps stay on this thread (waking the workers costs 30 to 50 us: 8 linear
+  // chirps 25 us here, 55 over the pool, 31 minimum-jerk ones 95 against 122; 100 of them take 265 us in
+  // 4 ranges and 269 in 13, 200 linear ones 74 in 7 and 100 in 26)
+  HostPool::get().parallel_for(pend.size(), pend.size() / 32 + 1, work);
   std::vector<int32_t> changed_tones, changed_slots;
   for (size_t pi = 0; pi < pend.size(); ++pi) {
     const Pending& p = pend[pi];
