@@ -603,7 +603,7 @@ struct awg {
   int64_t periodic_start = -1;
   cudaStream_t priv = nullptr;
   cudaEvent_t ev_done = nullptr;
-  unsigned long long* d_times = nullptr;   // device times of the last render's start and end
+  unsigned long long* d_times = nullptr;   // device times of the last render's start and end; the status word
   // stream-ordered uploads of changed records (awg_set_chirps): pinned staging, copied on the
   // private stream after the last render issued (ev_done); later launches wait for ev_upload
   unsigned char* stage = nullptr;
@@ -780,15 +780,10 @@ class HostPool {
 // split - 1 mod split; so they are zeroed when allocated and whenever the split changes.
 constexpr int32_t SPLIT_LAUNCH_TILES = 512;   // tiles per render launch when the split sums in scratch
 
-// Zeroed or copied, and complete on return: the kernels that use the bytes run on streams that do not wait
-// for the default stream (the caller's, the private and the side stream), and neither cudaMemset nor
-// cudaMemcpy from pageable memory says that the device is done when it returns.
+// Zeroed, and complete on return: the kernels that use the bytes run on streams that do not wait for the
+// default stream (the caller's, the private and the side stream), and cudaMemset may return before it.
 cudaError_t zero_now(awg_t* h, void* p, size_t bytes) {
   const cudaError_t e = cudaMemsetAsync(p, 0, bytes, h->priv);
-  return e == cudaSuccess ? cudaStreamSynchronize(h->priv) : e;
-}
-cudaError_t copy_now(awg_t* h, void* dev, const void* host, size_t bytes) {
-  const cudaError_t e = cudaMemcpyAsync(dev, host, bytes, cudaMemcpyHostToDevice, h->priv);
   return e == cudaSuccess ? cudaStreamSynchronize(h->priv) : e;
 }
 
@@ -828,14 +823,26 @@ unsigned long long* split_ctr(awg_t* h, int b) {
   return h->d_tctr + (size_t)b * (size_t)h->part_tiles * awgk::MAX_PARTS;
 }
 
+// Marks the completion of the copies queued on the private stream for later launches to wait on.
+int stage_end(awg_t* h) {
+  cudaError_t e = cudaEventRecord(h->ev_upload, h->priv);
+  if (e != cudaSuccess) return cuda_fail(e, "upload event");
+  h->upload_pending = true;
+  return AWG_OK;
+}
+
+// A copy from pageable memory with the device idle: on the private stream like the staged ones, so that
+// later launches wait for it.  (cudaMemcpy's own may still be under way when it returns, on a stream that
+// the renders' do not wait for.)  The source is free on return: it has been copied for the device to read.
+int upload(awg_t* h, void* dev, const void* host, size_t bytes, const char* what) {
+  const cudaError_t e = cudaMemcpyAsync(dev, host, bytes, cudaMemcpyHostToDevice, h->priv);
+  return e == cudaSuccess ? stage_end(h) : cuda_fail(e, what);
+}
+
 int upload_tones(awg_t* h) {
   int st = ensure(&h->d_tones, &h->cap_tones, std::max<size_t>(1, h->tones.size()), h, "tones");
   if (st) return st;
-  if (!h->tones.empty()) {
-    cudaError_t e = copy_now(h, h->d_tones, h->tones.data(), h->tones.size() * sizeof(ToneRec));
-    if (e != cudaSuccess) return cuda_fail(e, "upload tones");
-  }
-  return AWG_OK;
+  return h->tones.empty() ? AWG_OK : upload(h, h->d_tones, h->tones.data(), h->tones.size() * sizeof(ToneRec), "upload tones");
 }
 
 int upload_chirps(awg_t* h) {
@@ -857,11 +864,7 @@ int upload_chirps(awg_t* h) {
     h->d_act = q;
     h->cap_chirps = ncap;
   }
-  if (!h->chirps.empty()) {
-    cudaError_t e = copy_now(h, h->d_chirps, h->chirps.data(), h->chirps.size() * sizeof(ChirpRec));
-    if (e != cudaSuccess) return cuda_fail(e, "upload chirps");
-  }
-  return AWG_OK;
+  return h->chirps.empty() ? AWG_OK : upload(h, h->d_chirps, h->chirps.data(), h->chirps.size() * sizeof(ChirpRec), "upload chirps");
 }
 
 // Records at sorted unique indices as spans to copy: neighbours, and those with fewer unchanged records
@@ -881,15 +884,13 @@ std::vector<Span> copy_spans(const std::vector<int32_t>& idx, size_t record_byte
   return spans;
 }
 
-// Upload the records at the given (sorted, unique) indices; complete on return (copy_now).
+// Upload the records at the given (sorted, unique) indices.
 template <class T>
 int upload_runs(awg_t* h, T* dev, const std::vector<T>& host, const std::vector<int32_t>& idx, const char* what) {
-  cudaError_t e = cudaSuccess;
+  int st = AWG_OK;
   for (const Span& sp : copy_spans(idx, sizeof(T)))
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(dev + sp.first, host.data() + sp.first, sp.count * sizeof(T), cudaMemcpyHostToDevice, h->priv);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->priv);
-  return e == cudaSuccess ? AWG_OK : cuda_fail(e, what);
+    if (!st) st = upload(h, dev + sp.first, host.data() + sp.first, sp.count * sizeof(T), what);
+  return st;
 }
 
 // Largest |amplitude| any tone takes (its ramp target included), in FP32 as the kernels hold it.
@@ -956,13 +957,6 @@ size_t span_bytes(const std::vector<T>&, const std::vector<Span>& spans) {
   size_t n = 0;
   for (const Span& sp : spans) n += sp.count * sizeof(T);
   return n;
-}
-
-int stage_end(awg_t* h) {
-  cudaError_t e = cudaEventRecord(h->ev_upload, h->priv);
-  if (e != cudaSuccess) return cuda_fail(e, "upload event");
-  h->upload_pending = true;
-  return AWG_OK;
 }
 
 int set_tones_common(awg_t* h, const double* f, const double* amp, const double* ph, int32_t n, int32_t log2_len) {
@@ -1994,10 +1988,9 @@ awg_t* awg_create(double sample_rate_hz) {
     e = awgk::noalloc_scratch(h->device, &recs, &act);
   }
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->priv, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_status, sizeof(int32_t));
-  if (e == cudaSuccess) e = zero_now(h, h->d_status, sizeof(int32_t));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_times, 2 * sizeof(unsigned long long));
-  if (e == cudaSuccess) e = zero_now(h, h->d_times, 2 * sizeof(unsigned long long));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_times, 3 * sizeof(unsigned long long));
+  if (e == cudaSuccess) e = zero_now(h, h->d_times, 3 * sizeof(unsigned long long));
+  h->d_status = (int32_t*)(h->d_times + 2);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_done, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_upload, cudaEventDisableTiming);
   if (e != cudaSuccess) {
@@ -2029,7 +2022,6 @@ void awg_destroy(awg_t* h) {
   cudaFree(h->d_seq_recs);
   cudaFree(h->d_seq_act);
   cudaFree(h->d_seq_exit);
-  cudaFree(h->d_status);
   cudaFree(h->d_words);
   cudaFree(h->d_trace);
   cudaFree(h->d_tab);
