@@ -281,7 +281,10 @@ int32_t awg_tone_split(const awg_t* h);
 
 /* Device time (ms) of the last render, from the start of its first kernel to the end of its last
  * CTA (device clock); it is valid once that render has completed (e.g. after synchronising its
- * stream).  -1 if none. */
+ * stream).  -1 if none.  A call issued behind another one starts beside its end and then waits for
+ * it, so its time can hold part of that call; to time a call by itself, synchronise before it.
+ * Multiplexed channels share their launches: each channel's time spans its own part of them.  A
+ * chunk sequence counts as one render. */
 float awg_last_render_ms(awg_t* h);
 
 /* Profiling mode: while on, every render records CUDA events on its stream around its chirp

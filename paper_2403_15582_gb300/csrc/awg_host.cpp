@@ -1151,8 +1151,8 @@ struct Window {
 // takes all its tones at once and forms their chirp records itself.  A call then has one kernel, which
 // may run beside the end of the one before: 1000 chirps x 2^18 samples 93 -> 67 us among others (the
 // set-up alone 13 us, and the render waits for it).  Not in chunk sequences, where one set-up kernel
-// serves all chunks and the records cost less there than in the render's CTAs, not without chirps (100
-// static tones 25.2 against 26.2 us), and not with more tones, whose records would be formed in the middle
+// serves all chunks and the records cost less there than in the render's CTAs (35 ms record of 1000 chirps
+// 2534 against 2578 us), not without chirps (100 static tones 25.2 against 26.2 us), and not with more tones, whose records would be formed in the middle
 // of the sums.
 bool once_fits(const awg_t* h, int32_t split) { return (int64_t)h->K <= (int64_t)awgk::ONCE_TONES * split; }
 
@@ -1601,7 +1601,8 @@ int render_engine(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
     // for a render CTA, and a window's GEMM often leaves SMs idle (128 CTAs for 2^20 samples on 152).
     // The set-up runs beside the operand's; the render starts once the operand is made, so that the
     // GEMM's CTAs (one per SM, nearly all of its shared memory) are placed first.  10,000 tones x
-    // 2^20, 400 of them chirping in turn: 300 us one after the other, 208 us side by side.
+    // 2^20, 400 of them chirping in turn: 300 us one after the other, 216 us side by side (207 with the
+    // boundary tiles' mask, mixed_run).
     if ((e = cudaStreamWaitEvent(h->side, h->ev_fork, 0)) != cudaSuccess) return cuda_fail(e, "engine ordering");
     if (use_list && n_list > 0 &&
         (e = cudaMemcpyAsync(h->d_list, h->list.data(), (size_t)n_list * sizeof(int32_t), cudaMemcpyHostToDevice,

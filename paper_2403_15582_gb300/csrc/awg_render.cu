@@ -1622,7 +1622,8 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
 // 1000-chirp 35 ms record takes 2524 us at six, 2599 at seven (72 registers), 2587 at five; the batched
 // and cluster renders keep five (no spills).  Parts need fewer accumulators: eight, but six where the
 // CTA forms its records (at eight 1.2 KB of spills).  A kernel per mode: with the list's code in it the
-// plain render's registers change and the record takes 2640 instead of 2616 us.
+// plain render's record takes 2539 us where it takes 2534 without (before the stage buffers lay in one
+// object 2640 and 2616).
 #define AWG_RENDER_MIN_BLOCKS 5
 #define AWG_RENDER_SPLIT_MIN_BLOCKS 6
 #define AWG_RENDER_PART_MIN_BLOCKS 8
@@ -1872,8 +1873,9 @@ __global__ void replay_strided_kernel(const int16_t* __restrict__ tab, uint64_t 
 // boundary of the output, `head` samples into it; its vector v (8 samples) is the table's samples
 // 8 (v0 + v) + SHIFT .. + 7 mod period, SHIFT = shift samples.  A thread takes vectors u of one period
 // and writes each to its REPS repeats u, u + P, u + 2 P ... (P vectors per period), so a record that
-// repeats is read from the L2 once per REPS writes: 2^27 samples of a 2^24 table 52 -> 45.6 us (reading
-// the table for every vector ran at 5.4 TB/s written, plain fills at 6.9).  Streaming stores keep the
+// repeats is read from the L2 once per REPS writes: 2^27 samples of a 2^24 table 52 -> 45.6 us among others
+// (58.5 while timed events stood between the kernels; reading the table for every vector ran at 5.4 TB/s
+// written, plain fills at 6.9).  Streaming stores keep the
 // table in the L2.  Samples before `out` and after its last whole vector are copied one by one.
 constexpr int REPLAY_VEC = 2, REPLAY_REPS = 8;
 __global__ void __launch_bounds__(256) replay_kernel(const int16_t* __restrict__ tab, uint64_t mask, int64_t c, int64_t n,

@@ -168,7 +168,9 @@ __device__ __forceinline__ float2 unpack2<__half>(uint32_t u) {
 // store per half, a row of 128 bytes per half warp.  Warp g takes the rows 16 g .. 16 g + 15, lane l
 // tone l mod 16 and every second row.  (Before, each segment had a lane of its own with 64-bit tile
 // compares per row, and the tone records were read after the wait for the stage: 270 us for 10,000
-// tones x 2^20; now 177, of which the MMAs take about 155 at the rate of the table.)
+// tones x 2^20; now 177.  At the table's rate the MMAs over 40,000 columns take about 155 of them, and
+// half of that multiplies zeros where few tones have a second segment: with 400 chirping tones 20,800
+// columns would do.)
 //
 // The rows of a tone where a segment is live, as rows of this CTA's tile (clamped to 0 .. TM): segment
 // 0 in rows < pre, segment 1 in rows >= post, neither in the rows ramp_lo .. ramp_hi - 1 of an
@@ -178,7 +180,7 @@ struct WindowTone {
   int32_t pre, post, ramp_lo, ramp_hi;
   float amp, amp_end;
 };
-// first row of the tile ceil or floor of which the caller has formed, relative to the CTA's rows
+// The first row of a tile (given by its absolute index), relative to the CTA's first row R0.
 __device__ __forceinline__ int32_t clamp_row(int64_t tile, int64_t R0) {
   return (int32_t)max((int64_t)0, min((int64_t)TM, tile * (TILE / TN) - R0));
 }
