@@ -1179,6 +1179,12 @@ int window_plan(awg_t* h, int64_t n, bool may_once, Window* w) {
   w->once = may_once && once_fits(h, w->split) && !w->active.empty() && (w->together || once_pays(h, *w));
   if (w->once) w->active.clear();
   int st = ensure(&h->d_recs, &h->cap_recs, w->active.size() * (size_t)w->n_tiles, h, "tile records");
+  if (st == AWG_ENOMEM && may_once && once_fits(h, w->split)) {   // no room for the records: in the CTAs after all
+    cudaGetLastError();
+    w->once = true;
+    w->active.clear();
+    st = AWG_OK;
+  }
   if (st) return st;
   // With a split, the window goes out in launches of at most SPLIT_LAUNCH_TILES tiles, on
   // alternating scratch buffers.
