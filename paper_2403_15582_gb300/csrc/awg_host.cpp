@@ -1437,7 +1437,8 @@ namespace {
 // rows aligned to absolute sample indices, two column pairs per tone (before and after its
 // chirp); the others by the render kernel, which skips the static ones and adds the GEMM's FP32
 // sum before quantising.  The split depends on the tile and the tone state only, so a sample's
-// value does not depend on how the stream is cut into calls.  Pieces of at most 2^26 samples.
+// value does not depend on how the stream is cut into calls.  Pieces of at most 2^26 samples, shorter ones
+// where the device has no room for their sums.
 
 // The render part's tone split: the tones that hold a chirp or a ramp at all (they change only when
 // chirps, ramps or tones are set, never while rendering), about the same number of them in each of
@@ -1560,15 +1561,17 @@ int ensure_side_stream(awg_t* h, cudaStream_t s) {
   return AWG_OK;
 }
 
+constexpr int64_t MIN_PIECE = (int64_t)1 << 20;
 int render_engine(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* stream, int32_t q_stride, bool first) {
   cudaStream_t s = (cudaStream_t)stream;
-  const int64_t PIECE = (int64_t)1 << 26;
+  int64_t piece = (int64_t)1 << 26;
   const EngineSplit es = engine_split(h);
   // no tone has ever held a chirp or a ramp: every tone is static in one segment everywhere, and
   // the GEMM takes the table's two columns per tone instead of four (half the work)
   const bool two_segments = es.n_flagged > 0;
-  for (int64_t off = 0; off < n; off += PIECE) {
-    const int64_t m = std::min(PIECE, n - off), c = h->cursor;
+  for (int64_t off = 0, m; off < n; off += m) {
+    m = std::min(piece, n - off);
+    const int64_t c = h->cursor;
     engine_list(h, c, m, &h->list);
     const bool all_static = q_stride == 1 && h->K > 0 && h->list.empty();
     int16_t* oq = out_q ? out_q + (size_t)off * (size_t)q_stride : nullptr;
@@ -1583,10 +1586,16 @@ int render_engine(awg_t* h, int64_t n, float* out_f, int16_t* out_q, void* strea
     const bool use_list = n_list < h->K;
     const size_t live_at = ((size_t)m + 3) & ~(size_t)3;
     if (!all_static) {
-      if ((st = ensure(&h->d_base, &h->cap_base, live_at + (size_t)m, h, "engine sums"))) return st;
       const int64_t n_tiles = (c + m - 1) / awgk::TILE - c / awgk::TILE + 1;
-      if (use_list && (st = ensure(&h->d_list, &h->cap_list, list_entries(n_list, n_tiles, es.split), h, "tone list"))) return st;
-      if ((st = ensure_side_stream(h, s))) return st;
+      st = ensure(&h->d_base, &h->cap_base, live_at + (size_t)m, h, "engine sums");
+      if (!st && use_list) st = ensure(&h->d_list, &h->cap_list, list_entries(n_list, n_tiles, es.split), h, "tone list");
+      if (st == AWG_ENOMEM && m > MIN_PIECE) {   // the two sums do not fit: shorter pieces, the same samples
+        cudaGetLastError();
+        piece = m / 2;
+        m = 0;
+        continue;
+      }
+      if (st || (st = ensure_side_stream(h, s))) return st;
     }
     float* d_live = h->d_base + live_at;
     cudaError_t e;
