@@ -1200,7 +1200,9 @@ __device__ __forceinline__ void tile_epilogue_split(const RenderArgs& a, int uni
 //
 // The tones go through in stages of STAGE, in the stage's visit order: the groups of visit_group, each
 // in a loop of its own without a per-tone dispatch, then the rest.
-// MODE_ONCE: RenderArgs::once; MODE_LIST: a tone list, if a.tone_list is set; MODE_ALL: all tones.
+// MODE_ONCE: RenderArgs::once; MODE_LIST: a tone list, if a.tone_list is set, and renders for the tensor-core
+// engine; MODE_ALL: all tones, no engine (with the engine's test for plain order in it 4770 chirps x 3829
+// samples take 126.7 us, 124.6 without; 10,000 chirping tones on the engine 977 and, in MODE_LIST's kernel, 992).
 enum { MODE_ALL = 0, MODE_LIST = 1, MODE_ONCE = 2, N_MODES = 3 };
 template <int SPT, bool CLUSTER, int MODE>
 __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit, const int crank, const int split) {
@@ -1343,9 +1345,9 @@ __device__ __forceinline__ void render_tile(const RenderArgs& a, const int unit,
     // FP32 sums then depends on which tones share a stage; with a tone list (the window's listed
     // tones) that changes with the window.  So a render for the tensor-core engine keeps plain tone
     // order in every tile that some window may take with a list: all but those in which every tone
-    // chirps (full0 .. full1; there the groups save 5 to 9 %: 10,000 chirping tones x 2^18 samples 975
+    // chirps (full0 .. full1; there the groups save 5 to 8 %: 10,000 chirping tones x 2^18 samples 992
     // us, 1068 in plain order).  Every window cut gives the same bits.  Skipped tones are left out.
-    const bool plain = list != nullptr || (a.skip_static && (T0 < a.full0 || T0 > a.full1));
+    const bool plain = MODE != MODE_ALL && (list != nullptr || (a.skip_static && (T0 < a.full0 || T0 > a.full1)));
     const int grp = kind == DESC_SKIP ? -1 : visit_group(kind, plain, pairable);
     const unsigned below = (1u << lane) - 1u;
     int pos = 0, end = 0;
@@ -2036,7 +2038,7 @@ cudaError_t launch_render(const RenderArgs& a, cudaStream_t s) {
   if (!a.cluster) {   // the split sums through the scratch partials
     cfg.attrs = attr + 1;
     cfg.numAttrs = a.pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, split_kernel(parts, a.once ? MODE_ONCE : a.tone_list ? MODE_LIST : MODE_ALL), a);
+    return cudaLaunchKernelEx(&cfg, split_kernel(parts, a.once ? MODE_ONCE : a.tone_list || a.skip_static ? MODE_LIST : MODE_ALL), a);
   }
   cfg.attrs = attr;
   cfg.numAttrs = a.pdl ? 2 : 1;
